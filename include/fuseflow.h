@@ -156,8 +156,8 @@ int fuseflow_fuse_frame(fuseflow_ctx *ctx, const void *const *depth, const float
 /* A fuse call recorded once as a CUDA graph, for callers whose input images live in the
  * same device buffers every frame (a capture loop that refills them): replaying it with
  * fuseflow_graph_launch is the same as calling fuseflow_fuse_frame with the pointers
- * given here, whose contents may change between launches, at one launch instead of seven
- * (eight with a depth screen set).
+ * given here, whose contents may change between launches, at one launch instead of eight
+ * (nine with a depth screen set).
  * The graph keeps the context's launch geometry and trace registration as they were at
  * creation; results do not depend on the geometry.  It uses the context's tables, so
  * launches of graphs and fuse calls of one context must be ordered (one stream), and
@@ -295,28 +295,23 @@ int fuseflow_read_stage_times(fuseflow_ctx *ctx, double *ms, int64_t *n_frames);
 const char *fuseflow_stage_name(int stage);
 
 /* Launch geometry of a context: performance knobs only.  The fused cloud, its statistics
- * and any trace are bitwise the same for every admissible setting of the first four (the
- * path has no order-dependent arithmetic); tile_h changes how each cell's members are
- * grouped into per-tile fixed-point partial sums, so keys, counts, representatives, the
- * trace and the statistics stay bitwise the same while weights, positions and colours
- * may move in their last bits (far inside the 1e-5 relative tolerance: each partial is
- * exact at a scale of 2^-36 of the largest weight in its tile, and shifting it to the
- * cell's scale truncates below that).  A setting can be chosen by timing alone.
+ * and any trace are bitwise the same for every admissible setting (the path has no
+ * order-dependent arithmetic).  A setting can be chosen by timing alone.
  *   count_chunks    2048-pixel chunks per block of the coarse-count step, 1..64
  *   emit_blocks     blocks of the level, reduce and emit steps, 1..65536
- *   prefetch_tiles  how many assign tiles ahead each assign block prefetches its
- *                   depth rows into L2; 0 turns the prefetch off
+ *   prefetch_tiles  how many tiles ahead each block of the assign step's first kernel
+ *                   prefetches colours into L2 for its second; 0 turns the prefetch off
  *   programmatic    2: each kernel of a frame after the first is launched with
  *                   programmatic stream serialization, so that its blocks start while the
  *                   previous kernel's last blocks finish (they wait for its results on the
  *                   device); 1: the same except between the assign and reduce steps (early
  *                   reduce blocks slow the assign step's last wave on large frames); 0:
  *                   plain stream order.  Stage timing always uses plain order.
- *   tile_h          rows of the assign step's tiles of 32 columns: 8 (128 threads a
- *                   block), 16 (256) or 32 (512); 0 in fuseflow_set_tuning keeps the
- *                   current height
- * fuseflow_create picks count_chunks for one wave of four count blocks per SM (at most 6),
- * emit_blocks = 8 blocks per SM, prefetch_tiles = one wave of assign blocks,
+ *   tile_h          rows of the assign step's tiles of 32 columns: 8, 16 or 32 (64, 128 or
+ *                   256 threads a block, more for frames of few tiles); 0 in
+ *                   fuseflow_set_tuning keeps the current height
+ * fuseflow_create picks count_chunks for two waves of four count blocks per SM,
+ * emit_blocks = 8 blocks per SM, prefetch_tiles = 0 (on 8x1280x720 it costs 2 us),
  * programmatic = 2 for rigs of fewer than 2^21 pixels, 1 otherwise, and tile_h = 16. */
 typedef struct fuseflow_tuning {
   int32_t count_chunks;
@@ -364,13 +359,13 @@ int64_t fuseflow_device_bytes(const fuseflow_ctx *ctx);
  * change the process's memory footprint after start-up.  This call needs no context: it
  * takes the rig and parameters directly, calls no cudaMalloc, cudaFree or other
  * allocating routine (device or host), and keeps all of its scratch in one file-scope
- * device array of about 23 MiB that every GPU loading this library holds until exit.
+ * device array of about 31 MiB that every GPU loading this library holds until exit.
  *
  * Limits: at most 524,288 pixels per frame over all cameras, at most 65,536 ray-table
  * entries (sum over cameras of width + height), 2 (K - 1) times that at most 393,216
  * (K = min(k_views, n_cams)), and max_cells <= 32,768 (0 selects 32,768); larger
  * requests return FUSEFLOW_ERR_CAPACITY before anything is sent to the GPU.  A
- * frame that produces more than 131,072 (tile, cell) partial records reports a capacity
+ * frame with top_k > 0 that produces more than 131,072 (tile, cell) records reports a capacity
  * error in stats->error.
  * Inputs are device pointers as for fuseflow_fuse_frame; pos[3*max_cells],
  * rgb_out[3*max_cells], weight, count, rep, key[max_cells] and *stats are caller-owned

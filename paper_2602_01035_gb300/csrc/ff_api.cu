@@ -39,7 +39,7 @@ struct fuseflow_ctx {
   size_t out_bytes = 0;
   TraceDev trace{};
   Geometry geo{};
-  long long max_chunks = 0;            // 2048-pixel chunks of the largest camera
+  int n_units = 0;                     // units of 32 x 8 pixels over all cameras
   int bstats_cap = 0;                  // count-step block statistics allocated (chunks = 1)
   // staging for the host-buffer entry point
   void* d_stage = nullptr;
@@ -168,6 +168,19 @@ int validate(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* extr, i
   return FUSEFLOW_OK;
 }
 
+// The count step's grid for a number of 8-unit chunks per block.
+void count_geometry(Geometry* g, int n_units, int chunks) {
+  g->count_chunks = chunks;
+  g->count_blocks = (n_units + 8 * chunks - 1) / (8 * chunks);
+}
+
+// Chunks per count block: two waves of four resident blocks per SM, so that a block's set-up and its
+// statistics are shared by several units a warp and the last wave stays short.
+int default_chunks(int n_units, int sms) {
+  const int wave = 4 * sms * 8;                          // units of one wave at one chunk a block
+  return std::max(1, std::min(64, n_units / (2 * wave)));
+}
+
 bool screen_set(const fuseflow_params* p) {
   return p->screen_min_m > 0 || p->screen_max_m > 0 || p->screen_edge_rel > 0.0f;
 }
@@ -183,10 +196,87 @@ ScreenArgs screen_args(const fuseflow_intrinsics* intr, int n_cams, const fusefl
   return a;
 }
 
+// Depths (metres) that the grid evaluation of the consistency step covers for float32 depth; a
+// uint16 image reaches the same 65.5 m in millimetres.  Farther samples take the general
+// evaluation, point by point.
+constexpr double kGridDepthM = 65.536;
+
+// Relative pose T_ji = T_j T_i^-1 of Eq. 4 (R row-major, t in metres).
+void relative_pose(const fuseflow_extrinsics& e, const fuseflow_extrinsics& ej, double R[9], double t[3]) {
+  for (int r = 0; r < 3; ++r)
+    for (int s = 0; s < 3; ++s) {
+      double acc = 0;
+      for (int m = 0; m < 3; ++m) acc += ej.R[3 * r + m] * e.R[3 * s + m];   // R_j R_i^T
+      R[3 * r + s] = acc;
+    }
+  for (int r = 0; r < 3; ++r)
+    t[r] = ej.t[r] - (R[3 * r] * e.t[0] + R[3 * r + 1] * e.t[1] + R[3 * r + 2] * e.t[2]);
+}
+
+// Largest |ray component| over an image's columns and rows.
+double ray_bound(double c, double f, int n) { return std::max(std::fabs(c), std::fabs((double)(n - 1) - c)) / f; }
+
+// Grid units per depth unit: the largest power of two for which every camera-frame coordinate
+// the consistency step forms from depths up to zmax (a point in its neighbours' frames and a
+// neighbour's own sample) stays below 2^22.
+double grid_per_unit(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* extr, int n_cams,
+                     double unit, const int32_t* nbr, int k1, double zmax) {
+  double most = zmax;
+  for (int i = 0; i < n_cams; ++i) {
+    const double rx = ray_bound(intr[i].cx, intr[i].fx, intr[i].width);
+    const double ry = ray_bound(intr[i].cy, intr[i].fy, intr[i].height);
+    most = std::max(most, zmax * std::max(rx, ry));
+    for (int q = 0; q < k1; ++q) {
+      double R[9], t[3];
+      relative_pose(extr[i], extr[nbr[i * k1 + q]], R, t);
+      for (int a = 0; a < 3; ++a)
+        most = std::max(most, zmax * (std::fabs(R[3 * a]) * rx + std::fabs(R[3 * a + 1]) * ry + std::fabs(R[3 * a + 2])) +
+                                  std::fabs(t[a]) / unit);
+    }
+  }
+  int e = 0;
+  std::frexp(most * 1.001, &e);                  // most < 2^e
+  return std::ldexp(1.0, std::max(-60, std::min(60, 22 - e)));
+}
+
+// Pair rays of view q of one camera (layout: kPrayColGroup, kPrayRowGroup) in grid units per
+// depth unit.  The high parts of A_k and B_k are multiples of 2^-23 of a power of two above
+// max|A_k| + max|B_k|: their sum is exact in float32.
+void put_pair_rays(const fuseflow_intrinsics& k, const double R[9], double ginv, int q, int k1, float4* cam) {
+  const double rx = ray_bound(k.cx, k.fx, k.width), ry = ray_bound(k.cy, k.fy, k.height);
+  double step[3];
+  for (int a = 0; a < 3; ++a) {
+    int e = 0;
+    std::frexp(ginv * (std::fabs(R[3 * a]) * rx + std::fabs(R[3 * a + 2]) + std::fabs(R[3 * a + 1]) * ry) * 1.001, &e);
+    step[a] = std::ldexp(1.0, e - 23);
+  }
+  auto put = [&](float4* group, int plane2, int i, const double v[3]) {
+    float h[3], l[3];
+    for (int a = 0; a < 3; ++a) {
+      h[a] = (float)(std::nearbyint(ginv * v[a] / step[a]) * step[a]);
+      l[a] = (float)(ginv * v[a] - (double)h[a]);
+    }
+    group[i] = make_float4(h[0], h[1], h[2], l[0]);
+    reinterpret_cast<float2*>(group + plane2)[i] = make_float2(l[1], l[2]);
+  };
+  const int wg = (k.width + 31) / 32, hg = (k.height + 31) / 32 * 4;
+  for (int x = 0; x < 32 * wg; ++x) {            // the padding continues the last column
+    const double r = ((double)std::min(x, k.width - 1) - k.cx) / k.fx;
+    const double v[3] = {R[0] * r + R[2], R[3] * r + R[5], R[6] * r + R[8]};
+    put(cam + ((long long)(x / 32) * k1 + q) * kPrayColGroup, 32, x % 32, v);
+  }
+  float4* rows = cam + (long long)wg * k1 * kPrayColGroup;
+  for (int y = 0; y < 8 * hg; ++y) {
+    const double r = ((double)std::min(y, k.height - 1) - k.cy) / k.fy;
+    const double v[3] = {R[1] * r, R[4] * r, R[7] * r};
+    put(rows + ((long long)(y / 8) * k1 + q) * kPrayRowGroup, 8, y % 8, v);
+  }
+}
+
 // Rig constants shared by fuseflow_create and the static entry point: per-camera
 // intrinsics and poses, the ray tables rx(x) = (x - cx)/fx and ry(y) = (y - cy)/fy as ff,
 // the relative poses of Eq. 4 (T_ji = T_j T_i^-1) and the separable pair rays.
-// `rays` holds sum(W + H) entries and `pray` 2 k1 sum(W + H) float4.
+// `rays` holds sum(W + H) entries and `pray` the sum of pray_cam_size float4.
 void build_rig(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* extr, int n_cams,
                const fuseflow_params* params, const int32_t* nbr, int k1, RigDev& rig,
                float2* rays, float4* pray) {
@@ -194,18 +284,22 @@ void build_rig(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* extr,
   std::memset(&rig, 0, sizeof(rig));
   rig.n_cams = n_cams;
   rig.k1 = k1;
-  rig.tau = params->tau;
-  rig.use_conf = params->use_conf ? 1 : 0;
-  rig.use_cons = params->use_consistency ? 1 : 0;
-  rig.max_level = params->max_level;
+  rig.hot.tau = params->tau;
+  rig.hot.use_conf = params->use_conf ? 1 : 0;
+  rig.hot.use_cons = params->use_consistency ? 1 : 0;
+  rig.hot.max_level = params->max_level;
   rig.n_min = params->n_min;
-  rig.inv_s0u = (float)(unit / params->coarse_cell_m);
-  const double sig_u = params->sigma_m / unit;
-  if (k1 > 0) split(1.0 / (sig_u * sig_u * k1), rig.einv_h, rig.einv_l);
+  rig.hot.inv_s0u = (float)(unit / params->coarse_cell_m);
+  const double zmax = params->depth_format == FUSEFLOW_DEPTH_U16 ? 65535.0 : kGridDepthM / unit;
+  const double ginv = grid_per_unit(intr, extr, n_cams, unit, nbr, k1, zmax);
+  rig.hot.ginv = (float)ginv;
+  rig.hot.zmax = (float)zmax;
+  const double sig_g = params->sigma_m / unit * ginv;
+  if (k1 > 0) split(1.0 / (sig_g * sig_g * k1), rig.hot.einv_h, rig.hot.einv_l);
   rig.depth_f32 = params->depth_format == FUSEFLOW_DEPTH_F32;
   rig.top_k = params->top_k;
-  int nr = 0, np = 0;
-  long long off = 0;
+  int nr = 0;
+  long long off = 0, np = 0;
   for (int i = 0; i < n_cams; ++i) {
     const fuseflow_intrinsics& k = intr[i];
     const fuseflow_extrinsics& e = extr[i];
@@ -236,37 +330,15 @@ void build_rig(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* extr,
       PairDev& P = rig.pair[c.pair0 + q];
       P.j = j;
       double Rji[9], tji[3];
-      for (int r = 0; r < 3; ++r)
-        for (int s2 = 0; s2 < 3; ++s2) {
-          double acc = 0;
-          for (int m = 0; m < 3; ++m) acc += ej.R[3 * r + m] * e.R[3 * s2 + m];   // R_j R_i^T
-          Rji[3 * r + s2] = acc;
-        }
-      for (int r = 0; r < 3; ++r)
-        tji[r] = ej.t[r] - (Rji[3 * r] * e.t[0] + Rji[3 * r + 1] * e.t[1] + Rji[3 * r + 2] * e.t[2]);
-      for (int a = 0; a < 9; ++a) split(Rji[a], P.Rh[a], P.Rl[a]);
-      for (int a = 0; a < 3; ++a) split(tji[a] / unit, P.th[a], P.tl[a]);
-      // separable pair rays A_k(x) = R[k][0] rx(x) + R[k][2], B_k(y) = R[k][1] ry(y)
-      auto put = [&](double v0, double v1, double v2) {
-        float4& u = pray[np++];
-        float4& w = pray[np++];
-        split(v0, u.x, u.y);
-        split(v1, u.z, u.w);
-        split(v2, w.x, w.y);
-        w.z = 0.0f;
-        w.w = 0.0f;
-      };
-      P.ga = np;
-      for (int x = 0; x < k.width; ++x) {
-        const double rx = ((double)x - k.cx) / k.fx;
-        put(Rji[0] * rx + Rji[2], Rji[3] * rx + Rji[5], Rji[6] * rx + Rji[8]);
+      relative_pose(e, ej, Rji, tji);
+      for (int a = 0; a < 3; ++a) {
+        const double t = tji[a] / unit * ginv;
+        P.th[a] = (float)std::nearbyint(t);
+        P.tl[a] = (float)(t - (double)P.th[a]);
       }
-      P.gb = np;
-      for (int y = 0; y < k.height; ++y) {
-        const double ry = ((double)y - k.cy) / k.fy;
-        put(Rji[1] * ry, Rji[4] * ry, Rji[7] * ry);
-      }
+      put_pair_rays(k, Rji, ginv, q, k1, pray + np);
     }
+    np += pray_cam_size(k.width, k.height, k1);
   }
   rig.n_px = off;
 }
@@ -344,14 +416,15 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   // ---------------------------------------------------------------- rig constants
   RigDev* rig = new (std::nothrow) RigDev();
   if (!rig) { delete ctx; return FUSEFLOW_ERR_OUT_OF_MEMORY; }
-  long long off = 0, n_rays = 0, max_px = 0;
+  long long off = 0, n_rays = 0, n_pray = 0, max_px = 0;
   for (int i = 0; i < n_cams; ++i) {
     off += (long long)intr[i].width * intr[i].height;
     n_rays += intr[i].width + intr[i].height;
+    n_pray += pray_cam_size(intr[i].width, intr[i].height, ctx->k1);
     max_px = std::max(max_px, (long long)intr[i].width * intr[i].height);
   }
   std::vector<float2> rays((size_t)n_rays);
-  std::vector<float4> pray((size_t)std::max<long long>(1, 2 * ctx->k1 * n_rays));
+  std::vector<float4> pray((size_t)std::max<long long>(1, n_pray));
   build_rig(intr, extr, n_cams, params, ctx->nbr.data(), ctx->k1, *rig, rays.data(), pray.data());
   ctx->n_px = off;
   ctx->max_cells = params->max_cells > 0 ? params->max_cells : std::max<long long>(65536, off / 8);
@@ -366,21 +439,14 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   ctx->geo.top_k = params->top_k;
   ctx->geo.depth_f32 = rig->depth_f32;
   ctx->geo.max_px = max_px;
+  ctx->geo.hot = rig->hot;
   ctx->geo.scr = screen_args(intr, n_cams, params);
   ctx->geo.screen = screen_set(params) ? 1 : 0;
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
-  {
-    // several 2048-pixel chunks per count block: one wave of 4 blocks per SM (the kernel's
-    // residency), but at most 6 chunks, since a block's table of coarse cells (2048
-    // entries) spills to the global table when one block covers too much of the scene
-    long long total_chunks = 0;
-    for (int i = 0; i < n_cams; ++i) total_chunks += ((long long)intr[i].width * intr[i].height + 2047) / 2048;
-    const long long per = (total_chunks + 4ll * sms - 1) / (4ll * sms);
-    ctx->geo.count_chunks = (int)std::max<long long>(1, std::min<long long>(6, per));
-    ctx->max_chunks = (max_px + 2047) / 2048;
-    ctx->geo.count_blocks_x = (int)((ctx->max_chunks + ctx->geo.count_chunks - 1) / ctx->geo.count_chunks);
-  }
+  const int n_tiles = fill_tile_index(*rig, &ctx->geo.tiles, 16);
+  ctx->n_units = ctx->geo.tiles.unit[n_cams];
+  count_geometry(&ctx->geo, ctx->n_units, default_chunks(ctx->n_units, sms));
   ctx->geo.emit_blocks = std::max(1, sms * 8);
   ctx->geo.pdl = off < (1ll << 21) ? 2 : 1;
 
@@ -389,12 +455,14 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   const long long n_words = (off + 31) / 32;
   const int n_wblocks = (int)((n_words + 1023) / 1024);
   // block statistics for the finest count geometry a tuning may choose (one chunk a block)
-  ctx->bstats_cap = (int)(ctx->max_chunks * n_cams);
-  const int n_bstats = ctx->geo.count_blocks_x * n_cams;
+  ctx->bstats_cap = (ctx->n_units + 7) / 8;
   size_t o = 0;
   auto take = [&](size_t bytes, size_t align) { o = align_up(o, align); size_t at = o; o += bytes; return at; };
-  // (tile, cell) partials: at most one per gated pixel
-  const unsigned max_partials = (unsigned)std::min<long long>(off, 0xfffffffell);
+  // top-k variant: (tile, cell) partials, at most one per gated pixel; otherwise a gated pixel's slot
+  // and weight, and a cell's sums and key
+  const bool topk = params->top_k > 0;
+  const unsigned max_partials = topk ? (unsigned)std::min<long long>(off, 0xfffffffell) : 0u;
+  const size_t n_weighed = topk ? 0 : (size_t)off, n_summed = topk ? 0 : (size_t)ctx->max_cells;
   const size_t o_frec = take(sizeof(SlotRec) * ctx->max_slots, 256);
   const size_t o_fused = take(sizeof(unsigned) * ctx->max_slots, 256);
   const size_t o_coarse = take(sizeof(CoarseEntry) * ctx->ccap, 256);
@@ -405,6 +473,16 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   const size_t o_staged = take(sizeof(CellOut) * (size_t)ctx->max_cells, 256);
   const size_t o_wpre = take(sizeof(unsigned) * (size_t)n_words, 256);
   const size_t o_bsum = take(sizeof(unsigned) * (size_t)n_wblocks, 256);
+  const size_t o_lpix = take(sizeof(unsigned short) * (size_t)off, 256);
+  const size_t o_ldep = take((rig->depth_f32 ? 4 : 2) * (size_t)off, 256);
+  const size_t o_lconf = take(sizeof(float) * (size_t)off, 256);
+  const size_t o_lcnt = take(sizeof(unsigned) * (size_t)ctx->n_units, 256);
+  const size_t o_lcell = take(sizeof(unsigned) * kUnitCells * (size_t)ctx->n_units, 256);
+  const size_t o_wslot = take(sizeof(unsigned) * n_weighed, 256);
+  const size_t o_wmant = take(sizeof(float) * n_weighed, 256);
+  const size_t o_wexp = take(sizeof(int) * n_weighed, 256);
+  const size_t o_acc = take(8 * sizeof(unsigned long long) * n_summed, 256);
+  const size_t o_ckey = take(sizeof(unsigned long long) * n_summed, 256);
   ctx->table_bytes = o;
   size_t po = 0;
   auto take_out = [&](size_t bytes) { po = align_up(po, 256); size_t at = po; po += bytes; return at; };
@@ -417,8 +495,6 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   const size_t q_key = take_out(sizeof(unsigned long long) * (size_t)ctx->max_cells);
   ctx->out_bytes = po;
 
-  const int n_tiles = fill_tile_index(*rig, &ctx->geo.tiles, 16);
-  ctx->geo.tiles.ahead = assign_resident_blocks(16, rig->k1) * sms;
   std::vector<BlockConst> bconst((size_t)n_cams);
   fill_block_consts(*rig, bconst.data());
   const size_t pray_at = align_up(sizeof(BlockConst) * (size_t)n_cams, 256);
@@ -456,12 +532,23 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
     t.bconst = static_cast<const BlockConst*>(ctx->d_blocks);
     t.pray = reinterpret_cast<const float4*>(static_cast<char*>(ctx->d_blocks) + pray_at);
     t.n_tiles = n_tiles;
+    t.n_units = ctx->n_units;
+    t.lpix = reinterpret_cast<unsigned short*>(b + o_lpix);
+    t.ldepth = b + o_ldep;
+    t.lconf = reinterpret_cast<float*>(b + o_lconf);
+    t.lcount = reinterpret_cast<unsigned*>(b + o_lcnt);
+    t.lcell = reinterpret_cast<unsigned*>(b + o_lcell);
+    t.wslot = reinterpret_cast<unsigned*>(b + o_wslot);
+    t.wmant = reinterpret_cast<float*>(b + o_wmant);
+    t.wexp = reinterpret_cast<int*>(b + o_wexp);
+    t.acc = reinterpret_cast<unsigned long long*>(b + o_acc);
+    t.ckey = reinterpret_cast<unsigned long long*>(b + o_ckey);
     t.cused = reinterpret_cast<unsigned*>(b + o_cused);
     t.cmask = ctx->ccap - 1;
     t.cnt = reinterpret_cast<FrameCounters*>(b + o_cnt);
     t.bitmap = reinterpret_cast<unsigned*>(t.cnt + 1);
     t.bstats = reinterpret_cast<BlockStats*>(b + o_bst);
-    t.n_bstats = n_bstats;
+    t.n_bstats = ctx->geo.count_blocks;
     t.part = reinterpret_cast<Partial*>(b + o_part);
     t.max_partials = max_partials;
     t.staged = reinterpret_cast<CellOut*>(b + o_staged);
@@ -863,7 +950,7 @@ int fuseflow_fuse_points(fuseflow_ctx* ctx, const void* const* depth, const floa
                reinterpret_cast<unsigned long long*>(static_cast<char*>(ctx->d_mc) + kMcBytes),
                (float)ctx->params.depth_scale};
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (launch_points(ctx->d_rig, ctx->d_rays, fp, ctx->tab, pd, ctx->geo.depth_f32 != 0, ctx->n_cams,
+  if (launch_points(ctx->d_rig, ctx->geo.hot, ctx->d_rays, fp, ctx->tab, pd, ctx->geo.depth_f32 != 0, ctx->n_cams,
                     ctx->geo.max_px, s) != cudaSuccess)
     return FUSEFLOW_ERR_CUDA;
   if (n_valid || n_gated) {
@@ -933,9 +1020,8 @@ int fuseflow_read_stage_times(fuseflow_ctx* ctx, double* ms, int64_t* n_frames) 
 // Launch geometry from a (validated) tuning: the count step's grid follows its chunks per
 // block, and the scan step reads exactly the block statistics that grid writes.
 static void apply_tuning(fuseflow_ctx* ctx, const fuseflow_tuning& tu) {
-  ctx->geo.count_chunks = tu.count_chunks;
-  ctx->geo.count_blocks_x = (int)((ctx->max_chunks + tu.count_chunks - 1) / tu.count_chunks);
-  ctx->tab.n_bstats = ctx->geo.count_blocks_x * ctx->n_cams;
+  count_geometry(&ctx->geo, ctx->n_units, tu.count_chunks);
+  ctx->tab.n_bstats = ctx->geo.count_blocks;
   ctx->geo.emit_blocks = tu.emit_blocks;
   ctx->geo.tiles.ahead = tu.prefetch_tiles == 0 ? kNoPrefetch : std::min(tu.prefetch_tiles, kNoPrefetch);
   ctx->geo.pdl = tu.programmatic;
@@ -1023,9 +1109,7 @@ struct Autotuner {
       if ((st = consider(c)) != FUSEFLOW_OK) return st;
     }
     // count_chunks: one wave of b count blocks per SM, for b in 1..8
-    long long total_chunks = 0;
-    for (int i = 0; i < ctx->n_cams; ++i)
-      total_chunks += ((long long)ctx->intr[i].width * ctx->intr[i].height + 2047) / 2048;
+    const long long total_chunks = (ctx->n_units + 7) / 8;
     std::vector<int> chunks = {2, 4, 6, 8, 16};
     for (int b : {1, 2, 3, 4, 6, 8}) {
       const long long per = (total_chunks + (long long)b * sms - 1) / ((long long)b * sms);
@@ -1117,7 +1201,7 @@ int64_t fuseflow_device_bytes(const fuseflow_ctx* ctx) {
 // Allocation-free variant of fuseflow_fuse_frame.
 //
 // All scratch (rig constants, ray tables, hash tables, per-pixel records, scan buffers)
-// lives in one file-scope device array of kStaticBytes (about 23 MiB), held by every GPU
+// lives in one file-scope device array of kStaticBytes (about 31 MiB), held by every GPU
 // that loads this library until the process exits.  Host code never dereferences the
 // array's name: the device address comes from cudaGetSymbolAddress, taken once per device
 // on that device's first call (which also clears the hash tables and synchronizes the
@@ -1132,10 +1216,14 @@ constexpr long long kStaticMaxCells = 1ll << 15;       // 32,768 output cells
 constexpr unsigned kStaticSlots = 1u << 18;            // dense cell slots
 constexpr unsigned kStaticCoarse = 1u << 16;           // coarse hash slots
 constexpr int kStaticMaxRays = 1 << 16;                // sum over cameras of W + H
-constexpr int kStaticMaxPairRays = 6 * kStaticMaxRays;  // float4: 2 (K - 1) sum(W + H)
+constexpr int kStaticMaxPairRays = 6 * kStaticMaxRays;  // bound of 2 (K - 1) sum(W + H)
+// the padded tables of an admitted rig fit in as many float4: 1.5 (K - 1) (sum(W + H) + 62 a camera)
+static_assert(3 * (kStaticMaxPairRays / 2 + 62ll * kMaxCams * kMaxK1) / 2 <= kStaticMaxPairRays, "pair-ray tables fit");
 constexpr long long kStaticWords = kStaticMaxPixels / 32;
 constexpr int kStaticWBlocks = (int)((kStaticWords + 1023) / 1024);
-constexpr int kStaticBStats = kMaxCams * (int)(kStaticMaxPixels / 2048 + 1);   // chunks = 1
+// units of 32 x 8 pixels: at most W H / 256 + W / 32 + H / 8 + 1 a camera
+constexpr int kStaticUnits = (int)(kStaticMaxPixels / 256) + kStaticMaxRays / 8 + kMaxCams;
+constexpr int kStaticBStats = kStaticUnits / 8 + 1;    // chunks = 1
 constexpr int kStaticMaxDevices = 64;
 
 constexpr size_t al256(size_t v) { return (v + 255) / 256 * 256; }
@@ -1150,10 +1238,21 @@ constexpr size_t kSCUsed = al256(kSCoarse + sizeof(CoarseEntry) * kStaticCoarse)
 constexpr size_t kSCnt = al256(kSCUsed + sizeof(unsigned) * kStaticCoarse);
 constexpr size_t kSBStats = al256(kSCnt + sizeof(FrameCounters) + sizeof(unsigned) * kStaticWords);
 constexpr size_t kSPart = al256(kSBStats + sizeof(BlockStats) * kStaticBStats);
-constexpr size_t kSStaged = al256(kSPart + sizeof(Partial) * kStaticMaxPartials);
+// a call uses either the top-k variant's partials or, in the same place, the others' weights and sums
+constexpr size_t kSWMant = al256(kSPart + sizeof(unsigned) * kStaticMaxPixels);
+constexpr size_t kSWExp = al256(kSWMant + sizeof(float) * kStaticMaxPixels);
+constexpr size_t kSAcc = al256(kSWExp + sizeof(int) * kStaticMaxPixels);
+constexpr size_t kSCKey = al256(kSAcc + 8 * sizeof(unsigned long long) * kStaticMaxCells);
+constexpr size_t kSStaged = std::max(al256(kSPart + sizeof(Partial) * kStaticMaxPartials),
+                                     al256(kSCKey + sizeof(unsigned long long) * kStaticMaxCells));
 constexpr size_t kSWPre = al256(kSStaged + sizeof(CellOut) * kStaticMaxCells);
 constexpr size_t kSBSum = al256(kSWPre + sizeof(unsigned) * kStaticWords);
-constexpr size_t kStaticBytes = al256(kSBSum + sizeof(unsigned) * kStaticWBlocks);
+constexpr size_t kSLPix = al256(kSBSum + sizeof(unsigned) * kStaticWBlocks);
+constexpr size_t kSLDepth = al256(kSLPix + sizeof(unsigned short) * kStaticMaxPixels);
+constexpr size_t kSLConf = al256(kSLDepth + sizeof(float) * kStaticMaxPixels);
+constexpr size_t kSLCount = al256(kSLConf + sizeof(float) * kStaticMaxPixels);
+constexpr size_t kSLCell = al256(kSLCount + sizeof(unsigned) * kStaticUnits);
+constexpr size_t kStaticBytes = al256(kSLCell + sizeof(unsigned) * kUnitCells * kStaticUnits);
 static_assert(kStaticBytes <= (32u << 20), "static scratch must stay modest");
 
 __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
@@ -1214,9 +1313,19 @@ Tables static_tables(unsigned char* base, long long n_px, int n_bstats) {
   t.n_bstats = n_bstats;
   t.part = reinterpret_cast<Partial*>(base + kSPart);
   t.max_partials = kStaticMaxPartials;
+  t.wslot = reinterpret_cast<unsigned*>(base + kSPart);
+  t.wmant = reinterpret_cast<float*>(base + kSWMant);
+  t.wexp = reinterpret_cast<int*>(base + kSWExp);
+  t.acc = reinterpret_cast<unsigned long long*>(base + kSAcc);
+  t.ckey = reinterpret_cast<unsigned long long*>(base + kSCKey);
   t.staged = reinterpret_cast<CellOut*>(base + kSStaged);
   t.wprefix = reinterpret_cast<unsigned*>(base + kSWPre);
   t.bsum = reinterpret_cast<unsigned*>(base + kSBSum);
+  t.lpix = reinterpret_cast<unsigned short*>(base + kSLPix);
+  t.ldepth = base + kSLDepth;
+  t.lconf = reinterpret_cast<float*>(base + kSLConf);
+  t.lcount = reinterpret_cast<unsigned*>(base + kSLCount);
+  t.lcell = reinterpret_cast<unsigned*>(base + kSLCell);
   t.n_words = (n_px + 31) / 32;
   t.n_wblocks = (int)((t.n_words + 1023) / 1024);
   return t;
@@ -1254,17 +1363,16 @@ extern "C" int fuseflow_fuse_frame_static(const fuseflow_intrinsics* intr,
   if (!depth || !conf || !rgb || !pos || !rgb_out || !weight || !count || !rep || !key || !stats)
     return FUSEFLOW_ERR_INVALID_ARG;
   if (screen_set(params)) return FUSEFLOW_ERR_INVALID_ARG;     // no D^r buffer in the arena
-  long long n_px = 0, max_px = 0, n_rays = 0;
+  const int K = std::min<int>(params->k_views, n_cams);
+  const int k1 = K - 1;
+  long long n_px = 0, n_rays = 0, np = 0;
   for (int i = 0; i < n_cams; ++i) {
-    const long long px = (long long)intr[i].width * intr[i].height;
-    n_px += px;
-    max_px = std::max(max_px, px);
+    n_px += (long long)intr[i].width * intr[i].height;
     n_rays += intr[i].width + intr[i].height;
+    np += pray_cam_size(intr[i].width, intr[i].height, k1);
     if (!depth[i] || !conf[i] || !rgb[i]) return FUSEFLOW_ERR_INVALID_ARG;
   }
   const long long max_cells = params->max_cells > 0 ? params->max_cells : kStaticMaxCells;
-  const int K = std::min<int>(params->k_views, n_cams);
-  const int k1 = K - 1;
   if (n_px > kStaticMaxPixels || n_rays > kStaticMaxRays || max_cells > kStaticMaxCells ||
       2ll * k1 * n_rays > kStaticMaxPairRays)
     return FUSEFLOW_ERR_CAPACITY;
@@ -1290,14 +1398,8 @@ extern "C" int fuseflow_fuse_frame_static(const fuseflow_intrinsics* intr,
   RigDev& rig = g_static_rig;
   build_rig(intr, extr, n_cams, params, nbr, k1, rig, g_static_rays, g_static_pray);
   const int nr = (int)n_rays;
-  const int np = (int)(2ll * k1 * n_rays);
   Geometry geo{};
   const int n_tiles = fill_tile_index(rig, &geo.tiles, 16);
-  {
-    int sm_count = 152;
-    cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
-    geo.tiles.ahead = assign_resident_blocks(16, rig.k1) * sm_count;
-  }
   fill_block_consts(rig, g_static_bconst);
   // pageable host -> device copies return once the host buffers have been read
   if (cudaMemcpyAsync(base + kSBConst, g_static_bconst, sizeof(BlockConst) * (size_t)n_cams,
@@ -1310,15 +1412,17 @@ extern "C" int fuseflow_fuse_frame_static(const fuseflow_intrinsics* intr,
     return FUSEFLOW_ERR_CUDA;
 
   geo.n_cams = n_cams;
+  geo.hot = rig.hot;
   geo.top_k = params->top_k;
   geo.depth_f32 = rig.depth_f32;
-  geo.count_blocks_x = (int)((max_px + 2047) / 2048);
-  geo.count_chunks = 1;
+  const int n_units = geo.tiles.unit[n_cams];
+  count_geometry(&geo, n_units, 1);
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   geo.emit_blocks = std::max(1, sms * 8);
   geo.pdl = 2;                                         // at most 2^19 pixels: small frames
-  Tables t = static_tables(base, n_px, geo.count_blocks_x * n_cams);
+  Tables t = static_tables(base, n_px, geo.count_blocks);
+  t.n_units = n_units;
   t.n_min = params->n_min;
   t.max_level = params->max_level;
   t.bconst = reinterpret_cast<const BlockConst*>(base + kSBConst);

@@ -18,12 +18,14 @@ namespace ffl {
 
 constexpr int kMaxCams = 64;
 constexpr int kMaxK1 = 8;
-constexpr int kMaxTopK = 7;              // top-k keys travel in a partial record (rep + 6)
+constexpr int kMaxTopK = 7;              // top-k keys travel in a partial record
 constexpr unsigned long long kKeyEmpty = ~0ull;
 constexpr uint32_t kSlotNone = 0xffffffffu;
+constexpr uint32_t kSlotPending = 0xfffffffeu;
 constexpr int kFixShift = 36;            // per-cell fixed point: largest member weight ~ 2^36
 constexpr int kKeyBias = 1 << 19;        // cell index range [-2^19, 2^19) per axis
-constexpr float kTieBandPx = 4e-3f;      // float32 projection error bound (pixels), generous
+constexpr float kGridM = 12582912.0f;    // 1.5 2^23: adding it rounds |v| < 2^22 to an integer
+constexpr int kGridBits = 0x4B400000;    // its bits: an integer n is bits(kGridM + n) - kGridBits
 
 // error bits of FrameCounters::error
 constexpr unsigned kErrSlots = 1u;       // the cells' dense slot ranges exceed the slot capacity
@@ -47,23 +49,28 @@ struct CamDev {
 };
 
 struct PairDev {                 // camera i -> neighbour j: a = R_ji p_c + t_ji
-  float Rh[9], Rl[9];            // R_ji = R_j R_i^T as ff
-  float th[3], tl[3];            // t_ji = t_j - R_ji t_i as ff (depth units)
+  float th[3], tl[3];            // t_ji = t_j - R_ji t_i in grid units: th integral, tl the rest
   int j;
-  // separable pair rays: with p_c = z (rx(x), ry(y), 1), R_ji p_c = z (A(x) + B(y)),
-  // A_k(x) = R_ji[k][0] rx(x) + R_ji[k][2] and B_k(y) = R_ji[k][1] ry(y), each stored as
-  // ff in two float4 per column / row: (A0h, A0l, A1h, A1l), (A2h, A2l, 0, 0)
-  int ga, gb;                    // float4 index of column 0's A and row 0's B
-  int pad;
+};
+
+// Scalars of a rig that the frame kernels use per pixel; passed by value (constant bank).
+// The consistency step works in "grid units" (kGridM below): ginv grid units per depth unit, a
+// power of two chosen so that every camera-frame coordinate of the rig (depths up to zmax) is
+// below 2^22 of them.
+struct RigHot {
+  float tau;                     // Eq. 9 gate
+  int use_conf, use_cons;
+  int max_level;
+  float inv_s0u;                 // 1 / s0 in 1 / depth units
+  float einv_h, einv_l;          // 1 / (sigma^2 (K-1)) in 1 / grid units^2, as ff
+  float ginv;                    // grid units per depth unit
+  float zmax;                    // largest depth (depth units) the grid evaluation covers
 };
 
 struct RigDev {
   int n_cams, k1;                // k1 = K - 1 neighbours per camera
-  float tau;                     // Eq. 9 gate
-  int use_conf, use_cons;
-  int max_level, n_min;
-  float inv_s0u;                 // 1 / s0 in 1 / depth units
-  float einv_h, einv_l;          // 1 / (sigma_u^2 (K-1)) as ff
+  RigHot hot;
+  int n_min;
   int depth_f32;
   int top_k;                     // Sec. II.5(2)a variant: fuse the top_k members only (0: all)
   long long n_px;
@@ -71,62 +78,95 @@ struct RigDev {
   PairDev pair[kMaxCams * kMaxK1];
 };
 
-// Constants of one camera's tiles: the camera, its K-1 neighbour pairs and the neighbour
-// cameras, contiguous so that a block copies them to shared memory in one round trip.
-struct BlockConst {
-  CamDev cam;
-  PairDev pair[kMaxK1];
-  CamDev nb[kMaxK1];
+// What the consistency step reads of one camera's tiles, packed so that a tile copies it in a
+// few 16-byte words: the camera's pose and, per neighbour view, its projection.  Everything in
+// grid units; rare exact decisions read RigDev instead.
+struct __align__(16) CamHot {
+  float Rwc[9], cwc[3];          // world-from-camera pose (depth units)
+  int ray_x, ray_y;              // offsets of the camera's ray tables
+  int pray;                      // float4 index of its pair rays
+  int pair0;                     // its first PairDev
 };
+struct __align__(16) ViewHot {
+  float mt[3];                   // kGridM + integral part of t_ji
+  float tl[3];                   // rest of t_ji
+  float fx, fy, cx5, cy5;        // projection into view j; principal point + 1/2
+  int W, H;
+  int ray_x, ray_y;              // offsets of view j's ray tables
+  float band;                    // |u - integer| below this is decided exactly (pixels)
+  int j;
+};
+struct BlockConst {
+  CamHot cam;
+  ViewHot view[kMaxK1];
+};
+static_assert(sizeof(CamHot) == 64 && sizeof(ViewHot) == 64, "16-byte words of a tile's constants");
 
-// Where the assign step's tiles are: camera i owns tiles [first[i], first[i+1]), row-major
-// over its ceil(W/32) x ceil(H/th) grid.  Passed by value (constant bank) to the kernel.
+// Separable pair rays (Eq. 4): with p_c = z (rx(x), ry(y), 1), R_ji p_c = z (A(x) + B(y)),
+// A_k(x) = R_ji[k][0] rx(x) + R_ji[k][2] and B_k(y) = R_ji[k][1] ry(y), in grid units per depth
+// unit, each an ff whose high parts are multiples of one power of two, so that the sum of two
+// high parts is exact.  Per camera, columns go in groups of 32 and rows in groups of 8; a group
+// holds, view after view, a plane of (0h, 1h, 2h, 0l) and a plane of (1l, 2l), so that a tile's
+// share is contiguous and its planes are read without bank conflicts.  Padded to 32 columns / rows.
+constexpr int kPrayColGroup = 48;          // float4 per view and 32 columns
+constexpr int kPrayRowGroup = 12;          // float4 per view and 8 rows
+__host__ __device__ inline long long pray_cam_size(int W, int H, int k1) {   // float4 of one camera
+  return (long long)k1 * ((W + 31) / 32 * kPrayColGroup + (H + 31) / 32 * 4 * kPrayRowGroup);
+}
+
+// Where the assign step's tiles are: camera i owns tiles [first[i], first[i+1]), row-major over its
+// ceil(W/32) x ceil(H/th) grid; and its units of 32 x 8 pixels, the count step's share of a warp and
+// the grain of the lists of gated pixels: units [unit[i], unit[i+1]), row-major over ceil(W/32) x
+// ceil(H/8).  A unit's list starts where its pixels would if the image were stored unit by unit
+// (unit_list).  Passed by value (constant bank) to the kernels.
 struct TileIndex {
   int n_cams, k1;
   int th;                        // tile height (8, 16 or 32 rows of 32 columns)
   int first[kMaxCams + 1];
+  int unit[kMaxCams + 1];
   int W[kMaxCams], H[kMaxCams];
+  unsigned div_x[kMaxCams];      // fast_div factor of the camera's tile columns
   long long off[kMaxCams];       // global index of each camera's pixel (0, 0)
-  int pray[kMaxCams];            // float4 index of the camera's first pair ray: pair q's A
-                                 // starts at pray + 2 q (W + H), its B 2 W further
-  int per_cam;                   // tiles per camera when all cameras share W and H, else 0
+  int pray[kMaxCams];            // float4 index of the camera's pair rays: column groups, then rows
+  int per_cam, units_per_cam;    // tiles and units per camera when all cameras share W and H, else 0
+  unsigned div_cam, div_units;   // their fast_div factors
   int ahead;                     // tiles resident at once: block b prefetches tile b + ahead
 };
+constexpr int kUnitH = 8;
+constexpr int kUnitCells = 64;   // numbers that a unit's coarse cells can have
+constexpr unsigned kNoCellNumber = 0xffu;
 
-// Per (tile, cell) partial result of the assign step, pushed onto its cell's list when it
-// is written.  Sums are exact integers in units of 2^-(kFixShift + mmin) of the tile's own
-// smallest weight exponent mmin; the reduce step shifts them to the cell's smallest one.
-// Each sum is below 2^46 (at most 512 terms below 2^37), so 48 bits hold it: the record is
-// 64 bytes, two aligned 32-byte sectors.
+// First list entry of the unit at (x0, y0) of a camera of W x H pixels whose first pixel is off.
+__host__ __device__ inline long long unit_list(long long off, int W, int H, int x0, int y0) {
+  return off + (long long)y0 * W + (long long)x0 * (H - y0 < kUnitH ? H - y0 : kUnitH);
+}
+
+// n / d and the remainder, for a divisor whose factor floor((2^32 - 1) / d) is known: the product's
+// upper half is the quotient or one or two below it.
+__host__ __device__ inline unsigned fast_div_factor(unsigned d) { return 0xffffffffu / d; }
+__device__ __forceinline__ int fast_div(int n, int d, unsigned factor, int& rem) {
+  int q = (int)__umulhi((unsigned)n, factor);
+  rem = n - q * d;
+  if (rem >= d) { ++q; rem -= d; }
+  if (rem >= d) { ++q; rem -= d; }
+  return q;
+}
+
+// Top-k variant: per (tile, cell) partial result of the assign step, pushed onto its cell's list when
+// it is written; two aligned 32-byte sectors.
 struct __align__(64) Partial {
-  unsigned long long rep;        // max of ordered(C) << 32 | ~g (top-k: the tile's first key)
   unsigned next;                 // next partial of the same cell, kSlotNone at the end
   unsigned count;                // members in the tile
-  union {
-    struct {
-      int mmin;                  // smallest weight exponent m in the tile
-      unsigned lo[7];            // bits 0..31 of the sums of w, w frac_x, w frac_y, w frac_z,
-      unsigned short hi[7];      //   w r, w g, w b; bits 32..47
-      unsigned short pad;
-    } sum;
-    unsigned long long top[kMaxTopK - 1];   // top-k variant: the tile's keys 2..k
-  };
-  __device__ __forceinline__ void set_sum(int a, unsigned long long v) {
-    sum.lo[a] = (unsigned)v;
-    sum.hi[a] = (unsigned short)(v >> 32);
-  }
-  __device__ __forceinline__ unsigned long long get_sum(int a) const {
-    return ((unsigned long long)sum.hi[a] << 32) | sum.lo[a];
-  }
+  unsigned long long top[kMaxTopK];       // the tile's k largest ordered(C) << 32 | ~g, then 0
 };
 static_assert(sizeof(Partial) == 64, "partial record layout");
 
-// Per dense cell slot: the cell's key, its list head and its smallest weight exponent, in
-// one 16-byte record so that the reduce step reads a single sector per cell.
+// Per dense cell slot, in one 16-byte record so that a point reads a single sector.
 struct __align__(16) SlotRec {
-  unsigned long long key;
-  unsigned head;                 // last partial pushed, kSlotNone if none
-  int mmin;                      // smallest weight exponent over the cell's partials
+  unsigned long long key;        // representative: largest ordered(C) << 32 | ~g (top-k: the cell's key)
+  unsigned head;                 // the cell's number, kSlotPending while its claim is under way (top-k:
+                                 // last partial pushed); kSlotNone if none
+  int mmin;                      // smallest weight exponent of the cell's members
 };
 
 // Coarse hash-table record: key, density count (Sec. II.5(1)c) and, once every count is
@@ -193,6 +233,12 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long k) {
   return k;
 }
 
+// First table position of coarse cell (x, y, z): rows of cells lie side by side in the table, at
+// offsets scattered by odd multipliers.
+__device__ __forceinline__ unsigned coarse_hash(int x, int y, int z) {
+  return (unsigned)x + (unsigned)y * 0x9E3779B1u + (unsigned)z * 0x85EBCA77u;
+}
+
 __device__ __forceinline__ unsigned long long pack_key(int l, int kx, int ky, int kz) {
   return ((unsigned long long)l << 60) | ((unsigned long long)(kx + kKeyBias) << 40) |
          ((unsigned long long)(ky + kKeyBias) << 20) | (unsigned long long)(kz + kKeyBias);
@@ -211,28 +257,6 @@ __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& 
 __device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
   p = __fmul_rn(a, b);
   e = __fmaf_rn(a, b, -p);
-}
-
-// Row k of an affine map in ff: o = R[k,:] . (px, py, z) + t[k], with px, py ff and z exact.
-__device__ __forceinline__ void ff_affine_row(const float* Rh, const float* Rl, float th, float tl,
-                                              float pxh, float pxl, float pyh, float pyl, float z,
-                                              float& oh, float& ol) {
-  float p1, e1, p2, e2, p3, e3;
-  two_prod(Rh[0], pxh, p1, e1);
-  e1 = __fmaf_rn(Rh[0], pxl, e1);
-  e1 = __fmaf_rn(Rl[0], pxh, e1);
-  two_prod(Rh[1], pyh, p2, e2);
-  e2 = __fmaf_rn(Rh[1], pyl, e2);
-  e2 = __fmaf_rn(Rl[1], pyh, e2);
-  two_prod(Rh[2], z, p3, e3);
-  e3 = __fmaf_rn(Rl[2], z, e3);
-  float s, q1, q2, q3;
-  two_sum(p1, p2, s, q1);
-  two_sum(s, p3, s, q2);
-  two_sum(s, th, s, q3);
-  const float lo = __fadd_rn(__fadd_rn(__fadd_rn(e1, e2), __fadd_rn(e3, q1)),
-                             __fadd_rn(__fadd_rn(q2, q3), tl));
-  fast_two_sum(s, lo, oh, ol);
 }
 
 // One component of a = z (A + B) + t in ff (A, B, t as ff, z exact); the result (oh, ol)
@@ -261,7 +285,8 @@ template <> struct Depth<float> {
 
 // Eq. 8 in float32: world point (depth units) of pixel ray (rx, ry, 1) at z-depth z.
 // Every step uses the same rounding-explicit sequence so all kernels agree bit for bit.
-__device__ __forceinline__ void world_point(const CamDev& c, float z, float rx, float ry,
+template <typename Cam>                  // CamDev or CamHot
+__device__ __forceinline__ void world_point(const Cam& c, float z, float rx, float ry,
                                             float P[3]) {
   const float px = __fmul_rn(z, rx), py = __fmul_rn(z, ry);
 #pragma unroll
@@ -275,21 +300,19 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) 
 
 // Sec. II.5(1): coarse-grid coordinate r = P / s0 and the range test at the finest level:
 // floor(r 2^Lmax) in [-2^19, 2^19)  <=>  r 2^Lmax in [-2^19, 2^19).
-__device__ __forceinline__ bool grid_coords(const RigDev& rig, const float P[3], float r[3]) {
+// The range test is on floor(r): in [-2^(19-Lmax), 2^(19-Lmax)).  floor(v) of |v| < 2^22 is read
+// off the bits of kGridM + v rounded down; outside, and for NaN, the bits give an integer that
+// fails the range test (they are monotonic in v, and at least 2^22 away once wrapped).
+__device__ __forceinline__ bool grid_coords(const RigHot& rig, const float P[3], float r[3], int c[3]) {
+  const unsigned lim = (unsigned)kKeyBias >> rig.max_level;
   bool ok = true;
-  const float lim = (float)kKeyBias;
-  const float sL = pow2f(rig.max_level);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     r[k] = __fmul_rn(P[k], rig.inv_s0u);
-    const float v = __fmul_rn(r[k], sL);
-    ok = ok && (v >= -lim) && (v < lim);
+    c[k] = __float_as_int(__fadd_rd(r[k], kGridM)) - kGridBits;
+    ok = ok && (unsigned)c[k] + lim < 2u * lim;
   }
   return ok;
-}
-
-__device__ __forceinline__ unsigned long long coarse_key(const float r[3]) {
-  return pack_key(0, (int)floorf(r[0]), (int)floorf(r[1]), (int)floorf(r[2]));
 }
 
 // Sec. II.5(1)d: level of a coarse cell holding n_c points: largest l <= Lmax with
@@ -299,12 +322,6 @@ __device__ __forceinline__ int level_for(unsigned n_c, int n_min, int max_level)
   for (int c = 1; c <= max_level; ++c)
     if ((unsigned long long)n_c >= ((unsigned long long)n_min << (2 * c))) l = c;
   return l;
-}
-
-__device__ __forceinline__ unsigned long long fine_key(const float r[3], int l) {
-  const float sl = pow2f(l);
-  return pack_key(l, (int)floorf(__fmul_rn(r[0], sl)), (int)floorf(__fmul_rn(r[1], sl)),
-                  (int)floorf(__fmul_rn(r[2], sl)));
 }
 
 }  // namespace ffl

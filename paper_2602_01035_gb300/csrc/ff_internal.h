@@ -27,7 +27,14 @@ struct Tables {                  // context-owned device scratch
   FrameCounters* cnt;
   BlockStats* bstats;            // one per block of the coarse-count step
   int n_bstats;
-  Partial* part;                 // (tile, cell) partials, max_partials entries
+  // by list entry: level << 27 | dense slot of a gated pixel, its weight as mantissa and exponent
+  unsigned* wslot;
+  float* wmant;
+  int* wexp;
+  // by cell number, max_cells entries: exact sums of Eq. 11 (eight a cell) and the cell's key
+  unsigned long long* acc;
+  unsigned long long* ckey;
+  Partial* part;                 // top-k variant: (tile, cell) partials, max_partials entries
   unsigned max_partials;
   CellOut* staged;               // fused cells by claim order, max_cells entries
   unsigned* bitmap;              // representative bitmap, one bit per pixel
@@ -37,8 +44,15 @@ struct Tables {                  // context-owned device scratch
   int n_wblocks;
   int n_min, max_level;          // level rule (Sec. II.5(1)d)
   const BlockConst* bconst;      // per-camera block constants
-  const float4* pray;            // separable pair rays (PairDev::ga, gb)
-  int n_tiles;
+  const float4* pray;            // separable pair rays (TileIndex::pray)
+  int n_tiles, n_units;
+  // gated pixels, unit by unit (unit_list): pixel of the unit | number of its coarse cell << 8,
+  // depth sample, confidence; per unit, the pixels listed and the positions of the numbered cells
+  unsigned short* lpix;
+  void* ldepth;
+  float* lconf;
+  unsigned* lcount;
+  unsigned* lcell;               // kUnitCells a unit
 };
 
 struct TraceDev {
@@ -76,9 +90,10 @@ struct FrameArgs {
   TraceDev tr;
   OutDev out;
   TileIndex ti;
-  int count_blocks_x, count_chunks;
+  RigHot hot;
+  int count_chunks;
   float unit_m;
-  int pad;
+  int top_k;
 };
 
 // Frames of one launch of the frame kernels, passed as one __grid_constant__ kernel
@@ -115,12 +130,13 @@ struct Geometry {
   int screen;                    // a screen is set: fuse calls write D^r into screen_buf first
   ScreenArgs scr;                // bounds, sizes and the context's D^r buffers (out)
   long long max_px;
-  int count_blocks_x;            // blocks per camera of the coarse-count step (max over cams)
-  int count_chunks;              // 2048-pixel chunks per block of the coarse-count step
+  int count_blocks;              // blocks of the coarse-count step
+  int count_chunks;              // chunks of 8 units (2048 pixels) per block of the coarse-count step
   int emit_blocks;
   int top_k;                     // Sec. II.5(2)a variant (0: every member is fused)
   int pdl;                       // programmatic launches: 0 none, 1 all but assign -> reduce, 2 all
   TileIndex tiles;               // assign-step tiles
+  RigHot hot;                    // the rig's per-pixel scalars
 };
 
 cudaError_t launch_init_tables(const Tables& t, unsigned fcap, unsigned ccap, cudaStream_t s);
@@ -168,7 +184,7 @@ struct PointsDev {
   unsigned long long* counts;
   float unit_f;
 };
-cudaError_t launch_points(const RigDev* rig, const float2* rays, const FramePtrs& fp, const Tables& t,
+cudaError_t launch_points(const RigDev* rig, const RigHot& hot, const float2* rays, const FramePtrs& fp, const Tables& t,
                           const PointsDev& out, bool depth_f32, int n_cams, long long max_px,
                           cudaStream_t s);
 
@@ -187,7 +203,7 @@ cudaError_t launch_confidence(const ConfArgs& a, bool depth_f32, int max_w, int 
 
 // assign-step blocks resident per SM for tiles of th rows and k1 neighbour views
 int assign_resident_blocks(int th, int k1);
-// tiles of th rows (8, 16 or 32) of the rig's cameras; returns their number
+// tiles of th rows (8, 16 or 32) and units of the rig's cameras; returns the number of tiles
 int fill_tile_index(const RigDev& rig, TileIndex* out, int th);
 // the same index re-cut into tiles of th rows; returns their number
 int retile(TileIndex* ti, int th);

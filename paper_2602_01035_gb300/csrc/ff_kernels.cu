@@ -4,20 +4,20 @@
 // optionally as programmatic dependent launches, see pdl_release / pdl_wait):
 //   memset   frame counters + representative bitmap
 //   screen   (only with a depth screen set) D^r of Eq. 8 into the context's buffers
-//   count    (a) decode + gate + back-project (Eq. 8, 9), coarse density n_c (Sec. II.5(1)c)
-//            from equal-cell runs merged across each warp, per-block pixel counts and
-//            extent (Sec. II.5(1)b)
+//   count    (a) decode + gate (Eq. 9) of units of 32x8 pixels, a warp each; the gated pixels are
+//            listed, back-projected (Eq. 8) and counted per coarse cell (Sec. II.5(1)c); per-block
+//            pixel counts and extent (Sec. II.5(1)b)
 //   levels   level of each coarse cell (Sec. II.5(1)d) and its range of 8^level dense
 //            cell slots
-//   assign   per 32x16 tile: (b) consistency V (Eq. 4-7) in double-float, omega = C V
-//            (Eq. 10) as mantissa/exponent; (c) cell key (Sec. II.5(1)e) and dense slot;
-//            (d) per (tile, cell): member count, representative (Sec. II.5(2)a), smallest
-//            weight exponent and exact fixed-point sums of omega, omega P, omega RGB
-//            (Eq. 11), written as one partial record pushed onto its cell's list
-//   reduce   per cell: walk its partials, combine them, stage the fused cell, mark its
-//            representative; the used slots and coarse entries are cleared for the next frame
-//            (top-k variant: k_reduce_topk weighs and fuses each cell's k most confident
-//            members here instead)
+//   weigh    per listed pixel: (b) consistency V (Eq. 4-7) on the rig's grid, omega = C V (Eq. 10)
+//            as mantissa/exponent; (c) cell key (Sec. II.5(1)e) and dense slot; per cell its
+//            representative (Sec. II.5(2)a) and smallest weight exponent
+//   sum      (d) exact fixed-point sums of omega, omega P, omega RGB per cell (Eq. 11) at the scale
+//            of its smallest exponent
+//   reduce   per cell: Eq. 11 from its sums, stage the fused cell, mark its representative; the used
+//            slots and coarse entries are cleared for the next frame
+//            (top-k variant: k_assign_topk keeps each tile's most confident members of a cell
+//            instead of weigh and sum, and k_reduce_topk weighs and fuses each cell's k)
 //   scan     ranks of the representatives (output order) and frame statistics
 //   emit     fused cells in representative order
 // Outside the frame sequence: k_copyout (served frames: cloud into pinned host memory),
@@ -29,6 +29,8 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
+#include <cmath>
+#include <cstring>
 #include <cstdint>
 
 #include "ff_internal.h"
@@ -38,20 +40,23 @@ namespace ffl {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kCountPx = 8;                       // pixels per thread in the count step
-constexpr int kCountBlockPx = kThreads * kCountPx;
-constexpr int kTileW = 32;                        // assign tile: 32 columns by TH rows
+constexpr int kTileW = 32;                        // tiles: 32 columns by TH rows
 constexpr int kMaxProbe = 1 << 14;
 constexpr float kLn2H = 0.693147182464599609375f;         // float(ln 2)
 constexpr float kLn2L = -1.904654299957768e-09f;          // ln 2 - kLn2H
 constexpr float kInvLn2 = 1.44269504088896340736f;
 
 // ------------------------------------------------------------------ global hash tables
+__device__ __forceinline__ unsigned coarse_slot(unsigned long long key, unsigned cmask) {
+  return coarse_hash((int)((key >> 40) & 0xfffff), (int)((key >> 20) & 0xfffff), (int)(key & 0xfffff)) & cmask;
+}
 __device__ __forceinline__ unsigned coarse_insert(const Tables& t, unsigned long long key) {
-  unsigned h = (unsigned)mix64(key) & t.cmask;
+  unsigned h = coarse_slot(key, t.cmask);
   for (int probe = 0; probe < kMaxProbe; ++probe) {
-    // one round trip per probe: the swap either claims an empty slot or reports its key
-    const unsigned long long cur = atomicCAS(&t.coarse[h].key, kKeyEmpty, key);
+    // most keys are there already: a look first keeps their lines free of serialised swaps
+    unsigned long long cur = __ldcg(&t.coarse[h].key);
+    if (cur == key) return h;
+    if (cur == kKeyEmpty) cur = atomicCAS(&t.coarse[h].key, kKeyEmpty, key);
     if (cur == kKeyEmpty) {
       const unsigned n = atomicAdd(&t.cnt->n_coarse, 1u);
       if (n <= t.cmask) t.cused[n] = h;
@@ -64,15 +69,14 @@ __device__ __forceinline__ unsigned coarse_insert(const Tables& t, unsigned long
   return kSlotNone;
 }
 
-// Level and slot base (packed level << 27 | base) of an existing coarse key, continuing a
-// probe whose first record `e` (at position h) was loaded earlier.
-__device__ __forceinline__ unsigned coarse_lvbase(const Tables& t, unsigned long long key,
-                                                  unsigned h, ulonglong2 e) {
+// Level and slot base (packed level << 27 | base) of an existing coarse key.
+__device__ __forceinline__ unsigned coarse_lvbase(const Tables& t, unsigned long long key) {
+  unsigned h = coarse_slot(key, t.cmask);
   for (int probe = 0; probe < kMaxProbe; ++probe) {
+    const ulonglong2 e = __ldcg(reinterpret_cast<const ulonglong2*>(&t.coarse[h]));
     if (e.x == key) return (unsigned)(e.y >> 32);
     if (e.x == kKeyEmpty) break;
     h = (h + 1) & t.cmask;
-    e = __ldcg(reinterpret_cast<const ulonglong2*>(&t.coarse[h]));
   }
   atomicOr(&t.cnt->error, kErrCoarseMiss);
   return kBaseNone;
@@ -139,38 +143,26 @@ __global__ void __launch_bounds__(kThreads) k_levels(const __grid_constant__ Bat
   }
 }
 
-// Block-local open addressing (shared memory); returns the table position or -1, and sets
-// `fresh` when this call inserted the key.  32-bit keys (dense cell slots) take a
-// multiplicative (Fibonacci) hash, 64-bit keys (packed coarse keys) the 64-bit mixer.
-template <int TS, typename K>
-__device__ __forceinline__ int local_pos(K* tab, K empty, K key, int max_probe, bool& fresh) {
-  unsigned h;
-  if constexpr (sizeof(K) == 4) {
-    constexpr int kBits = TS == 512 ? 9 : TS == 1024 ? 10 : TS == 2048 ? 11 : TS == 4096 ? 12 : 0;
-    static_assert(kBits > 0, "block table size");
-    h = ((unsigned)key * 0x9E3779B1u) >> (32 - kBits);
-  } else {
-    h = (unsigned)mix64((unsigned long long)key) & (TS - 1);
-  }
+// Block-local open addressing of dense cell slots (shared memory, Fibonacci hash); returns the table
+// position or -1, and sets `fresh` when this call inserted the slot.
+template <int TS>
+__device__ __forceinline__ int local_pos(unsigned* tab, unsigned key, bool& fresh) {
+  constexpr int kBits = TS == 512 ? 9 : TS == 1024 ? 10 : TS == 2048 ? 11 : 0;
+  static_assert(kBits > 0, "block table size");
+  unsigned h = (key * 0x9E3779B1u) >> (32 - kBits);
   fresh = false;
-  for (int probe = 0; probe < max_probe; ++probe) {
-    const K cur = *static_cast<volatile K*>(&tab[h]);
+  for (int probe = 0; probe < TS; ++probe) {
+    const unsigned cur = *static_cast<volatile unsigned*>(&tab[h]);
     if (cur == key) return (int)h;
-    if (cur == empty) {
-      const K prev = atomicCAS(&tab[h], empty, key);
-      fresh = prev == empty;
+    if (cur == kSlotNone) {
+      const unsigned prev = atomicCAS(&tab[h], kSlotNone, key);
+      fresh = prev == kSlotNone;
       if (fresh || prev == key) return (int)h;
     }
     h = (h + 1) & (TS - 1);
   }
   return -1;
 }
-template <int TS, typename K>
-__device__ __forceinline__ int local_pos(K* tab, K empty, K key, int max_probe = TS) {
-  bool fresh;
-  return local_pos<TS>(tab, empty, key, max_probe, fresh);
-}
-
 
 // ------------------------------------------------------------------ Eq. 4-7 per point
 // Exact floor(u + 1/2) for u = fx a_x / a_z + cx near a tie at integer r (a_z > 0):
@@ -189,119 +181,221 @@ __device__ __forceinline__ int exact_round(float fh, float fl, float ch, float c
   return (f >= 0.0f) ? (int)r : (int)r - 1;
 }
 
-// Sum over the K-1 neighbour views of d_ij^2 (Eq. 6) in depth units^2, as ff (sh, sl).
-// A pixel at z-depth z; the transform into view j (Eq. 4) uses the pixel's separable pair
-// rays (from the tile's shared-memory copy or the global tables), so that
-// a = z (A(x) + B(y)) + t_ji costs one ff sum, one ff product and one ff sum per component.
-// Views go in groups of kViewGroup: every view of a group is projected and its depth gather
-// issued before any residual is formed.  Groups of one measure fastest on GB300 (larger
-// groups spill at four blocks per SM and grow the code past the instruction cache).
-constexpr int kViewGroup = 1;
-
-// Pair rays of a tile of TH rows staged in shared memory (pixel (lx, ly) of the tile): per
-// view, A of the 32 columns and B of the TH rows, each as two float4 planes.
+// Pair rays of a tile of TH rows staged in shared memory (pixel (lx, ly) of the tile): the
+// tile's column group, then its row groups (layout: kPrayColGroup, kPrayRowGroup).
 template <int TH>
 struct TilePairRays {
-  const float4* s_pr;
-  int lx, ly;
-  __device__ __forceinline__ void operator()(int q, const PairDev&, float4& a01, float4& a2,
-                                             float4& b01, float4& b2) const {
-    const float4* pr = s_pr + q * (2 * kTileW + 2 * TH);
-    a01 = pr[lx];
-    a2 = pr[kTileW + lx];
-    b01 = pr[2 * kTileW + ly];
-    b2 = pr[2 * kTileW + TH + ly];
+  const float4* a4;
+  const float2* a2;
+  const float4* b4;
+  const float2* b2;
+  __device__ __forceinline__ TilePairRays(const float4* s_cols, const float4* s_rows, int k1, int lx, int ly)
+      : a4(s_cols + lx), a2(reinterpret_cast<const float2*>(s_cols + 32) + lx) {
+    const float4* rows = s_rows + (ly >> 3) * k1 * kPrayRowGroup;
+    b4 = rows + (ly & 7);
+    b2 = reinterpret_cast<const float2*>(rows + 8) + (ly & 7);
+  }
+  __device__ __forceinline__ void operator()(int q, float4& a, float2& al, float4& b, float2& bl) const {
+    a = a4[q * kPrayColGroup];
+    al = a2[q * 2 * kPrayColGroup];
+    b = b4[q * kPrayRowGroup];
+    bl = b2[q * 2 * kPrayRowGroup];
   }
 };
 
-// Pair rays read from the global tables (pixel (x, y) of the camera).
+// Pair rays read from the global tables: pixel (x, y) of a camera of width W whose rays start
+// at pray.
 struct GlobalPairRays {
-  const float4* pray;
-  int x, y;
-  __device__ __forceinline__ void operator()(int, const PairDev& P, float4& a01, float4& a2,
-                                             float4& b01, float4& b2) const {
-    a01 = __ldg(pray + P.ga + 2 * x);
-    a2 = __ldg(pray + P.ga + 2 * x + 1);
-    b01 = __ldg(pray + P.gb + 2 * y);
-    b2 = __ldg(pray + P.gb + 2 * y + 1);
+  const float4* cols;
+  const float4* rows;
+  int ix, iy;
+  __device__ __forceinline__ GlobalPairRays(const float4* pray, int W, int k1, int x, int y)
+      : cols(pray + (long long)(x >> 5) * k1 * kPrayColGroup),
+        rows(pray + ((long long)((W + 31) >> 5) * kPrayColGroup + (long long)(y >> 3) * kPrayRowGroup) * k1),
+        ix(x & 31), iy(y & 7) {}
+  __device__ __forceinline__ void operator()(int q, float4& a, float2& al, float4& b, float2& bl) const {
+    const float4* c = cols + q * kPrayColGroup;
+    const float4* r = rows + q * kPrayRowGroup;
+    a = __ldg(c + ix);
+    al = __ldg(reinterpret_cast<const float2*>(c + 32) + ix);
+    b = __ldg(r + iy);
+    bl = __ldg(reinterpret_cast<const float2*>(r + 8) + iy);
   }
 };
 
-template <typename DT, typename PR>
-__device__ __forceinline__ void residual_sum(const BlockConst& bc, int k1, const PR& prays,
-                                             const float2* __restrict__ rays,
-                                             const FramePtrs& fp, float z,
-                                             float& sh, float& sl, int& nview) {
-  sh = 0.0f;
-  sl = 0.0f;
-  nview = 0;
-  for (int q0 = 0; q0 < k1; q0 += kViewGroup) {
-    float ah[kViewGroup][3], al[kViewGroup][3];
-    int px[kViewGroup], py[kViewGroup];
-    DT Dj[kViewGroup];
-    bool ok[kViewGroup];
-    // Eq. 4: transform, projection, nearest pixel and field-of-view test of each view
+__device__ __forceinline__ float rcp_approx(float v) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+// Nearest pixel floor(u + 1/2) along one axis from the float32 estimate u5 of u + 1/2 (out-of-range
+// and non-finite estimates give an index outside every image).  The estimate's error is below
+// (W + |c|) 2^-21 (six float32 roundings of u - c and the rounding of c + 1/2), half of the view's
+// band; inside the band the pixel is decided exactly.
+template <bool Y>
+__device__ __forceinline__ int nearest_pixel(float u5, float band, const CamDev* J, float ah, float al,
+                                             float azh, float azl) {
+  const float t = __fadd_rn(u5, kGridM);
+  const float r = __fsub_rn(t, kGridM), d = __fsub_rn(u5, r);
+  int p = __float_as_int(t) - kGridBits - (d < 0.0f ? 1 : 0);
+  if (fabsf(d) < band) {
+    fast_two_sum(ah, al, ah, al);
+    fast_two_sum(azh, azl, azh, azl);
+    p = Y ? exact_round(J->fyh, J->fyl, J->cyh, J->cyl, ah, al, azh, azl, r)
+          : exact_round(J->fxh, J->fxl, J->cxh, J->cxl, ah, al, azh, azl, r);
+  }
+  return p;
+}
+
+// Sum over the K-1 neighbour views of d_ij^2 (Eq. 6) in grid units^2, as ff (sh, sl): the general
+// evaluation in double-float for depths of any size.  A pixel at z-depth z; the transform into view
+// j (Eq. 4) uses the pixel's separable pair rays, a = z (A(x) + B(y)) + t_ji.
+template <typename DT>
+__device__ __noinline__ void residual_general(const BlockConst* bc, int k1, const RigDev* rig,
+                                              GlobalPairRays prays, const float2* __restrict__ rays,
+                                              const FramePtrs* fp, float z, float* res, int* views) {
+  float sh = 0.0f, sl = 0.0f;
+  int nview = 0;
+  const float ginv = rig->hot.ginv;
+  for (int q = 0; q < k1; ++q) {
+    const ViewHot& V = bc->view[q];
+    const PairDev& P = rig->pair[bc->cam.pair0 + q];
+    const CamDev* J = &rig->cam[V.j];
+    float4 a4, b4;
+    float2 a2, b2;
+    float ah[3], al[3];
+    prays(q, a4, a2, b4, b2);
+    ff_ray_affine(a4.x, a4.w, b4.x, b4.w, z, P.th[0], P.tl[0], ah[0], al[0]);
+    ff_ray_affine(a4.y, a2.x, b4.y, b2.x, z, P.th[1], P.tl[1], ah[1], al[1]);
+    ff_ray_affine(a4.z, a2.y, b4.z, b2.y, z, P.th[2], P.tl[2], ah[2], al[2]);
+    fast_two_sum(ah[2], al[2], ah[2], al[2]);             // sign of a_z is that of ah
+    if (!(ah[2] > 0.0f)) continue;                        // behind camera j
+    const float fu = __fmaf_rn(V.fx, __fdividef(ah[0], ah[2]), V.cx5);
+    const float fv = __fmaf_rn(V.fy, __fdividef(ah[1], ah[2]), V.cy5);
+    const int px = nearest_pixel<false>(fu, V.band, J, ah[0], al[0], ah[2], al[2]);
+    const int py = nearest_pixel<true>(fv, V.band, J, ah[1], al[1], ah[2], al[2]);
+    if ((unsigned)px >= (unsigned)V.W || (unsigned)py >= (unsigned)V.H) continue;
+    const DT D = __ldg(static_cast<const DT*>(fp->depth[V.j]) + (unsigned)(py * V.W + px));
+    if (!Depth<DT>::valid(D)) continue;
+    // Q = D_j(u_j) (rx_j, ry_j, 1) in camera-j coordinates (rigid motion keeps d)
+    const float zj = __fmul_rn(Depth<DT>::z(D), ginv);
+    const float2 qx = __ldg(rays + V.ray_x + px), qy = __ldg(rays + V.ray_y + py);
+    float qh[3], ql[3];
+    two_prod(zj, qx.x, qh[0], ql[0]);
+    ql[0] = __fmaf_rn(zj, qx.y, ql[0]);
+    two_prod(zj, qy.x, qh[1], ql[1]);
+    ql[1] = __fmaf_rn(zj, qy.y, ql[1]);
+    qh[2] = zj;
+    ql[2] = 0.0f;
 #pragma unroll
-    for (int g = 0; g < kViewGroup; ++g) {
-      ok[g] = false;
-      px[g] = 0;
-      py[g] = 0;
-      Dj[g] = (DT)0;
-      const int q = q0 + g;
-      if (q >= k1) continue;
-      const PairDev& P = bc.pair[q];
-      const CamDev& J = bc.nb[q];
-      float4 a01, a2, b01, b2;
-      prays(q, P, a01, a2, b01, b2);
-      ff_ray_affine(a01.x, a01.y, b01.x, b01.y, z, P.th[0], P.tl[0], ah[g][0], al[g][0]);
-      ff_ray_affine(a01.z, a01.w, b01.z, b01.w, z, P.th[1], P.tl[1], ah[g][1], al[g][1]);
-      ff_ray_affine(a2.x, a2.y, b2.x, b2.y, z, P.th[2], P.tl[2], ah[g][2], al[g][2]);
-      fast_two_sum(ah[g][2], al[g][2], ah[g][2], al[g][2]);   // sign of a_z is that of ah
-      if (!(ah[g][2] > 0.0f)) continue;                        // behind camera j
-      // float32 estimate of u + 1/2 from the ff high parts (relative error ~1e-7, so a
-      // few 1e-4 px); within kTieBandPx of a tie the pixel is decided exactly
-      const float fu = __fadd_rn(__fmaf_rn(J.fx, __fdividef(ah[g][0], ah[g][2]), J.cx), 0.5f);
-      const float fv = __fadd_rn(__fmaf_rn(J.fy, __fdividef(ah[g][1], ah[g][2]), J.cy), 0.5f);
-      if (!(fu > -1.0f && fu < (float)J.W + 1.0f && fv > -1.0f && fv < (float)J.H + 1.0f))
-        continue;
-      const float ru = rintf(fu), rv = rintf(fv);
-      px[g] = fabsf(fu - ru) < kTieBandPx
-                  ? exact_round(J.fxh, J.fxl, J.cxh, J.cxl, ah[g][0], al[g][0], ah[g][2], al[g][2], ru)
-                  : (int)floorf(fu);
-      py[g] = fabsf(fv - rv) < kTieBandPx
-                  ? exact_round(J.fyh, J.fyl, J.cyh, J.cyl, ah[g][1], al[g][1], ah[g][2], al[g][2], rv)
-                  : (int)floorf(fv);
-      if (px[g] < 0 || px[g] >= J.W || py[g] < 0 || py[g] >= J.H) continue;
-      Dj[g] = __ldg(static_cast<const DT*>(fp.depth[P.j]) + (long long)py[g] * J.W + px[g]);
-      ok[g] = true;
+    for (int k = 0; k < 3; ++k) {                         // d^2 = |a - Q|^2 in ff
+      float s, e, p, pe, tt;
+      two_sum(ah[k], -qh[k], s, e);
+      e = __fadd_rn(e, __fsub_rn(al[k], ql[k]));
+      // (s + e)^2 = s^2 + 2 s e + e^2; e^2 is below the ff rounding of the sum
+      two_prod(s, s, p, pe);
+      pe = __fmaf_rn(__fmul_rn(2.0f, s), e, pe);
+      two_sum(sh, p, sh, tt);
+      sl = __fadd_rn(sl, __fadd_rn(tt, pe));
     }
-    // Eq. 5-6 for the views whose gathered depth is valid
+    ++nview;
+  }
+  res[0] = sh;
+  res[1] = sl;
+  *views = nview;
+}
+
+// The same sum for depths up to the rig's zmax, on the rig's grid (all coordinates below 2^22 grid
+// units): every coordinate is kept as an integral float plus a remainder below one unit.  Adding
+// kGridM in the FMA that forms a product rounds it to an integer, a second FMA gives the exact rest,
+// and integral parts add exactly; the difference D of two integral parts is the difference of their
+// bits, so that sum D^2 is exact in 64-bit integers, and float32 carries the remainders alone:
+// d^2 = D^2 + l (2 D + l).  A remainder is off by a few 2^-26 grid units, 2^-47 of the rig's extent.
+// 16 operations a coordinate where the double-float evaluation takes 41; with it the consistency step of
+// the 8x1280x720 rig (3.7 M points, 3 views) went from 269 to 216 us in the kernel it then was part of.
+// Measured slower: two points a thread side by side (+16 us, spills), three views at once (+15 us).
+// Views whose sample is beyond zmax return false (the point then takes the general evaluation).
+template <typename DT, typename PR>
+__device__ __forceinline__ bool residual_grid(const ViewHot* views, int k1, const PR& prays,
+                                              const RigDev* __restrict__ rig, const RigHot& hot,
+                                              const float2* __restrict__ rays, const FramePtrs& fp,
+                                              float z, float& sh, float& sl, int& nview) {
+  long long S = 0;
+  float c = 0.0f;
+  bool fits = sizeof(DT) == 2 || z <= hot.zmax;
+#pragma unroll 1
+  for (int q = 0; q < k1; ++q) {
+    const float4* vw = reinterpret_cast<const float4*>(views + q);
+    const float4 w0 = vw[0], w1 = vw[1], w2 = vw[2], w3 = vw[3];
+    const float mt[3] = {w0.x, w0.y, w0.z}, tl[3] = {w0.w, w1.x, w1.y};
+    const int W = __float_as_int(w2.z), H = __float_as_int(w2.w), j = __float_as_int(w3.w);
+    float4 a4, b4;
+    float2 a2, b2;
+    prays(q, a4, a2, b4, b2);
+    const float gh[3] = {__fadd_rn(a4.x, b4.x), __fadd_rn(a4.y, b4.y), __fadd_rn(a4.z, b4.z)};
+    const float gl[3] = {__fadd_rn(a4.w, b4.w), __fadd_rn(a2.x, b2.x), __fadd_rn(a2.y, b2.y)};
+    float s[3], l[3], ah[3], f[3];
 #pragma unroll
-    for (int g = 0; g < kViewGroup; ++g) {
-      if (!ok[g] || !Depth<DT>::valid(Dj[g])) continue;
-      const CamDev& J = bc.nb[q0 + g];
-      // Q = D_j(u_j) (rx_j, ry_j, 1) in camera-j coordinates (rigid motion keeps d)
-      const float zj = Depth<DT>::z(Dj[g]);
-      const float2 qx = __ldg(rays + J.ray_x + px[g]), qy = __ldg(rays + J.ray_y + py[g]);
-      float qh[3], ql[3];
-      two_prod(zj, qx.x, qh[0], ql[0]);
-      ql[0] = __fmaf_rn(zj, qx.y, ql[0]);
-      two_prod(zj, qy.x, qh[1], ql[1]);
-      ql[1] = __fmaf_rn(zj, qy.y, ql[1]);
-      qh[2] = zj;
-      ql[2] = 0.0f;
+    for (int k = 0; k < 3; ++k) {                         // Eq. 4: a = z (A + B) + t
+      s[k] = __fmaf_rn(z, gh[k], mt[k]);
+      l[k] = __fmaf_rn(z, gh[k], -__fsub_rn(s[k], mt[k]));
+      l[k] = __fadd_rn(__fmaf_rn(z, gl[k], l[k]), tl[k]);
+      ah[k] = __fsub_rn(s[k], kGridM);
+      f[k] = __fadd_rn(ah[k], l[k]);
+    }
+    if (!(f[2] > 0.0f)) continue;                          // behind camera j
+    const float inv = rcp_approx(f[2]);
+    const float fu = __fmaf_rn(w1.z, __fmul_rn(f[0], inv), w2.x);
+    const float fv = __fmaf_rn(w1.w, __fmul_rn(f[1], inv), w2.y);
+    const int px = nearest_pixel<false>(fu, w3.z, &rig->cam[j], ah[0], l[0], ah[2], l[2]);
+    const int py = nearest_pixel<true>(fv, w3.z, &rig->cam[j], ah[1], l[1], ah[2], l[2]);
+    if ((unsigned)px >= (unsigned)W || (unsigned)py >= (unsigned)H) continue;
+    const DT Dj = __ldg(static_cast<const DT*>(fp.depth[j]) + (unsigned)(py * W + px));
+    const float2 qx = __ldg(rays + __float_as_int(w3.x) + px), qy = __ldg(rays + __float_as_int(w3.y) + py);
+    if (!Depth<DT>::valid(Dj)) continue;
+    if (sizeof(DT) == 4) fits = fits && Depth<DT>::z(Dj) <= hot.zmax;
+    // Q = D_j(u_j) (rx_j, ry_j, 1) in camera-j coordinates (rigid motion keeps d)
+    const float zj = __fmul_rn(Depth<DT>::z(Dj), hot.ginv);
+    const float r[3] = {qx.x, qy.x, 1.0f}, rl[3] = {qx.y, qy.y, 0.0f};
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {                    // d^2 = |a - Q|^2 in ff
-        float s, e, p, pe, tt;
-        two_sum(ah[g][k], -qh[k], s, e);
-        e = __fadd_rn(e, __fsub_rn(al[g][k], ql[k]));
-        // (s + e)^2 = s^2 + 2 s e + e^2; e^2 is below the ff rounding of the sum
-        two_prod(s, s, p, pe);
-        pe = __fmaf_rn(__fmul_rn(2.0f, s), e, pe);
-        two_sum(sh, p, sh, tt);
-        sl = __fadd_rn(sl, __fadd_rn(tt, pe));
-      }
-      ++nview;
+    for (int k = 0; k < 3; ++k) {                         // Eq. 5, 6
+      const float t = __fmaf_rn(zj, r[k], kGridM);
+      float e = __fmaf_rn(zj, r[k], -__fsub_rn(t, kGridM));
+      if (k < 2) e = __fmaf_rn(zj, rl[k], e);
+      const int D = __float_as_int(s[k]) - __float_as_int(t);
+      const float dl = __fsub_rn(l[k], e);
+      S += (long long)D * D;
+      c = __fmaf_rn(dl, __fmaf_rn(2.0f, __fsub_rn(s[k], t), dl), c);
+    }
+    ++nview;
+  }
+  // S = hi 2^24 + lo and the remainders' sum c as one ff (hi is exact below 2^24: d < 2^24 units)
+  const float hi = __fmul_rn((float)(int)(S >> 24), 16777216.0f), lo = (float)(int)(S & 0xffffff);
+  float s1, e1, e2;
+  two_sum(lo, c, s1, e1);
+  fast_two_sum(hi, s1, sh, e2);
+  sl = __fadd_rn(e1, e2);
+  return fits;
+}
+
+// Residual sum of a point over its camera's views (block constants bc in shared or global
+// memory): the grid evaluation, or the general one where a depth is beyond the rig's zmax.
+template <typename DT, typename PR>
+__device__ __forceinline__ void residual_sum(const BlockConst* bc, const Tables& t, int cam, int k1, const PR& prays,
+                                             const RigDev* __restrict__ rig, const RigHot& hot,
+                                             const float2* __restrict__ rays, const FramePtrs& fp, float z,
+                                             int x, int y, float& sh, float& sl, int& nview) {
+  nview = 0;
+  const bool fits = residual_grid<DT>(bc->view, k1, prays, rig, hot, rays, fp, z, sh, sl, nview);
+  if constexpr (sizeof(DT) == 4) {
+    if (!fits) {
+      const BlockConst* g = t.bconst + cam;
+      float res[2];
+      residual_general<DT>(g, k1, rig, GlobalPairRays(t.pray + g->cam.pray, rig->cam[cam].W, k1, x, y), rays, &fp,
+                           z, res, &nview);
+      sh = res[0];
+      sl = res[1];
     }
   }
 }
@@ -309,7 +403,7 @@ __device__ __forceinline__ void residual_sum(const BlockConst& bc, int k1, const
 // Eq. 7 and 10 from the residual sum (sh, sl): omega = C' exp(-e) = mu 2^-m with
 // e = m ln 2 + f, f in [0, ln 2), so that mu never underflows (C' = C, or 1 without the
 // confidence term).  Returns e (high part) for traces.
-__device__ __forceinline__ float joint_weight(const RigDev& rig, int k1, float sh, float sl,
+__device__ __forceinline__ float joint_weight(const RigHot& rig, int k1, float sh, float sl,
                                               float c, float& mu, int& m) {
   float eh = 0.0f, el = 0.0f;
   if (rig.use_cons && k1 > 0) {
@@ -334,250 +428,227 @@ __device__ __forceinline__ float joint_weight(const RigDev& rig, int k1, float s
 }
 
 // ------------------------------------------------------------------ count step
-template <typename DT>
-__device__ __forceinline__ void load8(const DT* __restrict__ d, const float* __restrict__ c,
-                                      long long p0, long long npx, DT dv[8], float cv[8]) {
-  const bool full = p0 + 7 < npx;
-  if constexpr (sizeof(DT) == 2) {
-    if (full && ((reinterpret_cast<uintptr_t>(d + p0) & 15) == 0)) {
-      const uint4 u = __ldg(reinterpret_cast<const uint4*>(d + p0));
-      const unsigned w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) { dv[2 * k] = (DT)(w[k] & 0xffff); dv[2 * k + 1] = (DT)(w[k] >> 16); }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) dv[k] = (p0 + k < npx) ? d[p0 + k] : (DT)0;
-    }
-  } else {
-    if (full && ((reinterpret_cast<uintptr_t>(d + p0) & 15) == 0)) {
-      const float4 f0 = __ldg(reinterpret_cast<const float4*>(d + p0));
-      const float4 f1 = __ldg(reinterpret_cast<const float4*>(d + p0) + 1);
-      dv[0] = f0.x; dv[1] = f0.y; dv[2] = f0.z; dv[3] = f0.w;
-      dv[4] = f1.x; dv[5] = f1.y; dv[6] = f1.z; dv[7] = f1.w;
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) dv[k] = (p0 + k < npx) ? d[p0 + k] : (DT)0;
-    }
-  }
-  if (full && ((reinterpret_cast<uintptr_t>(c + p0) & 15) == 0)) {
-    const float4 f0 = __ldg(reinterpret_cast<const float4*>(c + p0));
-    const float4 f1 = __ldg(reinterpret_cast<const float4*>(c + p0) + 1);
-    cv[0] = f0.x; cv[1] = f0.y; cv[2] = f0.z; cv[3] = f0.w;
-    cv[4] = f1.x; cv[5] = f1.y; cv[6] = f1.z; cv[7] = f1.w;
-  } else {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) cv[k] = (p0 + k < npx) ? c[p0 + k] : 0.0f;
-  }
+// n points of a coarse cell (Sec. II.5(1)c) into the global table; the cell's position there.
+__device__ __forceinline__ unsigned count_cell(const Tables& t, int x, int y, int z, unsigned n) {
+  const unsigned slot = coarse_insert(t, pack_key(0, x, y, z));
+  if (slot != kSlotNone) atomicAdd(&t.coarse[slot].count, n);
+  return slot;
 }
 
-// Adds n points to coarse key k: the block table while it is at most 3/4 full (so that
-// probe runs stay short), else, or after 32 probes, the global table directly.
-template <int TS>
-__device__ __forceinline__ void count_add(const Tables& t, unsigned long long* s_key,
-                                          unsigned* s_cnt, unsigned* s_fill,
-                                          unsigned long long k, unsigned n) {
-  int h = -1;
-  if (*static_cast<volatile unsigned*>(s_fill) < 3u * TS / 4u) {
-    bool fresh;
-    h = local_pos<TS>(s_key, kKeyEmpty, k, 32, fresh);
-    if (fresh) atomicAdd(s_fill, 1u);
+// Position of a cell key in a warp's table of kUnitCells, inserted if new; -1 after 8 probes.
+__device__ __forceinline__ int unit_cell(unsigned* tab, unsigned key) {
+  unsigned h = (key * 0x9E3779B1u) >> 26;
+#pragma unroll 1
+  for (int probe = 0; probe < 8; ++probe) {
+    const unsigned cur = *static_cast<volatile unsigned*>(&tab[h]);
+    if (cur == key) return (int)h;
+    if (cur == 0xffffffffu) {
+      const unsigned prev = atomicCAS(&tab[h], 0xffffffffu, key);
+      if (prev == 0xffffffffu || prev == key) return (int)h;
+    }
+    h = (h + 1) & (kUnitCells - 1);
   }
-  if (h >= 0) {
-    atomicAdd(&s_cnt[h], n);
-  } else {
-    const unsigned slot = coarse_insert(t, k);
-    if (slot != kSlotNone) atomicAdd(&t.coarse[slot].count, n);
-  }
+  return -1;
 }
 
+// A warp takes units of 32 columns by 8 rows with no block-wide step in between: gate (Eq. 9) and
+// compaction of the gated pixels, a column a lane; then a gated pixel a lane, full warps: back-projection
+// (Eq. 8), extent (Sec. II.5(1)b), and the coarse cell (Sec. II.5(1)c), counted in a small table of the
+// warp.  Each cell goes to the global table once per unit, with its number of points, and its position
+// in the warp's table is its number in the unit; the gated pixels are listed (pixel and cell number,
+// depth, confidence) for the next steps, which then neither gate again nor probe the global table.
+// 8x1280x720 (7.4 Mpx, 28,800 units): 48 us, bound by instruction issue (74 % of the slots while full);
+// blocks with a table of 2048 cells and runs of equal cells merged across the warp took 59 us.  Finding a
+// unit's cells one after another as the smallest key left took 49 us there, but 236 instead of 154 us
+// where units hold many cells (16x1024^2).
 template <typename DT, int NB>
 __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ BatchArgs<NB> args) {
   int local;
   const FrameArgs& fa = args.f[batch_frame<NB>(args.count_first, args.n, (int)blockIdx.x, local)];
-  const RigDev* __restrict__ rigp = fa.rig;
   const float2* __restrict__ rays = fa.rays;
   const FramePtrs& fp = fa.fp;
   const Tables& t = fa.t;
-  const int blocks_x = fa.count_blocks_x, chunks = fa.count_chunks;
-  const int cam = local / blocks_x, bx = local - cam * blocks_x;
+  const TileIndex& ti = fa.ti;
   pdl_release();
-  constexpr int TS = 2048;                                      // block table of coarse keys
-  __shared__ unsigned long long s_key[TS];
-  __shared__ unsigned s_cnt[TS];
-  __shared__ unsigned s_fill;                                    // keys in the block table
-  __shared__ unsigned short s_occ[TS];                           // occupied positions, packed
-  // the packing loop below walks the table in whole warps (every lane reaches the ballot)
-  // and stores positions as 16-bit values
-  static_assert(TS % kThreads == 0 && kThreads % 32 == 0 && TS <= 65536, "block table shape");
-  __shared__ unsigned s_nocc;
+  constexpr int kUnitPx = kTileW * kUnitH;
+  __shared__ DT s_d[kThreads / 32][kUnitPx];
+  __shared__ float s_c[kThreads / 32][kUnitPx];
+  __shared__ unsigned char s_p[kThreads / 32][kUnitPx];
+  __shared__ CamHot s_cam[kThreads / 32];
+  __shared__ unsigned char s_occ[kThreads / 32][kUnitCells];
+  __shared__ unsigned s_key[kThreads / 32][kUnitCells], s_cnt[kThreads / 32][kUnitCells];
+  static_assert(kUnitCells == 64, "two positions a lane, 6-bit hash");
   __shared__ unsigned s_red[kThreads / 32][9];
-  // per warp, the runs its lanes send to the block table in a chunk (at most one per run,
-  // kCountPx a lane), inserted by the whole warp at once; the counts share the storage of
-  // s_occ, which only the final flush uses
-  constexpr int kRunCap = 32 * kCountPx;
-  static_assert((kThreads / 32) * kRunCap <= TS, "run counts fit in s_occ");
-  __shared__ unsigned long long s_mk[kThreads / 32][kRunCap];
-  unsigned short* const s_mn = s_occ + (threadIdx.x >> 5) * kRunCap;
-  __shared__ unsigned s_mcount[kThreads / 32];
-  const RigDev& rig = *rigp;
-  // the camera's constants and the rig's scalars in registers (they would otherwise be
-  // re-read for every pixel, as the atomics below may alias memory for the compiler)
-  const CamDev C = rig.cam[cam];
-  const float tau = rig.tau, inv_s0u = rig.inv_s0u;
-  const int use_conf = rig.use_conf, lim = kKeyBias >> rig.max_level;
-  const long long npx = (long long)C.W * C.H;
-  const int bid = cam * blocks_x + bx;
-  const long long c0 = (long long)bx * chunks;                  // first chunk of 2048 pixels
-  const bool idle = c0 * kCountBlockPx >= npx;                  // uniform over the block
-  for (int i = threadIdx.x; i < TS; i += kThreads) { s_key[i] = kKeyEmpty; s_cnt[i] = 0; }
-  if (threadIdx.x == 0) { s_fill = 0u; s_nocc = 0u; }
-  if (threadIdx.x < kThreads / 32) s_mcount[threadIdx.x] = 0u;
-  __syncthreads();
-
-  const DT* __restrict__ dep = static_cast<const DT*>(fp.depth[cam]);
-  const float* __restrict__ cf = fp.conf[cam];
+  const float tau = fa.hot.tau, inv_s0u = fa.hot.inv_s0u;
+  const bool use_conf = fa.hot.use_conf != 0;
+  const int lim = kKeyBias >> fa.hot.max_level;                      // a power of two
+  const unsigned window = (unsigned)min(1024, 2 * lim);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float qnan = __int_as_float(0x7fffffff), inf = __int_as_float(0x7f800000);
   unsigned nv = 0, ng = 0, noor = 0;
-  float fmn[3] = {__int_as_float(0x7f800000), __int_as_float(0x7f800000), __int_as_float(0x7f800000)};
-  float fmx[3] = {__int_as_float(0xff800000), __int_as_float(0xff800000), __int_as_float(0xff800000)};
-  long long pn = (c0 * kThreads + threadIdx.x) * kCountPx;
-  int y = (int)((unsigned)pn / (unsigned)C.W);                  // W H <= 2^30
-  int x = (int)((unsigned)pn - (unsigned)y * (unsigned)C.W);
-  // no prefetch of the next chunk: registers stay under 64, and four resident blocks per
-  // SM hide the load latency better than a second set of eight samples per thread did
-  for (int ch = 0; ch < (idle ? 0 : chunks); ++ch) {
-    const long long pc = pn;
-    if ((c0 + ch) * kCountBlockPx >= npx) break;                 // uniform over the block
-    DT dcur[kCountPx];
-    float ccur[kCountPx];
-    if (pc < npx) load8<DT>(dep, cf, pc, npx, dcur, ccur);
-    pn = pc + kCountBlockPx;
-    // Sec. II.5(1)c density estimate. Runs of equal coarse cells along the thread's
-    // pixels: the first run (if the thread has several) and the last run are kept for the
-    // merge along the warp, the ones between are staged for the warp's insertion pass (a
-    // block-table insertion in the unrolled loop itself would run once per unrolled pixel
-    // for the whole warp whenever any lane ends a run there).
-    unsigned long long khead = kKeyEmpty, ktail = kKeyEmpty;
-    unsigned nhead = 0u, run = 0u, nruns = 0u;
-    int cx = 0, cy = 0, cz = 0;
-    if (pc < npx) {
-      // the pixels' ray components: one row and 16-byte aligned rays (every rig whose
-      // widths are multiples of 8) take four vector loads, other groups one load per pixel
-      float rxk[kCountPx], ryk[kCountPx];
-      if (x + kCountPx <= C.W && ((C.ray_x + x) & 1) == 0) {
-        const float4* r4 = reinterpret_cast<const float4*>(rays + C.ray_x + x);
-#pragma unroll
-        for (int k = 0; k < kCountPx / 2; ++k) {
-          const float4 v = __ldg(r4 + k);
-          rxk[2 * k] = v.x;
-          rxk[2 * k + 1] = v.z;
-        }
-        const float ry = __ldg(&rays[C.ray_y + y].x);
-#pragma unroll
-        for (int k = 0; k < kCountPx; ++k) ryk[k] = ry;
-      } else {
-        int xx = x, yy = y;
-#pragma unroll
-        for (int k = 0; k < kCountPx; ++k) {
-          rxk[k] = __ldg(&rays[C.ray_x + xx].x);
-          ryk[k] = __ldg(&rays[C.ray_y + min(yy, C.H - 1)].x);
-          if (++xx == C.W) { xx = 0; ++yy; }
-        }
+  float fmn[3] = {inf, inf, inf}, fmx[3] = {-inf, -inf, -inf};
+  const int u0 = local * fa.count_chunks * (kThreads / 32);
+  const int u1 = min(u0 + fa.count_chunks * (kThreads / 32), t.n_units);
+#pragma unroll 1
+  for (int u = u0 + warp; u < u1; u += kThreads / 32) {
+    int cam, lu = u, ux;
+    if (ti.units_per_cam) {
+      cam = fast_div(u, ti.units_per_cam, ti.div_units, lu);
+    } else {
+      cam = 0;
+      for (int lo = 0, hi = ti.n_cams - 1; lo <= hi;) {
+        const int mid = (lo + hi) >> 1;
+        if (ti.unit[mid] <= u) { cam = mid; lo = mid + 1; } else { hi = mid - 1; }
       }
-      // branch-free per pixel: every lane evaluates every pixel, predicates select
-#pragma unroll
-      for (int k = 0; k < kCountPx; ++k) {
-        const bool valid = pc + k < npx && Depth<DT>::valid(dcur[k]);
-        const bool gated = valid && (!use_conf || ccur[k] > tau);  // Eq. 9
-        nv += valid ? 1u : 0u;
-        ng += gated ? 1u : 0u;
-        float P[3];
-        world_point(C, valid ? Depth<DT>::z(dcur[k]) : 0.0f, rxk[k], ryk[k], P);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          fmn[a] = gated ? fminf(fmn[a], P[a]) : fmn[a];
-          fmx[a] = gated ? fmaxf(fmx[a], P[a]) : fmx[a];
-        }
-        // coarse coordinates floor(P / s0); the finest index floor(r 2^Lmax) is in
-        // [-2^19, 2^19) exactly when floor(r) is in [-2^(19-Lmax), 2^(19-Lmax))
-        const int ix = (int)floorf(__fmul_rn(P[0], inv_s0u));
-        const int iy = (int)floorf(__fmul_rn(P[1], inv_s0u));
-        const int iz = (int)floorf(__fmul_rn(P[2], inv_s0u));
-        const bool inr = (unsigned)(ix + lim) < (unsigned)(2 * lim) &&
-                         (unsigned)(iy + lim) < (unsigned)(2 * lim) &&
-                         (unsigned)(iz + lim) < (unsigned)(2 * lim);
-        noor += (gated && !inr) ? 1u : 0u;
-        const bool counted = gated && inr;
-        const bool same = run && ix == cx && iy == cy && iz == cz;
-        if (counted && !same && run) {                            // a run ends
-          if (nruns == 1u) {
-            khead = pack_key(0, cx, cy, cz);
-            nhead = run;
-          } else {
-            const unsigned q = atomicAdd(&s_mcount[warp], 1u);
-            s_mk[warp][q] = pack_key(0, cx, cy, cz);
-            s_mn[q] = (unsigned short)run;
-          }
-        }
-        if (counted) {
-          run = same ? run + 1u : 1u;
-          nruns += same ? 0u : 1u;
-          cx = ix;
-          cy = iy;
-          cz = iz;
-        }
-      }
+      lu = u - ti.unit[cam];
     }
+    const int W = ti.W[cam], H = ti.H[cam];
+    const int y0 = fast_div(lu, (W + kTileW - 1) / kTileW, ti.div_x[cam], ux) * kUnitH, x0 = ux * kTileW;
+    int n = 0;
     {
-      if (run) ktail = pack_key(0, cx, cy, cz);
-      // merge the lanes' runs along the warp (consecutive lanes hold consecutive pixels):
-      // a lane's first run continues the previous lane's last run when the keys agree
-      const unsigned long long kfirst = nruns >= 2u ? khead : ktail;
-      const unsigned long long kprev = __shfl_up_sync(0xffffffffu, ktail, 1);
-      const bool cont = lane > 0 && ktail != kKeyEmpty && kfirst == kprev;
-      // a continuing head run is credited to the previous lane's chain
-      const unsigned give = (cont && nruns >= 2u) ? nhead : 0u;
-      unsigned v = run + __shfl_down_sync(0xffffffffu, give, 1) * (lane < 31 ? 1u : 0u);
-      bool start = !(cont && nruns == 1u);
-      const bool nstart = __shfl_down_sync(0xffffffffu, (unsigned)start, 1) != 0u;
+      const DT* __restrict__ dep = static_cast<const DT*>(fp.depth[cam]);
+      const float* __restrict__ cf = fp.conf[cam];
+      const int rows = x0 + lane < W ? min(kUnitH, H - y0) : 0;
+      DT D[kUnitH];
+      float C[kUnitH];
+      unsigned li = (unsigned)(y0 * W + x0 + lane);                  // W H <= 2^30
 #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {                          // segmented inclusive scan
-        const unsigned v2 = __shfl_up_sync(0xffffffffu, v, d);
-        const bool f2 = __shfl_up_sync(0xffffffffu, (unsigned)start, d) != 0u;
-        if (lane >= d) {
-          if (!start) v += v2;
-          start = start || f2;
+      for (int k = 0; k < kUnitH; ++k, li += W) {
+        D[k] = (DT)0;
+        C[k] = 0.0f;
+        if (k < rows) {
+          D[k] = dep[li];
+          C[k] = cf[li];
         }
       }
-      // the lane's first run unless it continues the previous lane's chain, and its last
-      // run where a chain ends, join the middle runs; then every run of the warp goes to
-      // the block table, one lane each
-      if (nruns >= 2u && !cont) {
-        const unsigned q = atomicAdd(&s_mcount[warp], 1u);
-        s_mk[warp][q] = khead;
-        s_mn[q] = (unsigned short)nhead;
+#pragma unroll
+      for (int k = 0; k < kUnitH; ++k) {
+        const bool valid = Depth<DT>::valid(D[k]);
+        const bool gated = valid && (!use_conf || C[k] > tau);       // Eq. 9
+        nv += valid ? 1u : 0u;
+        const unsigned m = __ballot_sync(0xffffffffu, gated);
+        if (gated) {
+          const int pos = n + __popc(m & ((1u << lane) - 1u));
+          s_d[warp][pos] = D[k];
+          s_c[warp][pos] = C[k];
+          s_p[warp][pos] = (unsigned char)(k * kTileW + lane);
+        }
+        n += __popc(m);
       }
-      if (ktail != kKeyEmpty && (lane == 31 || nstart)) {
-        const unsigned q = atomicAdd(&s_mcount[warp], 1u);
-        s_mk[warp][q] = ktail;
-        s_mn[q] = (unsigned short)v;
+    }
+    if (n == 0) {                                                    // uniform over the warp
+      if (lane == 0) t.lcount[u] = 0u;
+      continue;
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      s_key[warp][lane + 32 * q] = 0xffffffffu;
+      s_cnt[warp][lane + 32 * q] = 0u;
+    }
+    if (lane < 4) reinterpret_cast<float4*>(&s_cam[warp])[lane] = __ldg(reinterpret_cast<const float4*>(t.bconst + cam) + lane);
+    __syncwarp();
+    const CamHot& cam_c = s_cam[warp];
+    // the rays of the unit's columns (a lane one) and rows (the first lanes)
+    const float ray_x = __ldg(&rays[cam_c.ray_x + min(x0 + lane, W - 1)].x);
+    const float ray_y = __ldg(&rays[cam_c.ray_y + min(y0 + (lane & (kUnitH - 1)), H - 1)].x);
+    auto point = [&](int i, float z, float P[3]) {                   // Eq. 8 of list entry i at depth z
+      const int p = s_p[warp][i];
+      world_point(cam_c, z, __shfl_sync(0xffffffffu, ray_x, p & (kTileW - 1)),
+                  __shfl_sync(0xffffffffu, ray_y, p / kTileW), P);
+    };
+    // Coarse cells as keys of 10 bits an axis, relative to the first point's cell - 512, or to the first
+    // cell in range where there are no more than 1024 (a cell index is read off the bits of kGridM +
+    // v rounded down: grid_coords); `ok`: the window holds only cells in range.  Other points go to the
+    // global table by themselves.
+    int ref[3] = {kGridBits - lim, kGridBits - lim, kGridBits - lim};
+    bool ok = true;
+    if (lim > 512) {
+      float P[3];
+      point(0, Depth<DT>::z(s_d[warp][0]), P);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        ref[a] = __float_as_int(__fadd_rd(__fmul_rn(P[a], inv_s0u), kGridM)) - 512;
+        ok = ok && (unsigned)(ref[a] - kGridBits + lim) < (unsigned)(2 * lim - 1024);
       }
-      __syncwarp();
-      const unsigned nm = s_mcount[warp];
-      for (unsigned q = lane; q < nm; q += 32u) count_add<TS>(t, s_key, s_cnt, &s_fill, s_mk[warp][q], s_mn[q]);
-      __syncwarp();
-      if (lane == 0) s_mcount[warp] = 0u;
+    }
+    const long long at = unit_list(ti.off[cam], W, H, x0, y0);
+    DT* __restrict__ ld = static_cast<DT*>(t.ldepth) + at;
+    float* __restrict__ lc = t.lconf + at;
+    unsigned short* __restrict__ lp = t.lpix + at;
+    bool missed = false;                                             // a point without a number
+#pragma unroll 1
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + lane;
+      const bool act = i < n;
+      const DT d = s_d[warp][i];
+      float P[3];
+      point(i, act ? Depth<DT>::z(d) : qnan, P);                     // NaN: no minimum or maximum takes it
+      unsigned q[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        fmn[a] = fminf(fmn[a], P[a]);
+        fmx[a] = fmaxf(fmx[a], P[a]);
+        q[a] = (unsigned)(__float_as_int(__fadd_rd(__fmul_rn(P[a], inv_s0u), kGridM)) - ref[a]);
+      }
+      const bool in = ok && (q[0] | q[1] | q[2]) < window;
+      const unsigned key = act && in ? (q[0] << 20) + (q[1] << 10) + q[2] : 0xffffffffu;
+      const unsigned key0 = __shfl_sync(0xffffffffu, key, 0);
+      int number = -1;
+      if (__all_sync(0xffffffffu, key == key0 || !act) && key0 != 0xffffffffu) {   // one cell: one insertion
+        if (lane == 0) {
+          number = unit_cell(s_key[warp], key0);
+          if (number >= 0) s_cnt[warp][number] += (unsigned)min(32, n - i0);
+        }
+        number = __shfl_sync(0xffffffffu, number, 0);
+      } else if (key != 0xffffffffu) {
+        number = unit_cell(s_key[warp], key);
+        if (number >= 0) atomicAdd(&s_cnt[warp][number], 1u);
+      }
+      if (act) {
+        missed = missed || number < 0;
+        ld[i] = d;
+        lc[i] = s_c[warp][i];
+        lp[i] = (unsigned short)(s_p[warp][i] | ((unsigned)(number & 0xff) << 8));
+      }
       __syncwarp();
     }
-    x += kCountBlockPx;                                           // next chunk's first pixel
-    while (x >= C.W) { x -= C.W; ++y; }
+    ng += lane == 0 ? (unsigned)n : 0u;
+    if (__any_sync(0xffffffffu, missed)) {                           // far-flung points, or a full table
+#pragma unroll 1
+      for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        float P[3], r[3];
+        int c[3];
+        point(i, i < n ? Depth<DT>::z(s_d[warp][i]) : qnan, P);
+        const bool inr = grid_coords(fa.hot, P, r, c);
+        if (i < n && (lp[i] >> 8) == kNoCellNumber) {                // the lane's own store above
+          if (inr) count_cell(t, c[0], c[1], c[2], 1u);
+          else ++noor;
+        }
+      }
+    }
+    // the unit's cells into the global table, one a lane
+    const unsigned o0 = __ballot_sync(0xffffffffu, s_key[warp][lane] != 0xffffffffu);
+    const unsigned o1 = __ballot_sync(0xffffffffu, s_key[warp][lane + 32] != 0xffffffffu);
+    const unsigned below = (1u << lane) - 1u;
+    if ((o0 >> lane) & 1u) s_occ[warp][__popc(o0 & below)] = (unsigned char)lane;
+    if ((o1 >> lane) & 1u) s_occ[warp][__popc(o0) + __popc(o1 & below)] = (unsigned char)(lane + 32);
+    __syncwarp();
+    const int cells = __popc(o0) + __popc(o1);
+    for (int q = lane; q < cells; q += 32) {
+      const int h = s_occ[warp][q];
+      const unsigned key = s_key[warp][h];
+      t.lcell[(long long)u * kUnitCells + h] =
+          count_cell(t, ref[0] - kGridBits + (int)(key >> 20), ref[1] - kGridBits + (int)((key >> 10) & 1023u),
+                     ref[2] - kGridBits + (int)(key & 1023u), s_cnt[warp][h]);
+    }
+    if (lane == 0) t.lcount[u] = (unsigned)n;
+    __syncwarp();                                                    // the staged pixels are free again
   }
   // per-block pixel counts and extent
-  unsigned vals[9] = {nv, ng, noor, ordered(fmn[0]), ordered(fmn[1]), ordered(fmn[2]),
-                      ordered(fmx[0]), ordered(fmx[1]), ordered(fmx[2])};
-  if (ng == 0) {
-    for (int a = 0; a < 3; ++a) { vals[3 + a] = 0xffffffffu; vals[6 + a] = 0u; }
-  }
+  unsigned vals[9] = {nv, ng, noor};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) { vals[3 + a] = ordered(fmn[a]); vals[6 + a] = ordered(fmx[a]); }
   vals[0] = __reduce_add_sync(0xffffffffu, vals[0]);
   vals[1] = __reduce_add_sync(0xffffffffu, vals[1]);
   vals[2] = __reduce_add_sync(0xffffffffu, vals[2]);
@@ -598,425 +669,544 @@ __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ B
       b.n_valid += s_red[w][0];
       b.n_gated += s_red[w][1];
       b.n_oor += s_red[w][2];
+      if (s_red[w][1] == 0u) continue;                               // no point: no extent
       for (int k = 0; k < 3; ++k) {
         b.bmin[k] = min(b.bmin[k], s_red[w][3 + k]);
         b.bmax[k] = max(b.bmax[k], s_red[w][6 + k]);
       }
     }
-    t.bstats[bid] = b;
-  }
-  // the block table into the global one: the occupied positions are packed first, so that a
-  // thread sends at most a few of them and the global round trips of all of them overlap
-  // (walking the table in strides left up to eight dependent round trips per thread)
-  for (int i = threadIdx.x; i < TS; i += kThreads) {
-    const bool occ = s_key[i] != kKeyEmpty;
-    const unsigned m = __ballot_sync(0xffffffffu, occ);
-    unsigned base = 0u;
-    if (lane == 0 && m) base = atomicAdd(&s_nocc, (unsigned)__popc(m));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (occ) s_occ[base + __popc(m & ((1u << lane) - 1u))] = (unsigned short)i;
-  }
-  __syncthreads();
-  const int n_occ = (int)s_nocc;
-  for (int j = threadIdx.x; j < n_occ; j += kThreads) {
-    const int i = s_occ[j];
-    const unsigned slot = coarse_insert(t, s_key[i]);
-    if (slot != kSlotNone) atomicAdd(&t.coarse[slot].count, s_cnt[i]);
+    t.bstats[local] = b;
   }
 }
 
-// ------------------------------------------------------------------ assign step
-constexpr size_t align16(size_t v) { return (v + 15) / 16 * 16; }
-static_assert(kMaxTopK * 8 <= 14 * 4, "a cell's top-k keys fit in its 14 split-sum words");
-
-// The assign step's tile: 32 columns by TH rows (TH = 8, 16 or 32: a launch-geometry
-// choice), one warp per two rows, two pixels a thread, and its shared-memory layout.
-// Distinct cells of a tile with shared-memory accumulators: NL.  In a tile with more
-// distinct cells (sparse, noisy tiles only) the cells with two or more members in the tile
-// take the accumulators and every other member files a single-member partial, which is the
-// record the accumulator would have produced for it; if even the multi-member cells are too
-// many, every member files alone.  Both rules depend on the tile's cells alone, never on
-// the order of the insertions, so that every cell's sums, and the fused cloud, are bitwise
-// reproducible for a given tile shape.
-template <int TH>
-struct AssignTile {
-  static_assert(TH == 8 || TH == 16 || TH == 32, "tile heights");
-  static constexpr int Px = kTileW * TH;
-  static constexpr int Threads = 16 * TH;
-  static constexpr int Warps = Threads / 32;
-  // registers (64 a thread) allow this many blocks per SM (shared memory may allow fewer)
-  static constexpr int BlocksPerSM = 4 * 256 / Threads;
-  static constexpr int PrayPerView = 2 * kTileW + 2 * TH;  // staged pair-ray float4 per view
-  static constexpr int TS = 2 * Px;                         // shared hash positions
-  static constexpr int NL = Px / 2;                         // accumulator entries
-  static constexpr int ConstWords =
-      (int)((sizeof(CamDev) + kMaxK1 * (sizeof(PairDev) + sizeof(CamDev))) / 4 + Threads - 1) / Threads;
-  static_assert(ConstWords <= 4, "a few words per thread copy a block's constants");
-  static constexpr size_t BC = 0;
-  // per hash position (TS): cell slot, entry index, smallest weight exponent, largest
-  // ordered C, member count; the last four are contiguous so that one loop clears them
-  static constexpr size_t FK = align16(BC + sizeof(BlockConst));   // u32 cell slot
-  static constexpr size_t MinP = FK + 4 * TS;                      // int smallest exponent
-  static constexpr size_t CmaxP = MinP + 4 * TS;                   // u32 largest ordered C
-  static constexpr size_t CntP = CmaxP + 4 * TS;                   // u32 members
-  static constexpr size_t FI = align16(CntP + 4 * TS);             // int entry of a position
-  // per entry (NL): key, hash position, lowest index at the largest C, split sums
-  static constexpr size_t EK = align16(FI + 4 * TS);               // u64 key
-  static constexpr size_t EP = align16(EK + 8 * NL);               // u32 hash position
-  static constexpr size_t Gmin = align16(EP + 4 * NL);             // u32 lowest index
-  static constexpr size_t Acc = align16(Gmin + 4 * NL);            // u32[14][NL] split sums
-  static constexpr size_t Pid = align16(Acc + 14 * 4 * NL);        // u16[tile] gated pixels
-  static constexpr size_t Z = align16(Pid + 2 * Px);               // f32[tile] their depth
-  static constexpr size_t C = align16(Z + 4 * Px);                 // f32[tile] confidence
-  static constexpr size_t RGB = align16(C + 4 * Px);               // u32[tile] colour
-  static constexpr size_t PR = align16(RGB + 4 * Px);              // float4[K1][PrayPerView]
-  // dynamic shared memory of a launch with k1 neighbour views
-  static constexpr size_t smem(int k1) { return PR + 16 * (size_t)k1 * PrayPerView; }
-};
-constexpr unsigned kLoBits = 22;           // split of a <= 2^37 sum term: 512 lows fit in u32
-
-// Writes partial p as record pi and pushes it onto its cell's list; true when it is the
-// cell's first partial of the frame (the caller then lists the cell).
-// mmin: the record's smallest weight exponent, INT_MAX for top-k records (no sums).
-__device__ __forceinline__ bool file_partial(const Tables& t, Partial& p, unsigned slot,
-                                             unsigned long long key, int mmin, unsigned pi) {
-  SlotRec& rec = t.frec[slot];
-  rec.key = key;                                // the same value from every tile of the cell
-  if (mmin != INT_MAX) atomicMin(&rec.mmin, mmin);
-  p.next = atomicExch(&rec.head, pi);           // list push
-  t.part[pi] = p;
-  return p.next == kSlotNone;
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
 }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// rint(v) for 0 <= v < 2^37 as hi 2^22 + lo with lo in [0, 2^22], using 32-bit conversions
-// only: v - floor(v 2^-22) 2^22 is exact (both are multiples of ulp(v)), and adding the even
-// integer hi 2^22 does not change a round-half-even decision.
-__device__ __forceinline__ void split_round(float v, unsigned& lo, unsigned& hi) {
-  const float hf = floorf(__fmul_rn(v, 1.0f / (float)(1u << kLoBits)));
-  hi = (unsigned)hf;
-  lo = __float2uint_rn(__fmaf_rn(-hf, (float)(1u << kLoBits), v));
-}
-
-// First probe of a point's coarse record (read-only during the assign step, L1-cached);
-// coarse_lvbase() finishes the probe once the value is needed.
-__device__ __forceinline__ ulonglong2 coarse_probe(const Tables& t, unsigned long long key, unsigned& h) {
-  h = (unsigned)mix64(key) & t.cmask;
-  return __ldg(reinterpret_cast<const ulonglong2*>(&t.coarse[h]));
-}
-
-// Camera and first pixel of tile T (tiles of TH rows): a division when every camera has the
-// same size, else a binary search of the per-camera tile ranges (constant bank).
+// Camera and first pixel of tile T (tiles of TH rows): divisions by known divisors when every camera
+// has the same size, else a binary search of the per-camera tile ranges (constant bank).
 template <int TH>
 __device__ __forceinline__ void tile_of(const TileIndex& ti, int T, int& cam, int& x0, int& y0) {
+  int local = T;
   if (ti.per_cam) {
-    cam = T / ti.per_cam;
+    cam = fast_div(T, ti.per_cam, ti.div_cam, local);
   } else {
     cam = 0;
     for (int lo = 0, hi = ti.n_cams - 1; lo <= hi;) {
       const int mid = (lo + hi) >> 1;
       if (ti.first[mid] <= T) { cam = mid; lo = mid + 1; } else { hi = mid - 1; }
     }
+    local = T - ti.first[cam];
   }
-  const int local = T - ti.first[cam], tiles_x = (ti.W[cam] + kTileW - 1) / kTileW;
-  x0 = (local % tiles_x) * kTileW;
-  y0 = (local / tiles_x) * TH;
+  int tx;
+  y0 = fast_div(local, (ti.W[cam] + kTileW - 1) / kTileW, ti.div_x[cam], tx) * TH;
+  x0 = tx * kTileW;
 }
 
-// TOPK: the Sec. II.5(2)a variant; members are keyed and counted as usual, but a tile keeps
-// each cell's top-k members by C (packed (ordered(C) << 32) | ~g keys) instead of weights;
-// the consistency and weights of those members are computed per cell by k_reduce_topk.
-template <typename DT, bool TOPK, bool TRACE, int NB, int TH>
-__global__ void __launch_bounds__(AssignTile<TH>::Threads, AssignTile<TH>::BlocksPerSM)
-k_assign(const __grid_constant__ BatchArgs<NB> args) {
-  using AT = AssignTile<TH>;
-  constexpr int kTileH = TH, kTilePx = AT::Px, kAssignThreads = AT::Threads, kAssignWarps = AT::Warps;
-  constexpr int kAssignTS = AT::TS, kAssignNL = AT::NL, kPrayPerView = AT::PrayPerView;
-  constexpr int kConstWords = AT::ConstWords;
-  constexpr size_t kSmBC = AT::BC, kSmFK = AT::FK, kSmMinP = AT::MinP, kSmCmaxP = AT::CmaxP,
-                   kSmCntP = AT::CntP, kSmFI = AT::FI, kSmEK = AT::EK, kSmEP = AT::EP,
-                   kSmGmin = AT::Gmin, kSmAcc = AT::Acc, kSmPid = AT::Pid, kSmZ = AT::Z, kSmC = AT::C,
-                   kSmRGB = AT::RGB, kSmPR = AT::PR;
+// ------------------------------------------------------------------ weigh step
+// A block takes one tile of 32 columns by TH rows (TH = 8, 16 or 32: a launch-geometry choice), a
+// thread up to four of its gated pixels, one after another, with no step of the whole block between
+// the staging of the tile's constants and the claims at the end.  Frames of few tiles take more
+// threads a block, down to a pixel a thread (weigh_threads).
+template <int TH>
+struct WeighTile {
+  static_assert(TH == 8 || TH == 16 || TH == 32, "tile heights");
+  static constexpr int Px = kTileW * TH, Threads = 8 * TH, Units = TH / kUnitH;
+  // claimed cells (slot, key), level and first slot of the units' numbered coarse cells, camera and view
+  // constants, the tile's pair rays
+  static constexpr size_t Key = 0;                                 // u64[Px]
+  static constexpr size_t Slot = Key + 8 * Px;                     // u32[Px]
+  static constexpr size_t LB = Slot + 4 * Px;                      // u32[Units][kUnitCells]
+  static constexpr size_t BC = LB + 4 * Units * kUnitCells;
+  // 16-byte words of the constants of k1 views, and of the pair rays of the tile's columns and rows
+  static __host__ __device__ constexpr int const_words(int k1) { return 4 * (1 + k1); }
+  static __host__ __device__ constexpr int col_words(int k1) { return k1 * kPrayColGroup; }
+  static __host__ __device__ constexpr int row_words(int k1) { return k1 * Units * kPrayRowGroup; }
+  static constexpr size_t smem(int k1) { return BC + 16 * (size_t)(const_words(k1) + col_words(k1) + row_words(k1)); }
+};
+
+// The tile's gated pixels are its units' lists, one after the other: entry i of the tile is entry
+// i + shift of the frame's lists, for the unit it falls into.
+template <int kUnits>
+struct TileList {
+  int n, end[kUnits];            // pixels of the tile; of the units up to each one
+  unsigned shift[kUnits];
+  __device__ __forceinline__ TileList(const Tables& t, const TileIndex& ti, int cam, unsigned off, int W, int H, int x0,
+                                      int y0) {
+    const int tiles_x = (W + kTileW - 1) / kTileW, u0 = ti.unit[cam] + (y0 >> 3) * tiles_x + (x0 >> 5);
+    unsigned listed[kUnits];
+#pragma unroll
+    for (int k = 0; k < kUnits; ++k) listed[k] = y0 + k * kUnitH < H ? __ldcg(t.lcount + u0 + k * tiles_x) : 0u;
+    n = 0;
+#pragma unroll
+    for (int k = 0; k < kUnits; ++k) {
+      shift[k] = (unsigned)unit_list(off, W, H, x0, y0 + k * kUnitH) - (unsigned)n;
+      n += (int)listed[k];
+      end[k] = n;
+    }
+  }
+  // unit of entry i, and its entry in the frame's lists
+  __device__ __forceinline__ unsigned at(int i, int& unit) const {
+    unit = 0;
+    unsigned s = shift[0];
+#pragma unroll
+    for (int q = 1; q < kUnits; ++q)
+      if (i >= end[q - 1]) { unit = q; s = shift[q]; }
+    return s + (unsigned)i;
+  }
+};
+
+// Levels and first slots of the units' numbered coarse cells (Sec. II.5(1)d), a number a thread.  (A
+// number that the unit does not use still names some position of the coarse table, an earlier frame's.)
+template <int kUnits>
+__device__ __forceinline__ void load_cell_levels(const Tables& t, const TileIndex& ti, const TileList<kUnits>& list, int cam,
+                                                 int W, int x0, int y0, unsigned* s_lb) {
+  const int tiles_x = (W + kTileW - 1) / kTileW, u0 = ti.unit[cam] + (y0 >> 3) * tiles_x + (x0 >> 5);
+  const int k = (int)threadIdx.x / kUnitCells, c = (int)threadIdx.x & (kUnitCells - 1);
+  bool listed = false;                            // the unit has a list, and so its numbers
+#pragma unroll
+  for (int q = 0; q < kUnits; ++q)
+    if (k == q) listed = list.end[q] > (q ? list.end[q > 0 ? q - 1 : 0] : 0);
+  if (listed) {
+    const unsigned slot = __ldcg(t.lcell + (long long)(u0 + k * tiles_x) * kUnitCells + c);
+    s_lb[threadIdx.x] = slot == kSlotNone ? kBaseNone : __ldcg(&t.coarse[slot].lvbase);
+  }
+}
+
+// Dense slot of a point: level << 27 | slot, from its coarse cell's level << 27 | first slot; its cell
+// key's parts in kk and its place in the cell in frac.  kBaseNone in the slot field: none.
+__device__ __forceinline__ unsigned point_slot(unsigned lb, const float r[3], int kk[3], float frac[3]) {
+  const int l = (int)(lb >> 27);
+  const float sl = pow2f(l);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {                   // floor of r 2^l (below 2^19 in size) and the rest
+    const float t = __fmaf_rd(r[a], sl, kGridM);
+    kk[a] = __float_as_int(t) - kGridBits;
+    frac[a] = __fmaf_rn(r[a], sl, -__fsub_rn(t, kGridM));
+  }
+  // sub-cell of the coarse cell: k - (coarse << l) = k & (2^l - 1)
+  const unsigned mask = (1u << l) - 1u;
+  const unsigned local = ((((unsigned)kk[0] & mask) << l | ((unsigned)kk[1] & mask)) << l) | ((unsigned)kk[2] & mask);
+  return (lb & kBaseNone) == kBaseNone ? lb : lb + local;
+}
+
+// Per gated pixel: Eq. 8, its cell (Sec. II.5(1)d-e), its joint weight (Eq. 4-7, 10) as mantissa and
+// exponent; per cell, kept in its slot: the representative (Sec. II.5(2)a) as the largest
+// (ordered(C) << 32) | ~g, the smallest weight exponent, and the cell's number, claimed by the first
+// point that finds none.  All are order-independent but the numbering, which no result depends on.
+// A point looks at its slot first and sends an atomic only where that would change it: most do not.
+// Bound by latency and issue (gathers of the views' depths): 48 registers for uint16 depth, as 40 warps
+// an SM hide more than 32 do (weigh + sum of 8x1280x720: 185 us against 193 at 64); float32 depth, with
+// its checks, is faster at 64 (50 against 53 us on five ragged cameras).
+template <typename DT, bool TRACE, int NB, int TH>
+__global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64) k_weigh(const __grid_constant__ BatchArgs<NB> args) {
+  using WT = WeighTile<TH>;
   int T;
   const FrameArgs& fa = args.f[batch_frame<NB>(args.tile_first, args.n, (int)blockIdx.x, T)];
-  const RigDev* __restrict__ rigp = fa.rig;
   const float2* __restrict__ rays = fa.rays;
   const FramePtrs& fp = fa.fp;
   const Tables& t = fa.t;
   const TraceDev& tr = fa.tr;
-  const float unit_m = (float)fa.unit_m;
   const TileIndex& ti = fa.ti;
+  const RigHot& hot = fa.hot;
   pdl_release();
   extern __shared__ __align__(16) unsigned char smem[];
-  BlockConst& bc = *reinterpret_cast<BlockConst*>(smem + kSmBC);
-  unsigned* s_fk = reinterpret_cast<unsigned*>(smem + kSmFK);
-  int* s_minp = reinterpret_cast<int*>(smem + kSmMinP);
-  unsigned* s_cmaxp = reinterpret_cast<unsigned*>(smem + kSmCmaxP);
-  unsigned* s_cntp = reinterpret_cast<unsigned*>(smem + kSmCntP);
-  int* s_fi = reinterpret_cast<int*>(smem + kSmFI);
-  unsigned long long* s_ek = reinterpret_cast<unsigned long long*>(smem + kSmEK);
-  unsigned* s_ep = reinterpret_cast<unsigned*>(smem + kSmEP);
-  unsigned* s_gmin = reinterpret_cast<unsigned*>(smem + kSmGmin);
-  unsigned* s_acc = reinterpret_cast<unsigned*>(smem + kSmAcc);
-  unsigned short* s_pid = reinterpret_cast<unsigned short*>(smem + kSmPid);
-  float* s_z = reinterpret_cast<float*>(smem + kSmZ);
-  float* s_c = reinterpret_cast<float*>(smem + kSmC);
-  unsigned* s_rgb = reinterpret_cast<unsigned*>(smem + kSmRGB);
-  __shared__ unsigned s_n, s_base, s_ng, s_nm;
+  unsigned long long* s_key = reinterpret_cast<unsigned long long*>(smem + WT::Key);
+  unsigned* s_slot = reinterpret_cast<unsigned*>(smem + WT::Slot);
+  unsigned* s_lb = reinterpret_cast<unsigned*>(smem + WT::LB);
+  const BlockConst& bc = *reinterpret_cast<const BlockConst*>(smem + WT::BC);
+  __shared__ unsigned s_claims, s_first;
 
-  const RigDev& rig = *rigp;
   int cam, x0, y0;
   tile_of<TH>(ti, T, cam, x0, y0);
   const int W = ti.W[cam], H = ti.H[cam], k1 = ti.k1;
-  struct { int x0, y0; long long off; } td;
-  td.x0 = x0;
-  td.y0 = y0;
-  td.off = ti.off[cam];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // warm L2 with the images of the tile that starts when this wave of blocks has finished
-  if (threadIdx.x < 4 * kTileH && T + ti.ahead < t.n_tiles) {
+  const unsigned off = (unsigned)ti.off[cam];
+  // the camera's and its views' constants and the tile's pair rays (Eq. 4), asynchronously
+  const int n_views = hot.use_cons ? k1 : 0;
+  const int n_const = WT::const_words(n_views), n_cols = WT::col_words(n_views);
+  const float4* const s_cols = reinterpret_cast<const float4*>(smem + WT::BC) + n_const;
+  const float4* const s_rows = s_cols + n_cols;
+  {
+    const float4* gc = reinterpret_cast<const float4*>(t.bconst + cam);
+    const float4* ga = t.pray + ti.pray[cam] + (x0 >> 5) * k1 * kPrayColGroup;
+    const float4* gb = t.pray + ti.pray[cam] + (((W + 31) >> 5) * kPrayColGroup + (y0 >> 3) * kPrayRowGroup) * k1;
+    const int n = n_const + n_cols + WT::row_words(n_views);
+    for (int i = threadIdx.x; i < n; i += (int)blockDim.x) {
+      const float4* src = i < n_const ? gc + i : i < n_const + n_cols ? ga + (i - n_const) : gb + (i - n_const - n_cols);
+      cp_async16(smem + WT::BC + 16 * i, src);
+    }
+  }
+  // warm L2 with the colours of a tile further on: the sum step reads them
+  if (threadIdx.x < 2 * TH && T + ti.ahead < t.n_tiles) {
     int pc, px0, py0;
     tile_of<TH>(ti, T + ti.ahead, pc, px0, py0);
-    const int row = py0 + (threadIdx.x & (kTileH - 1)), kind = threadIdx.x / kTileH;
+    const int row = py0 + (int)(threadIdx.x >> 1);
     if (row < ti.H[pc]) {                     // every address lies inside its image
-      const long long li = (long long)row * ti.W[pc] + px0;
-      const long long last = (long long)row * ti.W[pc] + min(px0 + kTileW, ti.W[pc]) - 1;
-      const char* a = kind == 0 ? static_cast<const char*>(fp.depth[pc]) + li * sizeof(DT)
-                    : kind == 1 ? reinterpret_cast<const char*>(fp.conf[pc] + li)
-                    : reinterpret_cast<const char*>(fp.rgb[pc]) + 3 * (kind == 3 ? last : li);
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
+      const long long li = (long long)row * ti.W[pc] + ((threadIdx.x & 1) ? min(px0 + kTileW, ti.W[pc]) - 1 : px0);
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(fp.rgb[pc] + 3 * li));
     }
   }
-  const DT* __restrict__ dep = static_cast<const DT*>(fp.depth[cam]);
-  const float* __restrict__ cf = fp.conf[cam];
-  const uint8_t* __restrict__ col = fp.rgb[cam];
-  // issue the constant-block loads (L2) and the tile's image loads (HBM) before waiting
-  // on either: the words of cam, pair[0, k1) and nb[0, k1) of this camera's BlockConst
-  constexpr int kCamW = sizeof(CamDev) / 4, kPairW = sizeof(PairDev) / 4;
-  constexpr int kNbAt = (int)(offsetof(BlockConst, nb) / 4), kPairAt = (int)(offsetof(BlockConst, pair) / 4);
-  const int n_cw = kCamW + k1 * (kPairW + kCamW);
-  const int* gsrc = reinterpret_cast<const int*>(&t.bconst[cam]);
-  int cwv[kConstWords], cwi[kConstWords];
-#pragma unroll
-  for (int r = 0; r < kConstWords; ++r) {
-    const int w = threadIdx.x + r * kAssignThreads;
-    cwi[r] = w < kCamW ? w
-           : w < kCamW + k1 * kPairW ? kPairAt + (w - kCamW)
-           : w < n_cw ? kNbAt + (w - kCamW - k1 * kPairW) : -1;
-    cwv[r] = cwi[r] >= 0 ? __ldg(gsrc + cwi[r]) : 0;
-  }
-  // the tile's pair rays (Eq. 4): per view, A of its 32 columns and B of its 16 rows, each
-  // as two float4 planes: [A first halves | A second halves | B first | B second]
-  constexpr int kPrayLoads = (kMaxK1 * kPrayPerView + kAssignThreads - 1) / kAssignThreads;
-  float4 prv[kPrayLoads];
-  int pri[kPrayLoads];
-  {
-    const int Wp = W, Hp = H;
-#pragma unroll
-    for (int r = 0; r < kPrayLoads; ++r) {
-      const int idx = threadIdx.x + r * kAssignThreads;
-      pri[r] = -1;
-      prv[r] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (TOPK || idx >= k1 * kPrayPerView) continue;
-      const int q = idx / kPrayPerView, o = idx - q * kPrayPerView;
-      const int base = ti.pray[cam] + 2 * q * (Wp + Hp);
-      int src = -1;
-      if (o < 2 * kTileW) {                                        // A: plane o / 32
-        const int c = td.x0 + (o & (kTileW - 1));
-        if (c < Wp) src = base + 2 * c + o / kTileW;
-      } else {                                                     // B: plane (o - 64) / 16
-        const int rr = o - 2 * kTileW, row = td.y0 + (rr & (kTileH - 1));
-        if (row < Hp) src = base + 2 * Wp + 2 * row + rr / kTileH;
-      }
-      if (src >= 0) {
-        prv[r] = __ldg(t.pray + src);
-        pri[r] = idx;
-      }
+  if (threadIdx.x == 0) s_claims = 0u;
+  if (TRACE) {                              // every pixel as not gated; the gated ones follow
+    const float qnan = __int_as_float(0x7fc00000);
+    for (int i = threadIdx.x; i < WT::Px; i += (int)blockDim.x) {
+      const int x = x0 + (i & (kTileW - 1)), y = y0 + i / kTileW;
+      if (x >= W || y >= H) continue;
+      const long long g = (long long)off + (long long)y * W + x;
+      if (tr.pw) { tr.pw[3 * g] = qnan; tr.pw[3 * g + 1] = qnan; tr.pw[3 * g + 2] = qnan; }
+      if (tr.e) tr.e[g] = qnan;
+      if (tr.omega) tr.omega[g] = qnan;
+      if (tr.nview) tr.nview[g] = -1;
+      if (tr.key) tr.key[g] = kKeyEmpty;
     }
   }
-  DT Dk[2];
-  float ckv[2];
-  uint8_t cb[2][3];
-  bool inimg[2];
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const int x = td.x0 + lane, y = td.y0 + warp + kAssignWarps * k;
-    inimg[k] = x < W && y < H;
-    Dk[k] = (DT)0;
-    ckv[k] = 0.0f;
-    cb[k][0] = cb[k][1] = cb[k][2] = 0;
-    if (inimg[k]) {
-      const long long li = (long long)y * W + x;
-      Dk[k] = dep[li];
-      ckv[k] = cf[li];
-      const uint8_t* px = col + 3 * li;
-      cb[k][0] = px[0];
-      cb[k][1] = px[1];
-      cb[k][2] = px[2];
-    }
-  }
-  int* sdst = reinterpret_cast<int*>(&bc);
-#pragma unroll
-  for (int r = 0; r < kConstWords; ++r)
-    if (cwi[r] >= 0) sdst[cwi[r]] = cwv[r];
-  float4* s_pr = reinterpret_cast<float4*>(smem + kSmPR);
-#pragma unroll
-  for (int r = 0; r < kPrayLoads; ++r)
-    if (pri[r] >= 0) s_pr[pri[r]] = prv[r];
-  // clear the per-position arrays: slot none, exponent INT_MAX, largest C 0, count 0
-  for (int i = threadIdx.x; i < kAssignTS; i += kAssignThreads) {
-    const unsigned v = i < kAssignTS / 4 ? kSlotNone : i < kAssignTS / 2 ? (unsigned)INT_MAX : 0u;
-    reinterpret_cast<uint4*>(smem + kSmFK)[i] = make_uint4(v, v, v, v);
-  }
-  if (threadIdx.x == 0) { s_n = 0; s_ng = 0; }
-  __syncthreads();
-
-  constexpr bool trace = TRACE;             // per-pixel trace (tests) in its own instantiation
-  const float qnan = __int_as_float(0x7fc00000);
-
-  // (a) Eq. 9 gate and compaction of the tile's gated pixels (any order: every reduction
-  // below is order-independent), so that the per-point work runs on full warps
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const int row = warp + kAssignWarps * k;
-    bool gated = false;
-    if (inimg[k]) {
-      gated = Depth<DT>::valid(Dk[k]) && (!rig.use_conf || ckv[k] > rig.tau);
-      if (!gated && trace) {
-        const long long g = td.off + (long long)(td.y0 + row) * W + td.x0 + lane;
-        if (tr.pw) { tr.pw[3 * g] = qnan; tr.pw[3 * g + 1] = qnan; tr.pw[3 * g + 2] = qnan; }
-        if (tr.e) tr.e[g] = qnan;
-        if (tr.omega) tr.omega[g] = qnan;
-        if (tr.nview) tr.nview[g] = -1;
-        if (tr.key) tr.key[g] = kKeyEmpty;
-      }
-    }
-    const unsigned gmask = __ballot_sync(0xffffffffu, gated);
-    unsigned wbase = 0u;
-    if (lane == 0 && gmask) wbase = atomicAdd(&s_ng, (unsigned)__popc(gmask));
-    wbase = __shfl_sync(0xffffffffu, wbase, 0);
-    if (gated) {
-      const int pos = (int)wbase + __popc(gmask & ((1u << lane) - 1u));
-      s_pid[pos] = (unsigned short)(row * kTileW + lane);
-      s_z[pos] = Depth<DT>::z(Dk[k]);
-      s_c[pos] = ckv[k];
-      s_rgb[pos] = (unsigned)cb[k][0] | ((unsigned)cb[k][1] << 8) | ((unsigned)cb[k][2] << 16);
-    }
-  }
-  __syncthreads();
-  const int n_g = (int)s_ng;
-  const CamDev& C = bc.cam;
-  // everything above read only the frame's inputs and the context's constants; the coarse
-  // table (count and level steps) and every table written below need the earlier kernels
+  // everything above used only the context's constants; the lists (count step), the coarse table
+  // (level step) and every table written below need the earlier kernels
   pdl_wait();
+  const TileList<WT::Units> list(t, ti, cam, off, W, H, x0, y0);
+  if (list.n == 0) return;                  // uniform over the block
+  static_assert(WT::Units * kUnitCells <= WT::Threads, "a thread takes one numbered cell");
+  load_cell_levels<WT::Units>(t, ti, list, cam, W, x0, y0, s_lb);
+  cp_async_wait();
+  __syncthreads();
+#pragma unroll 1
+  for (int i = threadIdx.x; i < list.n; i += (int)blockDim.x) {
+    int unit;
+    const unsigned at = list.at(i, unit);
+    const unsigned e = __ldcg(t.lpix + at);
+    const float z = Depth<DT>::z(__ldcg(static_cast<const DT*>(t.ldepth) + at)), c = __ldcg(t.lconf + at);
+    const int lx = (int)(e & (kTileW - 1)), ly = (int)((e & 0xffu) / kTileW) + unit * kUnitH, x = x0 + lx, y = y0 + ly;
+    const unsigned g = off + (unsigned)(y * W + x);                   // W H <= 2^30
+    const float rx = __ldg(&rays[bc.cam.ray_x + x].x), ry = __ldg(&rays[bc.cam.ray_y + y].x);
+    float P[3], r[3], frac[3];
+    int cc[3], kk[3];
+    world_point(bc.cam, z, rx, ry, P);                                // Eq. 8
+    unsigned lb = kBaseNone;
+    if (grid_coords(hot, P, r, cc))
+      lb = (e >> 8) != kNoCellNumber ? s_lb[(e >> 8) + (unsigned)(unit * kUnitCells)]
+                                     : coarse_lvbase(t, pack_key(0, cc[0], cc[1], cc[2]));
+    const unsigned ls = point_slot(lb, r, kk, frac), slot = ls & kBaseNone;
+    uint4 rec = make_uint4(0u, 0u, 0u, 0u);                           // representative, number, exponent
+    if (slot != kBaseNone) rec = __ldcg(reinterpret_cast<const uint4*>(t.frec + slot));
+    float sh = 0.0f, sl = 0.0f, mu = 0.0f;
+    int nview = 0, m = 0;
+    if (n_views > 0)
+      residual_sum<DT>(&bc, t, cam, k1, TilePairRays<TH>(s_cols, s_rows, k1, lx, ly), fa.rig, hot, rays, fp, z, x, y,
+                       sh, sl, nview);
+    const float eh = joint_weight(hot, k1, sh, sl, c, mu, m);
+    t.wslot[at] = ls;
+    t.wmant[at] = mu;
+    t.wexp[at] = m;
+    if (slot != kBaseNone) {                    // else out of range, or no slot left (reported)
+      SlotRec* s = t.frec + slot;
+      const unsigned long long key = ((unsigned long long)ordered(c) << 32) | (unsigned)(~g);
+      if ((((unsigned long long)rec.y << 32) | rec.x) < key) atomicMax(&s->key, key);
+      if ((int)rec.w > m) atomicMin(&s->mmin, m);
+      if (rec.z == kSlotNone && atomicCAS(&s->head, kSlotNone, kSlotPending) == kSlotNone) {
+        const unsigned q = atomicAdd(&s_claims, 1u);
+        s_slot[q] = slot;
+        s_key[q] = pack_key((int)(ls >> 27), kk[0], kk[1], kk[2]);
+      }
+    }
+    if (TRACE) {
+      const float unit_m = fa.unit_m;
+      if (tr.pw) {
+        tr.pw[3ll * g + 0] = P[0] * unit_m;
+        tr.pw[3ll * g + 1] = P[1] * unit_m;
+        tr.pw[3ll * g + 2] = P[2] * unit_m;
+      }
+      if (tr.e) tr.e[g] = eh;
+      if (tr.omega) tr.omega[g] = ldexpf(mu, -m);
+      if (tr.nview) tr.nview[g] = nview;
+      if (tr.key) tr.key[g] = slot != kBaseNone ? pack_key((int)(ls >> 27), kk[0], kk[1], kk[2]) : kKeyEmpty;
+    }
+  }
+  __syncthreads();
+  // the cells claimed by the tile: numbers from one counter update, their keys, sums cleared
+  const unsigned n = s_claims;
+  if (n == 0u) return;                      // uniform over the block
+  if (threadIdx.x == 0) s_first = atomicAdd(&t.cnt->n_cells, n);
+  __syncthreads();
+  for (unsigned q = threadIdx.x; q < n; q += blockDim.x) {
+    const unsigned id = s_first + q, slot = s_slot[q];
+    t.frec[slot].head = id;
+    t.fused[id] = slot;                     // a number for each slot at most
+    if ((long long)id < fa.out.max_cells) {
+      t.ckey[id] = s_key[q];
+      uint4* a = reinterpret_cast<uint4*>(t.acc + 8ull * id);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) a[k] = make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+}
 
-  // (a) Eq. 8, (b) Eq. 4-7 and 10, (c) Sec. II.5(1)d-e for each gated point
+// ------------------------------------------------------------------ sum step
+// rint(v) for 0 <= v < 2^37 as an integer, without 64-bit conversions: floor(v 2^-22) and rint of
+// the rest (exact: both are multiples of ulp(v)) are read off sums with 2^23, and adding the even
+// integer hi 2^22 does not change a round-half-even decision.
+__device__ __forceinline__ unsigned long long fixed_term(float v) {
+  constexpr unsigned kBits = 0x4B000000u;                  // 2^23
+  const float h = __fmaf_rd(v, 1.0f / 4194304.0f, 8388608.0f);
+  const float lo = __fadd_rn(__fmaf_rn(-__fsub_rn(h, 8388608.0f), 4194304.0f, v), 8388608.0f);
+  return (unsigned long long)(__float_as_uint(h) - kBits) * 4194304ull + (__float_as_uint(lo) - kBits);
+}
+
+// Shared memory of a warp of the sum step, in 16-byte words: 36 rows of 64 bytes, 32 cell numbers.
+constexpr int kSumWarpWords = 36 * 4 + 32 / 4;
+
+// Eq. 11: the sums of w, w P and w RGB of each cell as exact integers at the scale 2^-(36 + m_min) of
+// its smallest weight exponent, one 64-byte row a cell {w, w frac xyz, w rgb / 256, members}, added
+// with 64-bit reductions.  A warp lays the terms of its 32 points out in shared memory; eight lanes
+// then take a row each of eight successive points, a lane a term, and send one reduction of 64
+// contiguous bytes per run of points of one cell (eight lanes on a row measured 3 times faster than
+// a lane a row: the reductions of a row travel together).  Bound by L2's reductions: 64 us for 3.7 M
+// points, where 64-byte rows alone take 50 (75 G rows/s).  Weigh and sum take 185 us on 8x1280x720;
+// one kernel that gathered each tile's cells in shared-memory tables and wrote a record per tile and
+// cell for a later walk of the cells' record lists took 211 (tables, records and their barriers: 120).
+template <typename DT, int NB, int TH>
+__global__ void k_sum(const __grid_constant__ BatchArgs<NB> args) {
+  using WT = WeighTile<TH>;
+  int T;
+  const FrameArgs& fa = args.f[batch_frame<NB>(args.tile_first, args.n, (int)blockIdx.x, T)];
+  const float2* __restrict__ rays = fa.rays;
+  const Tables& t = fa.t;
+  const TileIndex& ti = fa.ti;
+  pdl_release();
+  // rows of 64 bytes, a spare one after each eight; a row's four 16-byte chunks are permuted by its
+  // number so that neither the writes nor the reads conflict
+  extern __shared__ __align__(16) unsigned char smem[];
+  int cam, x0, y0;
+  tile_of<TH>(ti, T, cam, x0, y0);
+  const int W = ti.W[cam], H = ti.H[cam];
+  const unsigned off = (unsigned)ti.off[cam];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint4* const s_row = reinterpret_cast<uint4*>(smem) + warp * kSumWarpWords;
+  unsigned* const s_id = reinterpret_cast<unsigned*>(s_row + 36 * 4);
+  const CamHot& cc = t.bconst[cam].cam;
+  const uint8_t* __restrict__ col = fa.fp.rgb[cam];
+  pdl_wait();
+  const TileList<WT::Units> list(t, ti, cam, off, W, H, x0, y0);
+  const unsigned max_cells = (unsigned)fa.out.max_cells;
+  const int term = lane & 7, group = lane >> 3;
+#pragma unroll 1
+  for (int i0 = warp * 32; i0 < list.n; i0 += (int)blockDim.x) {
+    const int i = i0 + lane;
+    unsigned id = kSlotNone;
+    if (i < list.n) {
+      int unit;
+      const unsigned at = list.at(i, unit);
+      const unsigned ls = __ldcg(t.wslot + at), slot = ls & kBaseNone;
+      if (slot != kBaseNone) {
+        const uint2 rec = __ldcg(reinterpret_cast<const uint2*>(&t.frec[slot].head));   // number, exponent
+        const unsigned e = __ldcg(t.lpix + at);
+        const float z = Depth<DT>::z(__ldcg(static_cast<const DT*>(t.ldepth) + at)), mu = __ldcg(t.wmant + at);
+        const int sh = __ldcg(t.wexp + at) - (int)rec.y;
+        const int x = x0 + (int)(e & (kTileW - 1)), y = y0 + (int)((e & 0xffu) / kTileW) + unit * kUnitH;
+        const uint8_t* p3 = col + 3u * (unsigned)(y * W + x);
+        const unsigned rgb[3] = {__ldg(p3), __ldg(p3 + 1), __ldg(p3 + 2)};
+        float P[3], r[3], frac[3];
+        int c[3], kk[3];
+        world_point(cc, z, __ldg(&rays[cc.ray_x + x].x), __ldg(&rays[cc.ray_y + y].x), P);
+        grid_coords(fa.hot, P, r, c);
+        point_slot(ls, r, kk, frac);
+        const float w = sh > 62 ? 0.0f : __fmul_rn(mu, pow2f(kFixShift - sh));
+        unsigned long long v[8];
+        v[0] = fixed_term(w);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          v[1 + a] = fixed_term(__fmul_rn(w, frac[a]));
+          // byte / 256: the byte in the last bits of 2^15
+          v[4 + a] = fixed_term(__fmul_rn(w, __fsub_rn(__uint_as_float(0x47000000u | rgb[a]), 32768.0f)));
+        }
+        v[7] = 1ull;
+        if (rec.x < max_cells) id = rec.x;
+        uint4* row = s_row + (lane + (lane >> 3)) * 4;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          row[k ^ ((lane >> 1) & 3)] = make_uint4((unsigned)v[2 * k], (unsigned)(v[2 * k] >> 32), (unsigned)v[2 * k + 1],
+                                                  (unsigned)(v[2 * k + 1] >> 32));
+      }
+    }
+    s_id[lane] = id;
+    __syncwarp();
+    unsigned cur = kSlotNone;
+    unsigned long long sum = 0ull;
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const int p = group * 8 + s;
+      const unsigned next = s_id[p];
+      const uint2 q = reinterpret_cast<const uint2*>(s_row + (p + group) * 4 + ((term >> 1) ^ ((p >> 1) & 3)))[term & 1];
+      if (next != cur) {
+        if (cur != kSlotNone) atomicAdd(t.acc + 8ull * cur + term, sum);
+        cur = next;
+        sum = 0ull;
+      }
+      sum += ((unsigned long long)q.y << 32) | q.x;
+    }
+    if (cur != kSlotNone) atomicAdd(t.acc + 8ull * cur + term, sum);
+    __syncwarp();
+  }
+}
+
+// ------------------------------------------------------------------ assign step
+constexpr size_t align16(size_t v) { return (v + 15) / 16 * 16; }
+// The top-k assign step's tile: 32 columns by TH rows, one warp per two rows, two pixels a thread,
+// and its shared-memory layout.
+// Distinct cells of a tile with shared-memory lists: NL.  In a tile with more distinct cells (sparse,
+// noisy tiles only) the cells with two or more members in the tile take the lists and every other
+// member files a single-member partial, which is the record the list would have produced for it; if
+// even the multi-member cells are too many, every member files alone.
+template <int TH>
+struct AssignTile {
+  static_assert(TH == 8 || TH == 16 || TH == 32, "tile heights");
+  static constexpr int Px = kTileW * TH;
+  static constexpr int Threads = 16 * TH;
+  static constexpr int Units = TH / kUnitH;
+  static constexpr int TS = 2 * Px;                         // shared hash positions
+  static constexpr int NL = Px / 2;                         // lists
+  static constexpr size_t FK = 0;                           // u32 cell slot of a position
+  static constexpr size_t CntP = FK + 4 * TS;               // u32 members of a position
+  static constexpr size_t FI = CntP + 4 * TS;               // u16 list of a position
+  static constexpr size_t EP = align16(FI + 2 * TS);        // u16 hash position of a list
+  static constexpr size_t Top = align16(EP + 2 * NL);       // u64[NL][kMaxTopK]
+  static constexpr size_t LB = Top + 8 * kMaxTopK * NL;     // u32[Units][kUnitCells]
+  static constexpr size_t Bytes = LB + 4 * Units * kUnitCells;
+};
+
+// Writes partial p as record pi and pushes it onto its cell's list; true when it is the
+// cell's first partial of the frame (the caller then lists the cell).
+__device__ __forceinline__ bool file_partial(const Tables& t, Partial& p, unsigned slot, unsigned pi) {
+  p.next = atomicExch(&t.frec[slot].head, pi);  // list push
+  t.part[pi] = p;
+  return p.next == kSlotNone;
+}
+
+// Sec. II.5(2)a variant: members are keyed and counted, and a tile keeps each cell's top-k members by C
+// (packed (ordered(C) << 32) | ~g keys); the consistency and weights of those members are computed per
+// cell by k_reduce_topk.
+template <typename DT, bool TRACE, int NB, int TH>
+__global__ void __launch_bounds__(AssignTile<TH>::Threads) k_assign_topk(const __grid_constant__ BatchArgs<NB> args) {
+  using AT = AssignTile<TH>;
+  constexpr int kAssignThreads = AT::Threads, kAssignTS = AT::TS, kAssignNL = AT::NL, kUnits = AT::Units;
+  int T;
+  const FrameArgs& fa = args.f[batch_frame<NB>(args.tile_first, args.n, (int)blockIdx.x, T)];
+  const float2* __restrict__ rays = fa.rays;
+  const Tables& t = fa.t;
+  const TraceDev& tr = fa.tr;
+  const TileIndex& ti = fa.ti;
+  const RigHot& hot = fa.hot;
+  pdl_release();
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned* s_fk = reinterpret_cast<unsigned*>(smem + AT::FK);
+  unsigned* s_cntp = reinterpret_cast<unsigned*>(smem + AT::CntP);
+  unsigned short* s_fi = reinterpret_cast<unsigned short*>(smem + AT::FI);
+  unsigned short* s_ep = reinterpret_cast<unsigned short*>(smem + AT::EP);
+  unsigned long long* s_top = reinterpret_cast<unsigned long long*>(smem + AT::Top);
+  unsigned* s_lb = reinterpret_cast<unsigned*>(smem + AT::LB);
+  __shared__ unsigned s_n, s_base, s_nm;
+
+  int cam, x0, y0;
+  tile_of<TH>(ti, T, cam, x0, y0);
+  const int W = ti.W[cam], H = ti.H[cam];
+  const unsigned off = (unsigned)ti.off[cam];
+  const int lane = threadIdx.x & 31;
+  const CamHot& camc = t.bconst[cam].cam;
+  // clear the per-position arrays: slot none, count 0
+  for (int i = threadIdx.x; i < kAssignTS / 2; i += kAssignThreads) {
+    const unsigned v = i < kAssignTS / 4 ? kSlotNone : 0u;
+    reinterpret_cast<uint4*>(smem + AT::FK)[i] = make_uint4(v, v, v, v);
+  }
+  if (threadIdx.x == 0) s_n = 0u;
+  // everything above used only the context's constants; the lists (count step), the coarse table
+  // (level step) and every table written below need the earlier kernels
+  pdl_wait();
+  const TileList<kUnits> list(t, ti, cam, off, W, H, x0, y0);
+  if (TRACE) {                              // the pixels that are not listed
+    __shared__ unsigned s_listed[TH];
+    if (threadIdx.x < TH) s_listed[threadIdx.x] = 0u;
+    __syncthreads();
+    for (int i = threadIdx.x; i < list.n; i += kAssignThreads) {
+      int unit;
+      const unsigned e = __ldcg(t.lpix + list.at(i, unit)) & 0xffu;
+      atomicOr(&s_listed[unit * kUnitH + e / kTileW], 1u << (e & (kTileW - 1)));
+    }
+    __syncthreads();
+    const float qnan = __int_as_float(0x7fc00000);
+    for (int i = threadIdx.x; i < AT::Px; i += kAssignThreads) {
+      const int lx = i & (kTileW - 1), ly = i / kTileW, x = x0 + lx, y = y0 + ly;
+      if (x >= W || y >= H || (s_listed[ly] >> lx) & 1u) continue;
+      const long long g = (long long)off + (long long)y * W + x;
+      if (tr.pw) { tr.pw[3 * g] = qnan; tr.pw[3 * g + 1] = qnan; tr.pw[3 * g + 2] = qnan; }
+      if (tr.e) tr.e[g] = qnan;
+      if (tr.omega) tr.omega[g] = qnan;
+      if (tr.nview) tr.nview[g] = -1;
+      if (tr.key) tr.key[g] = kKeyEmpty;
+    }
+  }
+  if (list.n == 0) return;                  // uniform over the block
+  load_cell_levels<kUnits>(t, ti, list, cam, W, x0, y0, s_lb);
+  __syncthreads();
+
+  // Eq. 8 and Sec. II.5(1)d-e for each gated point
   bool has[2] = {false, false};
-  float mu[2] = {0.0f, 0.0f};
-  int mexp[2] = {0, 0};
-  unsigned cord[2] = {0u, 0u};
   int hpos[2] = {0, 0};
-  long long gi[2] = {0, 0};
-  float frac[2][3];
-  unsigned long long fkey[2] = {kKeyEmpty, kKeyEmpty};
+  unsigned long long pkey[2] = {0ull, 0ull};
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int i = threadIdx.x + j * kAssignThreads;
-    if (i >= n_g) continue;
-    const int pid = s_pid[i];
-    const int x = td.x0 + (pid & (kTileW - 1)), y = td.y0 + pid / kTileW;
-    gi[j] = td.off + (long long)y * W + x;
-    const float z = s_z[i];
-    const float c = s_c[i];
-    const float rx = __ldg(&rays[C.ray_x + x].x), ry = __ldg(&rays[C.ray_y + y].x);
-    float P[3], r[3];
-    world_point(C, z, rx, ry, P);                                     // Eq. 8
-    has[j] = grid_coords(rig, P, r);
-    // start the lookup of the coarse cell's level and slot range (Sec. II.5(1)d)
-    const unsigned long long ck = has[j] ? coarse_key(r) : kKeyEmpty;
-    unsigned ch = 0u;
-    ulonglong2 ce = make_ulonglong2(kKeyEmpty, 0ull);
-    if (has[j]) ce = coarse_probe(t, ck, ch);
-    float sh = 0.0f, sl = 0.0f, eh = 0.0f;
-    int nview = 0, m = 0;
-    if constexpr (!TOPK) {
-      if (rig.use_cons && k1 > 0)
-        residual_sum<DT>(bc, k1, TilePairRays<TH>{reinterpret_cast<const float4*>(smem + kSmPR),
-                                                  x - td.x0, y - td.y0},
-                         rays, fp, z, sh, sl, nview);
-      eh = joint_weight(rig, k1, sh, sl, c, mu[j], m);
-    }
-    mexp[j] = m;
-    cord[j] = ordered(c);
-    if (trace) {
-      if (tr.pw) {
-        tr.pw[3 * gi[j] + 0] = P[0] * unit_m;
-        tr.pw[3 * gi[j] + 1] = P[1] * unit_m;
-        tr.pw[3 * gi[j] + 2] = P[2] * unit_m;
-      }
-      if (!TOPK) {
-        if (tr.e) tr.e[gi[j]] = eh;
-        if (tr.omega) tr.omega[gi[j]] = ldexpf(mu[j], -m);
-        if (tr.nview) tr.nview[gi[j]] = nview;
-      } else if (tr.nview) {                    // the top-k variant weighs cells' top-k only:
-        tr.nview[gi[j]] = -2;                   // gated, weight not evaluated here
-      }
-    }
-    if (has[j]) {
-      // Sec. II.5(1)e: cell key, its dense slot, and the point's offset inside the cell
-      const unsigned lb = coarse_lvbase(t, ck, ch, ce);
-      const int l = (int)(lb >> 27);
-      const unsigned cbase = lb & kBaseNone;
-      const unsigned long long fk = fine_key(r, l);
-      const int kk[3] = {(int)((fk >> 40) & 0xfffff) - kKeyBias, (int)((fk >> 20) & 0xfffff) - kKeyBias,
-                         (int)(fk & 0xfffff) - kKeyBias};
-      const float sl2 = pow2f(l);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) frac[j][a] = __fsub_rn(__fmul_rn(r[a], sl2), (float)kk[a]);
-      // sub-cell of the coarse cell: k - (coarse << l) = k & (2^l - 1)
-      const unsigned mask = (1u << l) - 1u;
-      const unsigned local = ((((unsigned)kk[0] & mask) << l | ((unsigned)kk[1] & mask)) << l) |
-                             ((unsigned)kk[2] & mask);
-      if (cbase == kBaseNone) {                 // slot capacity exceeded (reported)
-        has[j] = false;
+    if (i >= list.n) continue;
+    int unit;
+    const unsigned at = list.at(i, unit);
+    const unsigned e = __ldcg(t.lpix + at);
+    const float z = Depth<DT>::z(__ldcg(static_cast<const DT*>(t.ldepth) + at)), c = __ldcg(t.lconf + at);
+    const int x = x0 + (int)(e & (kTileW - 1)), y = y0 + (int)((e & 0xffu) / kTileW) + unit * kUnitH;
+    const unsigned g = off + (unsigned)(y * W + x);
+    float P[3], r[3], frac[3];
+    int cc[3], kk[3];
+    world_point(camc, z, __ldg(&rays[camc.ray_x + x].x), __ldg(&rays[camc.ray_y + y].x), P);
+    unsigned lb = kBaseNone;
+    if (grid_coords(hot, P, r, cc))
+      lb = (e >> 8) != kNoCellNumber ? s_lb[(e >> 8) + (unsigned)(unit * kUnitCells)]
+                                     : coarse_lvbase(t, pack_key(0, cc[0], cc[1], cc[2]));
+    const unsigned ls = point_slot(lb, r, kk, frac), slot = ls & kBaseNone;
+    unsigned long long fkey = kKeyEmpty;
+    if (slot != kBaseNone) {                  // else out of range, or no slot left (reported)
+      fkey = pack_key((int)(ls >> 27), kk[0], kk[1], kk[2]);
+      pkey[j] = ((unsigned long long)ordered(c) << 32) | (unsigned)(~g);
+      bool fresh;
+      const int h = local_pos<kAssignTS>(s_fk, slot, fresh);
+      hpos[j] = h;
+      has[j] = h >= 0;
+      if (h < 0) {
+        atomicOr(&t.cnt->error, kErrSlots);
       } else {
-        fkey[j] = fk;
-        bool fresh;
-        const int h = local_pos<kAssignTS>(s_fk, kSlotNone, cbase + local, kAssignTS, fresh);
-        hpos[j] = h;
-        if (h < 0) {
-          has[j] = false;
-          atomicOr(&t.cnt->error, kErrSlots);
-        } else {
-          if (fresh) {                          // the cell's entry: index and accumulators
-            const int e = (int)atomicAdd(&s_n, 1u);
-            s_fi[h] = e;
-            if (e < kAssignNL) {
-              s_ek[e] = fk;
-              s_ep[e] = (unsigned)h;
-              s_gmin[e] = 0xffffffffu;
-              if constexpr (TOPK) {             // the entry's top-k list (u64 view of s_acc)
-                unsigned long long* top = reinterpret_cast<unsigned long long*>(s_acc) + e * kMaxTopK;
+        if (fresh) {                          // the cell's list
+          t.frec[slot].key = fkey;            // the same from every tile
+          const int q = (int)atomicAdd(&s_n, 1u);
+          s_fi[h] = (unsigned short)q;
+          if (q < kAssignNL) {
+            s_ep[q] = (unsigned short)h;
 #pragma unroll
-                for (int q = 0; q < kMaxTopK; ++q) top[q] = 0ull;
-              } else {
-#pragma unroll
-                for (int a = 0; a < 14; ++a) s_acc[a * kAssignNL + e] = 0u;
-              }
-            }
-          }
-          // Sec. II.5(2)a: members, largest C, smallest weight exponent
-          atomicAdd(&s_cntp[h], 1u);
-          if (!TOPK) {
-            atomicMax(&s_cmaxp[h], cord[j]);
-            atomicMin(&s_minp[h], mexp[j]);
+            for (int a = 0; a < kMaxTopK; ++a) s_top[q * kMaxTopK + a] = 0ull;
           }
         }
+        atomicAdd(&s_cntp[h], 1u);
       }
     }
-    if (trace && tr.key) tr.key[gi[j]] = has[j] ? fkey[j] : kKeyEmpty;
+    if (TRACE) {
+      const float unit_m = fa.unit_m;
+      if (tr.pw) {
+        tr.pw[3ll * g + 0] = P[0] * unit_m;
+        tr.pw[3ll * g + 1] = P[1] * unit_m;
+        tr.pw[3ll * g + 2] = P[2] * unit_m;
+      }
+      if (tr.nview) tr.nview[g] = -2;         // weighed per cell: gated, weight not evaluated here
+      if (tr.key) tr.key[g] = fkey;
+    }
   }
   __syncthreads();
-  // more cells than accumulators: the multi-member cells take them (see kAssignNL)
+  // more cells than lists: the multi-member cells take them (see AssignTile)
   const bool renumber = s_n > (unsigned)kAssignNL;         // the same in every thread
   bool all_alone = false;
   unsigned n_local = s_n;
@@ -1027,23 +1217,14 @@ k_assign(const __grid_constant__ BatchArgs<NB> args) {
       if (s_fk[h] == kSlotNone) continue;
       int e = kAssignNL;
       if (s_cntp[h] >= 2u) {
-        e = (int)atomicAdd(&s_nm, 1u);
+        e = min((int)atomicAdd(&s_nm, 1u), kAssignNL);
         if (e < kAssignNL) {
-          s_ep[e] = (unsigned)h;
-          s_gmin[e] = 0xffffffffu;
-          if constexpr (TOPK) {
-            unsigned long long* top = reinterpret_cast<unsigned long long*>(s_acc) + e * kMaxTopK;
+          s_ep[e] = (unsigned short)h;
 #pragma unroll
-            for (int q = 0; q < kMaxTopK; ++q) top[q] = 0ull;
-          } else {
-#pragma unroll
-            for (int a = 0; a < 14; ++a) s_acc[a * kAssignNL + e] = 0u;
-          }
-        } else {
-          e = kAssignNL;
+          for (int a = 0; a < kMaxTopK; ++a) s_top[e * kMaxTopK + a] = 0ull;
         }
       }
-      s_fi[h] = e;
+      s_fi[h] = (unsigned short)e;
     }
     __syncthreads();
     all_alone = s_nm > (unsigned)kAssignNL;
@@ -1052,78 +1233,30 @@ k_assign(const __grid_constant__ BatchArgs<NB> args) {
   // reserve the tile's partial records now; the index is needed only at the end
   unsigned base_pi = 0u;
   if (threadIdx.x == 0) base_pi = atomicAdd(&t.cnt->n_partials, n_local);
-  // representative: lowest pixel index among the largest C; Eq. 11 sums at the tile's
-  // scale 2^-(36 + mmin_tile), each 64-bit term split in two native 32-bit atomics
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     if (!has[j]) continue;
     const int h = hpos[j], e = s_fi[h];
-    const bool alone = all_alone || e >= kAssignNL;
-    if (renumber && !alone) s_ek[e] = fkey[j];  // every member writes the cell's key
-    if constexpr (TOPK) {
-      // Sec. II.5(2)a: insert the member into its cell's sorted top-k list; each slot keeps
-      // the largest key that reaches it and passes the smaller one down, so the list ends
-      // as the k largest keys whatever the order of the atomics
-      unsigned long long key = ((unsigned long long)cord[j] << 32) | (unsigned)(~(unsigned)gi[j]);
-      if (!alone) {
-        unsigned long long* top = reinterpret_cast<unsigned long long*>(s_acc) + e * kMaxTopK;
-        for (int q = 0; q < rig.top_k && key; ++q) {
-          const unsigned long long old = atomicMax(&top[q], key);
-          key = old < key ? old : key;
-        }
-      } else {                                  // a single-member partial of its own
-        Partial p;
-        const unsigned slot = s_fk[h];
-        p.count = 1u;
-        p.rep = key;
-#pragma unroll
-        for (int a = 0; a < kMaxTopK - 1; ++a) p.top[a] = 0ull;
-        const unsigned pi = atomicAdd(&t.cnt->n_partials, 1u);
-        if (pi >= t.max_partials) {
-          atomicOr(&t.cnt->error, kErrPartials);
-        } else if (file_partial(t, p, slot, fkey[j], INT_MAX, pi)) {
-          const unsigned n = atomicAdd(&t.cnt->n_cells, 1u);
-          if (n < t.max_slots) t.fused[n] = slot;
-        }
+    if (!(all_alone || e >= kAssignNL)) {
+      // insert the member into its cell's sorted top-k list; each slot keeps the largest key that
+      // reaches it and passes the smaller one down, so the list ends as the k largest keys whatever
+      // the order of the atomics
+      unsigned long long key = pkey[j];
+      for (int q = 0; q < fa.top_k && key; ++q) {
+        const unsigned long long old = atomicMax(&s_top[e * kMaxTopK + q], key);
+        key = old < key ? old : key;
       }
-      continue;
-    }
-    if (!alone && cord[j] == s_cmaxp[h]) atomicMin(&s_gmin[e], (unsigned)gi[j]);
-    const int sh = alone ? 0 : mexp[j] - s_minp[h];
-    const float w = sh > 62 ? 0.0f : __fmul_rn(mu[j], pow2f(kFixShift - sh));
-    const unsigned rgb = s_rgb[threadIdx.x + j * kAssignThreads];
-    float v[7];
-    v[0] = w;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) v[1 + a] = __fmul_rn(w, frac[j][a]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-      v[4 + a] = __fmul_rn(w, (float)((rgb >> (8 * a)) & 0xffu) * 0.00390625f);
-    if (!alone) {
-#pragma unroll
-      for (int a = 0; a < 7; ++a) {
-        unsigned lo, hi;
-        split_round(v[a], lo, hi);
-        atomicAdd(&s_acc[(2 * a) * kAssignNL + e], lo);
-        atomicAdd(&s_acc[(2 * a + 1) * kAssignNL + e], hi);
-      }
-    } else {                                    // a single-member partial of its own
+    } else {                                  // a single-member partial of its own
       Partial p;
-      const unsigned slot = s_fk[hpos[j]];
+      const unsigned slot = s_fk[h];
       p.count = 1u;
-      p.sum.mmin = mexp[j];
-      p.sum.pad = 0;
-      p.rep = ((unsigned long long)cord[j] << 32) | (unsigned)(~(unsigned)gi[j]);
+      p.top[0] = pkey[j];
 #pragma unroll
-      for (int a = 0; a < 7; ++a) {
-        unsigned lo, hi;
-        split_round(v[a], lo, hi);
-        p.set_sum(a, ((unsigned long long)hi << kLoBits) + lo);
-      }
+      for (int a = 1; a < kMaxTopK; ++a) p.top[a] = 0ull;
       const unsigned pi = atomicAdd(&t.cnt->n_partials, 1u);
       if (pi >= t.max_partials) {
         atomicOr(&t.cnt->error, kErrPartials);
-      } else if (file_partial(t, p, slot, fkey[j], mexp[j], pi)) {
+      } else if (file_partial(t, p, slot, pi)) {
         const unsigned n = atomicAdd(&t.cnt->n_cells, 1u);
         if (n < t.max_slots) t.fused[n] = slot;
       }
@@ -1145,21 +1278,9 @@ k_assign(const __grid_constant__ BatchArgs<NB> args) {
         Partial p;
         slot = s_fk[h];
         p.count = s_cntp[h];
-        if constexpr (TOPK) {
-          const unsigned long long* top = reinterpret_cast<const unsigned long long*>(s_acc) + e * kMaxTopK;
-          p.rep = top[0];
 #pragma unroll
-          for (int a = 0; a < kMaxTopK - 1; ++a) p.top[a] = top[a + 1];
-        } else {
-          p.sum.mmin = s_minp[h];
-          p.sum.pad = 0;
-          p.rep = ((unsigned long long)s_cmaxp[h] << 32) | (unsigned)(~s_gmin[e]);
-#pragma unroll
-          for (int a = 0; a < 7; ++a)
-            p.set_sum(a, ((unsigned long long)s_acc[(2 * a + 1) * kAssignNL + e] << kLoBits) +
-                             s_acc[(2 * a) * kAssignNL + e]);
-        }
-        first = file_partial(t, p, slot, s_ek[e], TOPK ? INT_MAX : s_minp[h], pi);
+        for (int a = 0; a < kMaxTopK; ++a) p.top[a] = s_top[e * kMaxTopK + a];
+        first = file_partial(t, p, slot, pi);
       }
     }
     // one counter update per warp for the cells claimed in it
@@ -1188,54 +1309,45 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Bat
   pdl_wait();
   const unsigned n_cells = min(t.cnt->n_cells, t.max_slots);
   const unsigned n_coarse = min(t.cnt->n_coarse, t.cmask + 1u);
-  const unsigned n_part = min(t.cnt->n_partials, t.max_partials);
   const unsigned n = max(n_cells, n_coarse);
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     if (i < n_cells) {
       const unsigned slot = t.fused[i];
-      const SlotRec rec = t.frec[slot];
-      const unsigned long long key = rec.key;
-      const unsigned head = rec.head;
-      const int mmin = rec.mmin;
-      unsigned count = 0u, steps = 0u;
-      unsigned long long rep = 0ull;
-      unsigned long long S[7] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
-      for (unsigned p = head; p != kSlotNone && steps <= n_part; ++steps) {
-        const Partial P = t.part[p];
-        count += P.count;
-        rep = max(rep, P.rep);
-        const int sh = P.sum.mmin - mmin;      // shift to the cell's smallest exponent
-#pragma unroll
-        for (int a = 0; a < 7; ++a) S[a] += sh < 64 ? (P.get_sum(a) >> sh) : 0ull;
-        p = P.next;
-      }
-      if (steps > n_part) atomicOr(&t.cnt->error, kErrList);
-      const unsigned g = head != kSlotNone ? ~(unsigned)(rep & 0xffffffffull) : 0xffffffffu;
-      CellOut c;
-      // Eq. 11 in float32: position = edge (k + S_k / S_0), colour = 256 S_c / S_0,
-      // weight = S_0 2^-(36 + mmin); each result is within a few float32 roundings
-      const int l = (int)(key >> 60);
-      const float edge = __fmul_rn(out.s0_m, pow2f(-l));
-      const float Wf = u64_to_f32(S[0]);
-      const float inv = S[0] ? __frcp_rn(Wf) : __int_as_float(0x7fc00000);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const int ka = (int)((key >> (40 - 20 * a)) & 0xfffff) - kKeyBias;
-        c.pos[a] = __fmaf_rn(edge, (float)ka, __fmul_rn(edge, __fmul_rn(u64_to_f32(S[1 + a]), inv)));
-        c.rgb[a] = __fmul_rn(256.0f, __fmul_rn(u64_to_f32(S[4 + a]), inv));
-      }
-      c.weight = ldexpf(Wf, -kFixShift - min(mmin, 1 << 30));
-      c.count = count;
-      c.rep = g;
-      c.pad = 0u;
-      c.key = key;
+      const uint4 rec = __ldcg(reinterpret_cast<const uint4*>(t.frec + slot));
+      // ready for the next frame: no representative, no number, exponent INT_MAX
+      *reinterpret_cast<uint4*>(t.frec + slot) = make_uint4(0u, 0u, kSlotNone, (unsigned)INT_MAX);
       if ((long long)i < out.max_cells) {
+        const int mmin = (int)rec.w;
+        const unsigned long long key = t.ckey[i];
+        const ulonglong2* row = reinterpret_cast<const ulonglong2*>(t.acc + 8ull * i);
+        unsigned long long S[8];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          const ulonglong2 v = __ldcg(row + a);
+          S[2 * a] = v.x;
+          S[2 * a + 1] = v.y;
+        }
+        CellOut c;
+        // Eq. 11 in float32: position = edge (k + S_k / S_0), colour = 256 S_c / S_0,
+        // weight = S_0 2^-(36 + mmin); each result is within a few float32 roundings
+        const int l = (int)(key >> 60);
+        const float edge = __fmul_rn(out.s0_m, pow2f(-l));
+        const float Wf = u64_to_f32(S[0]);
+        const float inv = S[0] ? __frcp_rn(Wf) : __int_as_float(0x7fc00000);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int ka = (int)((key >> (40 - 20 * a)) & 0xfffff) - kKeyBias;
+          c.pos[a] = __fmaf_rn(edge, (float)ka, __fmul_rn(edge, __fmul_rn(u64_to_f32(S[1 + a]), inv)));
+          c.rgb[a] = __fmul_rn(256.0f, __fmul_rn(u64_to_f32(S[4 + a]), inv));
+        }
+        c.weight = ldexpf(Wf, -kFixShift - min(mmin, 1 << 30));
+        c.count = (unsigned)S[7];
+        c.rep = ~rec.x;
+        c.pad = 0u;
+        c.key = key;
         t.staged[i] = c;
-        if (head != kSlotNone) atomicOr(&t.bitmap[g >> 5], 1u << (g & 31));
+        atomicOr(&t.bitmap[c.rep >> 5], 1u << (c.rep & 31));
       }
-      // ready for the next frame: head = none, mmin = INT_MAX (one 8-byte store)
-      reinterpret_cast<unsigned long long*>(&t.frec[slot])[1] =
-          ((unsigned long long)(unsigned)INT_MAX << 32) | kSlotNone;
     }
     if (i < n_coarse) {
       const unsigned cs = t.cused[i];
@@ -1281,7 +1393,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_reduce_topk(const __grid_consta
         const Partial P = t.part[p];
         count += P.count;
         for (int a = 0; a < K; ++a) {           // insert the tile's key a into the sorted list
-          unsigned long long key = a == 0 ? P.rep : P.top[a - 1];
+          unsigned long long key = P.top[a];
 #pragma unroll
           for (int q = 0; q < kMaxTopK; ++q) {
             if (q < K && key > top[q]) {
@@ -1321,10 +1433,10 @@ __global__ void __launch_bounds__(kThreads, 3) k_reduce_topk(const __grid_consta
         world_point(C, z, __ldg(&rays[C.ray_x + x].x), __ldg(&rays[C.ray_y + y].x), P3[q]);
         float sh = 0.0f, sl = 0.0f;
         int nview = 0;
-        if (rig.use_cons && rig.k1 > 0)
-          residual_sum<DT>(t.bconst[cam], rig.k1, GlobalPairRays{t.pray, x, y}, rays, fp, z, sh,
-                           sl, nview);
-        joint_weight(rig, rig.k1, sh, sl, c, mu[q], mx[q]);
+        if (fa.hot.use_cons && rig.k1 > 0)
+          residual_sum<DT>(t.bconst + cam, t, cam, rig.k1, GlobalPairRays(t.pray + fa.ti.pray[cam], C.W, rig.k1, x, y),
+                           rigp, fa.hot, rays, fp, z, x, y, sh, sl, nview);
+        joint_weight(fa.hot, rig.k1, sh, sl, c, mu[q], mx[q]);
         mmin = min(mmin, mx[q]);
         col[q][0] = px[0];
         col[q][1] = px[1];
@@ -1382,9 +1494,10 @@ __global__ void __launch_bounds__(kThreads, 3) k_reduce_topk(const __grid_consta
 // copied), so the cloud is in pixel order without a compaction pass.  One thread a pixel,
 // cameras along the grid's second dimension.
 template <typename DT>
-__global__ void __launch_bounds__(kThreads) k_points(const RigDev* __restrict__ rigp,
-                                                     const float2* __restrict__ rays, FramePtrs fp,
-                                                     Tables t, PointsDev out) {
+__global__ void __launch_bounds__(kThreads) k_points(const RigDev* __restrict__ rigp, const __grid_constant__ RigHot hot,
+                                                     const float2* __restrict__ rays,
+                                                     const __grid_constant__ FramePtrs fp,
+                                                     const __grid_constant__ Tables t, PointsDev out) {
   const RigDev& rig = *rigp;
   const int cam = blockIdx.y;
   const CamDev& C = rig.cam[cam];
@@ -1400,7 +1513,7 @@ __global__ void __launch_bounds__(kThreads) k_points(const RigDev* __restrict__ 
     const DT D = dep[li];
     const float c = cf[li];
     const bool valid = Depth<DT>::valid(D);
-    const bool gated = valid && (!rig.use_conf || c > rig.tau);          // Eq. 9
+    const bool gated = valid && (!hot.use_conf || c > hot.tau);          // Eq. 9
     nv += valid ? 1u : 0u;
     ng += gated ? 1u : 0u;
     out.rgb[3 * g] = col[3 * li];
@@ -1419,9 +1532,10 @@ __global__ void __launch_bounds__(kThreads) k_points(const RigDev* __restrict__ 
     world_point(C, z, __ldg(&rays[C.ray_x + x].x), __ldg(&rays[C.ray_y + y].x), P);   // Eq. 8
     float sh = 0.0f, sl = 0.0f, mu;
     int nview = 0, m;
-    if (rig.use_cons && rig.k1 > 0)
-      residual_sum<DT>(t.bconst[cam], rig.k1, GlobalPairRays{t.pray, x, y}, rays, fp, z, sh, sl, nview);
-    joint_weight(rig, rig.k1, sh, sl, c, mu, m);                          // Eq. 7, 10
+    if (hot.use_cons && rig.k1 > 0)
+      residual_sum<DT>(t.bconst + cam, t, cam, rig.k1, GlobalPairRays(t.pray + t.bconst[cam].cam.pray, C.W, rig.k1, x, y),
+                       rigp, hot, rays, fp, z, x, y, sh, sl, nview);
+    joint_weight(hot, rig.k1, sh, sl, c, mu, m);                          // Eq. 7, 10
     out.pos[3 * g] = __fmul_rn(P[0], out.unit_f);
     out.pos[3 * g + 1] = __fmul_rn(P[1], out.unit_f);
     out.pos[3 * g + 2] = __fmul_rn(P[2], out.unit_f);
@@ -1798,7 +1912,7 @@ __global__ void k_init_tables(Tables t, unsigned fcap, unsigned ccap) {
   const unsigned n = max(fcap, ccap);
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     if (i < fcap) {
-      t.frec[i].key = kKeyEmpty;
+      t.frec[i].key = 0ull;
       t.frec[i].head = kSlotNone;
       t.frec[i].mmin = INT_MAX;
     }
@@ -1955,31 +2069,32 @@ __global__ void __launch_bounds__(kThreads) k_screen_rows(ScreenArgs a) {
 }
 
 template <typename DT, int TH>
-cudaError_t set_assign_attributes_th() {
-  const int sm = (int)AssignTile<TH>::smem(kMaxK1);
+cudaError_t set_tile_attributes_th() {
+  const int sm = (int)WeighTile<TH>::smem(kMaxK1);
   const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(k_assign<DT, false, false, 1, TH>, at, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_assign<DT, false, true, 1, TH>, at, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_assign<DT, true, false, 1, TH>, at, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_assign<DT, true, true, 1, TH>, at, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_assign<DT, false, false, kMaxBatch, TH>, at, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_assign<DT, true, false, kMaxBatch, TH>, at, sm);
+  cudaError_t e = cudaFuncSetAttribute(k_weigh<DT, false, 1, TH>, at, sm);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_weigh<DT, true, 1, TH>, at, sm);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_weigh<DT, false, kMaxBatch, TH>, at, sm);
+  const int tk = (int)AssignTile<TH>::Bytes;
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_assign_topk<DT, false, 1, TH>, at, tk);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_assign_topk<DT, true, 1, TH>, at, tk);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_assign_topk<DT, false, kMaxBatch, TH>, at, tk);
   return e;
 }
 
-// Dynamic shared memory limit of the assign kernels for one depth type, set once per device
+// Dynamic shared memory limits of the tile kernels for one depth type, set once per device
 // (the first call comes from context creation, outside any stream capture).  The attribute
 // call is idempotent, so two host threads that race here only repeat it.
 template <typename DT>
-cudaError_t set_assign_attributes() {
+cudaError_t set_tile_attributes() {
   static std::atomic<unsigned long long> done{0ull};       // one bit per device (< 64)
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
   const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
   if (bit && (done.load(std::memory_order_acquire) & bit)) return cudaSuccess;
-  cudaError_t e = set_assign_attributes_th<DT, 8>();
-  if (e == cudaSuccess) e = set_assign_attributes_th<DT, 16>();
-  if (e == cudaSuccess) e = set_assign_attributes_th<DT, 32>();
+  cudaError_t e = set_tile_attributes_th<DT, 8>();
+  if (e == cudaSuccess) e = set_tile_attributes_th<DT, 16>();
+  if (e == cudaSuccess) e = set_tile_attributes_th<DT, 32>();
   if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
   return e;
 }
@@ -2002,27 +2117,43 @@ cudaError_t launch_k(bool pdl, void (*kernel)(P...), dim3 grid, dim3 block, size
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// The assign step over the batch's tiles (TH rows a tile; the traced instantiation exists for
-// single frames only).
+// Threads of a weigh or sum block: a thread for four pixels, or fewer while all of a launch's blocks
+// fit on the chip at once (a frame of 80 tiles then takes a pixel a thread instead of four in turn).
+int weigh_threads(int tiles, int th) {
+  int n = 8 * th;
+  while (n < 32 * th && n < 512 && 2ll * n * tiles <= 152 * 1024) n *= 2;
+  return n;
+}
+
+// The assign step over the batch's tiles (TH rows a tile; the traced instantiations exist for
+// single frames only): weigh and sum, or the top-k variant's kernel.
 template <typename DT, int NB, int TH>
 cudaError_t launch_assign(const BatchArgs<NB>& a, int n, bool top_k, bool traced, int max_k1, bool pdl,
                           cudaStream_t s) {
-  const dim3 tiles(a.tile_first[n]), at(AssignTile<TH>::Threads);
-  const size_t sm = AssignTile<TH>::smem(top_k ? 0 : max_k1);
-  if constexpr (NB == 1) {
-    if (traced)
-      return top_k ? launch_k(pdl, k_assign<DT, true, true, NB, TH>, tiles, at, sm, s, a)
-                   : launch_k(pdl, k_assign<DT, false, true, NB, TH>, tiles, at, sm, s, a);
+  const int threads = weigh_threads(a.tile_first[n], TH);
+  const dim3 tiles(a.tile_first[n]), at(AssignTile<TH>::Threads), wt(threads);
+  if (top_k) {
+    if constexpr (NB == 1)
+      if (traced) return launch_k(pdl, k_assign_topk<DT, true, NB, TH>, tiles, at, AssignTile<TH>::Bytes, s, a);
+    return launch_k(pdl, k_assign_topk<DT, false, NB, TH>, tiles, at, AssignTile<TH>::Bytes, s, a);
   }
-  return top_k ? launch_k(pdl, k_assign<DT, true, false, NB, TH>, tiles, at, sm, s, a)
-               : launch_k(pdl, k_assign<DT, false, false, NB, TH>, tiles, at, sm, s, a);
+  const size_t sm = WeighTile<TH>::smem(max_k1);
+  cudaError_t e = cudaSuccess;
+  bool done = false;
+  if constexpr (NB == 1)
+    if (traced) {
+      e = launch_k(pdl, k_weigh<DT, true, NB, TH>, tiles, wt, sm, s, a);
+      done = true;
+    }
+  if (!done) e = launch_k(pdl, k_weigh<DT, false, NB, TH>, tiles, wt, sm, s, a);
+  return e != cudaSuccess ? e : launch_k(pdl, k_sum<DT, NB, TH>, tiles, wt, 16 * kSumWarpWords * (threads / 32), s, a);
 }
 
 // The frame kernels over n frames (NB = 1: one frame; NB = kMaxBatch: a batch of up to
 // that many frames of any rigs, every kernel launched once for all of them).
 template <typename DT, int NB>
 cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEvent_t* ev) {
-  const cudaError_t ae = set_assign_attributes<DT>();
+  const cudaError_t ae = set_tile_attributes<DT>();
   if (ae != cudaSuccess) return ae;
   if (n < 1 || n > NB) return cudaErrorInvalidValue;
   auto mark = [&](int i) { if (ev) cudaEventRecord(ev[i], s); };
@@ -2046,7 +2177,8 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
     fa.tr = fr[f].tr;
     fa.out = fr[f].out;
     fa.ti = geo.tiles;
-    fa.count_blocks_x = geo.count_blocks_x;
+    fa.hot = geo.hot;
+    fa.top_k = geo.top_k;
     fa.count_chunks = geo.count_chunks;
     fa.unit_m = (float)fr[f].out.unit_m;
     if (geo.screen) {                      // D^r of Eq. 8 into the context's buffers
@@ -2057,7 +2189,7 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
       }
       if ((err = launch_screen(sa, sizeof(DT) == 4, geo.max_px, s)) != cudaSuccess) return err;
     }
-    a.count_first[f + 1] = a.count_first[f] + geo.count_blocks_x * geo.n_cams;
+    a.count_first[f + 1] = a.count_first[f] + geo.count_blocks;
     a.tile_first[f + 1] = a.tile_first[f] + t.n_tiles;
     emit = std::max(emit, geo.emit_blocks);
     pdl_level = std::min(pdl_level, geo.pdl);
@@ -2108,12 +2240,12 @@ int resident_th(int k1) {
   const int known = cache[k1].load(std::memory_order_relaxed);
   if (known > 0) return known;
   int n = 0;
-  const int sm = (int)AssignTile<TH>::smem(k1);
-  if (set_assign_attributes<uint16_t>() != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_assign<uint16_t, false, false, 1, TH>,
-                                                    AssignTile<TH>::Threads, sm) != cudaSuccess) {
+  const int sm = (int)WeighTile<TH>::smem(k1);
+  if (set_tile_attributes<uint16_t>() != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_weigh<uint16_t, false, 1, TH>, WeighTile<TH>::Threads, sm) !=
+          cudaSuccess) {
     cudaGetLastError();
-    return AssignTile<TH>::BlocksPerSM;
+    return 1024 / WeighTile<TH>::Threads;
   }
   n = std::max(1, n);
   cache[k1].store(n, std::memory_order_relaxed);
@@ -2127,15 +2259,23 @@ int assign_resident_blocks(int th, int k1) {
 
 int retile(TileIndex* ti, int th) {
   ti->th = th;
-  int n = 0;
+  int n = 0, u = 0;
+  bool same = true;
   for (int i = 0; i < ti->n_cams; ++i) {
+    const int tx = (ti->W[i] + kTileW - 1) / kTileW;
     ti->first[i] = n;
-    n += ((ti->W[i] + kTileW - 1) / kTileW) * ((ti->H[i] + th - 1) / th);
+    ti->unit[i] = u;
+    ti->div_x[i] = fast_div_factor((unsigned)tx);
+    n += tx * ((ti->H[i] + th - 1) / th);
+    u += tx * ((ti->H[i] + kUnitH - 1) / kUnitH);
+    same = same && ti->W[i] == ti->W[0] && ti->H[i] == ti->H[0];
   }
   ti->first[ti->n_cams] = n;
-  bool same = true;
-  for (int i = 1; i < ti->n_cams; ++i) same = same && ti->W[i] == ti->W[0] && ti->H[i] == ti->H[0];
+  ti->unit[ti->n_cams] = u;
   ti->per_cam = same && ti->n_cams > 0 ? ti->first[1] : 0;
+  ti->units_per_cam = same && ti->n_cams > 0 ? ti->unit[1] : 0;
+  ti->div_cam = ti->per_cam ? fast_div_factor((unsigned)ti->per_cam) : 0u;
+  ti->div_units = ti->units_per_cam ? fast_div_factor((unsigned)ti->units_per_cam) : 0u;
   return n;
 }
 
@@ -2143,24 +2283,50 @@ int fill_tile_index(const RigDev& rig, TileIndex* out, int th) {
   memset(out, 0, sizeof(*out));
   out->n_cams = rig.n_cams;
   out->k1 = rig.k1;
+  long long pray = 0;
   for (int i = 0; i < rig.n_cams; ++i) {
     out->W[i] = rig.cam[i].W;
     out->H[i] = rig.cam[i].H;
     out->off[i] = rig.cam[i].off;
-    out->pray[i] = rig.k1 > 0 ? rig.pair[rig.cam[i].pair0].ga : 0;
+    out->pray[i] = (int)pray;
+    pray += pray_cam_size(rig.cam[i].W, rig.cam[i].H, rig.k1);
   }
   out->ahead = kNoPrefetch;                      // no prefetch unless the caller sets it
   return retile(out, th);
 }
 
 void fill_block_consts(const RigDev& rig, BlockConst* out) {
+  long long pray = 0;
   for (int i = 0; i < rig.n_cams; ++i) {
     BlockConst& b = out[i];
     memset(&b, 0, sizeof(b));
-    b.cam = rig.cam[i];
+    const CamDev& c = rig.cam[i];
+    memcpy(b.cam.Rwc, c.Rwc, sizeof(c.Rwc));
+    memcpy(b.cam.cwc, c.cwc, sizeof(c.cwc));
+    b.cam.ray_x = c.ray_x;
+    b.cam.ray_y = c.ray_y;
+    b.cam.pray = (int)pray;
+    b.cam.pair0 = c.pair0;
+    pray += pray_cam_size(c.W, c.H, rig.k1);
     for (int q = 0; q < rig.k1; ++q) {
-      b.pair[q] = rig.pair[rig.cam[i].pair0 + q];
-      b.nb[q] = rig.cam[b.pair[q].j];
+      const PairDev& p = rig.pair[c.pair0 + q];
+      const CamDev& n = rig.cam[p.j];
+      ViewHot& v = b.view[q];
+      for (int a = 0; a < 3; ++a) {
+        v.mt[a] = kGridM + p.th[a];
+        v.tl[a] = p.tl[a];
+      }
+      v.fx = n.fx;
+      v.fy = n.fy;
+      v.cx5 = (float)((double)n.cxh + (double)n.cxl + 0.5);
+      v.cy5 = (float)((double)n.cyh + (double)n.cyl + 0.5);
+      v.W = n.W;
+      v.H = n.H;
+      v.ray_x = n.ray_x;
+      v.ray_y = n.ray_y;
+      // twice the error bound of the float32 projection (nearest_pixel)
+      v.band = (float)std::max(n.W + std::fabs((double)n.cx), n.H + std::fabs((double)n.cy)) / 1048576.0f;
+      v.j = p.j;
     }
   }
 }
@@ -2196,15 +2362,15 @@ cudaError_t launch_mc(const RigDev* rig, const FramePtrs& fp, bool depth_f32, co
   return cudaGetLastError();
 }
 
-cudaError_t launch_points(const RigDev* rig, const float2* rays, const FramePtrs& fp, const Tables& t,
+cudaError_t launch_points(const RigDev* rig, const RigHot& hot, const float2* rays, const FramePtrs& fp, const Tables& t,
                           const PointsDev& out, bool depth_f32, int n_cams, long long max_px,
                           cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(out.counts, 0, 2 * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   const long long per = (max_px + kThreads - 1) / kThreads;
   const dim3 g((unsigned)std::max(1ll, std::min<long long>(per, 4 * 152)), n_cams);
-  if (depth_f32) k_points<float><<<g, kThreads, 0, s>>>(rig, rays, fp, t, out);
-  else k_points<uint16_t><<<g, kThreads, 0, s>>>(rig, rays, fp, t, out);
+  if (depth_f32) k_points<float><<<g, kThreads, 0, s>>>(rig, hot, rays, fp, t, out);
+  else k_points<uint16_t><<<g, kThreads, 0, s>>>(rig, hot, rays, fp, t, out);
   return cudaGetLastError();
 }
 
@@ -2231,7 +2397,7 @@ cudaError_t launch_screen(const ScreenArgs& a, bool depth_f32, long long max_px,
 }
 
 cudaError_t prepare_launch(bool depth_f32) {
-  return depth_f32 ? set_assign_attributes<float>() : set_assign_attributes<uint16_t>();
+  return depth_f32 ? set_tile_attributes<float>() : set_tile_attributes<uint16_t>();
 }
 
 cudaError_t launch_frame(const RigDev* rig, const float2* rays, const FramePtrs& fp, const Tables& t,

@@ -1,0 +1,64 @@
+"""Edges of the steps that work on units of 32 x 8 pixels, against the oracle at the parity
+tolerances: units with more coarse cells than they have numbers, cells outside a unit's key
+window, grids of no more than 1024 cells an axis (where points leave the grid), float32 depths
+beyond the range of the grid evaluation of the consistency step, and image sizes one pixel to
+each side of the units' and tiles' edges."""
+import numpy as np
+import pytest
+
+from paper_2602_01035_gb300 import scenes as S
+from parity import compare, run_gpu
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _check(oracle_mod, rig, fr, **params):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_01035_gb300 import fuseflow
+    ff = fuseflow.FuseFlow(rig, **params)
+    try:
+        gpu = run_gpu(ff, fr, torch)
+        again = run_gpu(ff, fr, torch, with_trace=False)
+    finally:
+        ff.close()
+    assert gpu["status"] == fuseflow.FUSEFLOW_OK, gpu["stats"]
+    for k, v in gpu["cells"].items():                      # reproducible, traced or not
+        assert np.array_equal(v, again["cells"][k], equal_nan=v.dtype.kind == "f"), k
+    orc = oracle_mod.fuse_frame(rig, fr, {k: v for k, v in params.items() if k != "max_cells"})
+    return compare(gpu, orc, oracle_mod), gpu
+
+
+def _scattered(rig, seed, lo, hi, dtype=np.uint16):
+    rng = np.random.default_rng(seed)
+    shape = [(c.height, c.width) for c in rig.cameras]
+    z = [rng.uniform(lo, hi, size=s).astype(dtype) for s in shape]
+    return S.Frame(z, [rng.uniform(0.55, 1.0, size=s).astype(np.float32) for s in shape],
+                   [rng.integers(0, 256, size=s + (3,), dtype=np.uint8) for s in shape])
+
+
+@pytest.mark.parametrize("coarse,level", [
+    (0.32, 2),      # more than 64 coarse cells in a unit, all in one window
+    (0.015, 1),     # points more than 512 cells apart in a unit
+    (0.32, 10),     # 1024 cells an axis: every cell in the window
+    (0.32, 14),     # 64 cells an axis: points leave the grid
+])
+def test_scattered_units(oracle_mod, coarse, level):
+    rig = S.tiny_rig(n=3, width=71, height=35, fx=60.0, fy=60.0)
+    rep, gpu = _check(oracle_mod, rig, _scattered(rig, 5, 500, 40000), coarse_cell_m=coarse, max_level=level, n_min=2)
+    assert rep["n_points_compared"] > 0.3 * gpu["stats"]["n_gated"] or level == 14
+    assert (gpu["stats"]["n_out_of_range"] > 0) == (level == 14)
+
+
+@pytest.mark.parametrize("coarse", [0.32, 8.0])
+def test_float_depths_beyond_the_grid_range(oracle_mod, coarse):
+    rig = S.tiny_rig(n=4, width=64, height=40, depth_format="f32", depth_scale=1.0, fx=60.0, fy=60.0)
+    rep, gpu = _check(oracle_mod, rig, _scattered(rig, 6, 1.0, 100.0, np.float32), coarse_cell_m=coarse, max_level=1)
+    assert rep["n_points_compared"] > 0.5 * gpu["stats"]["n_gated"]
+
+
+@pytest.mark.parametrize("w,h", [(31, 7), (32, 8), (33, 9), (65, 17), (1, 16), (64, 33)])
+def test_sizes_around_units(oracle_mod, w, h):
+    rig = S.tiny_rig(n=3, width=w, height=h, fx=40.0, fy=40.0)
+    _check(oracle_mod, rig, S.random_frame(rig, seed=7), n_min=2)
