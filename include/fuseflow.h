@@ -156,8 +156,8 @@ int fuseflow_fuse_frame(fuseflow_ctx *ctx, const void *const *depth, const float
 /* A fuse call recorded once as a CUDA graph, for callers whose input images live in the
  * same device buffers every frame (a capture loop that refills them): replaying it with
  * fuseflow_graph_launch is the same as calling fuseflow_fuse_frame with the pointers
- * given here, whose contents may change between launches, at one launch instead of eight
- * (nine with a depth screen set).
+ * given here, whose contents may change between launches, at one launch instead of five
+ * (six with a depth screen set).
  * The graph keeps the context's launch geometry and trace registration as they were at
  * creation; results do not depend on the geometry.  It uses the context's tables, so
  * launches of graphs and fuse calls of one context must be ordered (one stream), and
@@ -286,8 +286,9 @@ int fuseflow_get_neighbours(const fuseflow_ctx *ctx, int32_t *out, int32_t *k_mi
  * events between its stages on its own stream (a ring of the last 1024 frames).
  * fuseflow_read_stage_times waits for the last recorded event, writes the summed
  * milliseconds of each of the FUSEFLOW_N_STAGES stages to ms[] and the number of frames
- * to *n_frames, then resets the ring.  Stages: 0 clear (and the depth screen when one is
- * set), 1 count (a, c2), 2 assign (b, c, d per tile), 3 reduce (d per cell), 4 scan,
+ * to *n_frames, then resets the ring.  Stages: 0 clear (the depth screen
+ * when one is set; nothing else is cleared ahead of a frame), 1 count (a, c2), 2 assign (b, c
+ * per point), 3 reduce (d: sums per cell), 4 scan (nothing: ranks are found by the emit step),
  * 5 emit. */
 #define FUSEFLOW_N_STAGES 6
 int fuseflow_enable_stage_timing(fuseflow_ctx *ctx, int enable);
@@ -298,7 +299,7 @@ const char *fuseflow_stage_name(int stage);
  * and any trace are bitwise the same for every admissible setting (the path has no
  * order-dependent arithmetic).  A setting can be chosen by timing alone.
  *   count_chunks    2048-pixel chunks per block of the coarse-count step, 1..64
- *   emit_blocks     blocks of the level, reduce and emit steps, 1..65536
+ *   emit_blocks     blocks of the level step and of the top-k reduce step, 1..65536
  *   prefetch_tiles  how many tiles ahead each block of the assign step's first kernel
  *                   prefetches colours into L2 for its second; 0 turns the prefetch off
  *   programmatic    2: each kernel of a frame after the first is launched with

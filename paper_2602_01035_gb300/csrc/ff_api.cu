@@ -453,7 +453,7 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   // ---------------------------------------------------------------- device memory
   int status = FUSEFLOW_OK;
   const long long n_words = (off + 31) / 32;
-  const int n_wblocks = (int)((n_words + 1023) / 1024);
+  const int n_wblocks = (int)((n_words + kRankWords - 1) / kRankWords);
   // block statistics for the finest count geometry a tuning may choose (one chunk a block)
   ctx->bstats_cap = (ctx->n_units + 7) / 8;
   size_t o = 0;
@@ -470,8 +470,7 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   const size_t o_cnt = take(sizeof(FrameCounters) + sizeof(unsigned) * (size_t)n_words, 256);
   const size_t o_bst = take(sizeof(BlockStats) * (size_t)ctx->bstats_cap, 256);
   const size_t o_part = take(sizeof(Partial) * (size_t)max_partials, 256);
-  const size_t o_staged = take(sizeof(CellOut) * (size_t)ctx->max_cells, 256);
-  const size_t o_wpre = take(sizeof(unsigned) * (size_t)n_words, 256);
+  const size_t o_staged = take(topk ? sizeof(CellOut) * (size_t)ctx->max_cells : 0, 256);
   const size_t o_bsum = take(sizeof(unsigned) * (size_t)n_wblocks, 256);
   const size_t o_lpix = take(sizeof(unsigned short) * (size_t)off, 256);
   const size_t o_ldep = take((rig->depth_f32 ? 4 : 2) * (size_t)off, 256);
@@ -481,8 +480,7 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   const size_t o_wslot = take(sizeof(unsigned) * n_weighed, 256);
   const size_t o_wmant = take(sizeof(float) * n_weighed, 256);
   const size_t o_wexp = take(sizeof(int) * n_weighed, 256);
-  const size_t o_acc = take(8 * sizeof(unsigned long long) * n_summed, 256);
-  const size_t o_ckey = take(sizeof(unsigned long long) * n_summed, 256);
+  const size_t o_rows = take(sizeof(CellRow) * n_summed, 256);
   ctx->table_bytes = o;
   size_t po = 0;
   auto take_out = [&](size_t bytes) { po = align_up(po, 256); size_t at = po; po += bytes; return at; };
@@ -541,8 +539,8 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
     t.wslot = reinterpret_cast<unsigned*>(b + o_wslot);
     t.wmant = reinterpret_cast<float*>(b + o_wmant);
     t.wexp = reinterpret_cast<int*>(b + o_wexp);
-    t.acc = reinterpret_cast<unsigned long long*>(b + o_acc);
-    t.ckey = reinterpret_cast<unsigned long long*>(b + o_ckey);
+    t.rows = reinterpret_cast<CellRow*>(b + o_rows);
+    t.cell_at = reinterpret_cast<unsigned*>(t.lconf);
     t.cused = reinterpret_cast<unsigned*>(b + o_cused);
     t.cmask = ctx->ccap - 1;
     t.cnt = reinterpret_cast<FrameCounters*>(b + o_cnt);
@@ -552,7 +550,6 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
     t.part = reinterpret_cast<Partial*>(b + o_part);
     t.max_partials = max_partials;
     t.staged = reinterpret_cast<CellOut*>(b + o_staged);
-    t.wprefix = reinterpret_cast<unsigned*>(b + o_wpre);
     t.bsum = reinterpret_cast<unsigned*>(b + o_bsum);
     t.n_words = n_words;
     t.n_wblocks = n_wblocks;
@@ -1220,7 +1217,7 @@ constexpr int kStaticMaxPairRays = 6 * kStaticMaxRays;  // bound of 2 (K - 1) su
 // the padded tables of an admitted rig fit in as many float4: 1.5 (K - 1) (sum(W + H) + 62 a camera)
 static_assert(3 * (kStaticMaxPairRays / 2 + 62ll * kMaxCams * kMaxK1) / 2 <= kStaticMaxPairRays, "pair-ray tables fit");
 constexpr long long kStaticWords = kStaticMaxPixels / 32;
-constexpr int kStaticWBlocks = (int)((kStaticWords + 1023) / 1024);
+constexpr int kStaticWBlocks = (int)((kStaticWords + kRankWords - 1) / kRankWords);
 // units of 32 x 8 pixels: at most W H / 256 + W / 32 + H / 8 + 1 a camera
 constexpr int kStaticUnits = (int)(kStaticMaxPixels / 256) + kStaticMaxRays / 8 + kMaxCams;
 constexpr int kStaticBStats = kStaticUnits / 8 + 1;    // chunks = 1
@@ -1241,12 +1238,10 @@ constexpr size_t kSPart = al256(kSBStats + sizeof(BlockStats) * kStaticBStats);
 // a call uses either the top-k variant's partials or, in the same place, the others' weights and sums
 constexpr size_t kSWMant = al256(kSPart + sizeof(unsigned) * kStaticMaxPixels);
 constexpr size_t kSWExp = al256(kSWMant + sizeof(float) * kStaticMaxPixels);
-constexpr size_t kSAcc = al256(kSWExp + sizeof(int) * kStaticMaxPixels);
-constexpr size_t kSCKey = al256(kSAcc + 8 * sizeof(unsigned long long) * kStaticMaxCells);
+constexpr size_t kSRows = al256(kSWExp + sizeof(int) * kStaticMaxPixels);
 constexpr size_t kSStaged = std::max(al256(kSPart + sizeof(Partial) * kStaticMaxPartials),
-                                     al256(kSCKey + sizeof(unsigned long long) * kStaticMaxCells));
-constexpr size_t kSWPre = al256(kSStaged + sizeof(CellOut) * kStaticMaxCells);
-constexpr size_t kSBSum = al256(kSWPre + sizeof(unsigned) * kStaticWords);
+                                     al256(kSRows + sizeof(CellRow) * kStaticMaxCells));
+constexpr size_t kSBSum = al256(kSStaged + sizeof(CellOut) * kStaticMaxCells);
 constexpr size_t kSLPix = al256(kSBSum + sizeof(unsigned) * kStaticWBlocks);
 constexpr size_t kSLDepth = al256(kSLPix + sizeof(unsigned short) * kStaticMaxPixels);
 constexpr size_t kSLConf = al256(kSLDepth + sizeof(float) * kStaticMaxPixels);
@@ -1316,18 +1311,17 @@ Tables static_tables(unsigned char* base, long long n_px, int n_bstats) {
   t.wslot = reinterpret_cast<unsigned*>(base + kSPart);
   t.wmant = reinterpret_cast<float*>(base + kSWMant);
   t.wexp = reinterpret_cast<int*>(base + kSWExp);
-  t.acc = reinterpret_cast<unsigned long long*>(base + kSAcc);
-  t.ckey = reinterpret_cast<unsigned long long*>(base + kSCKey);
+  t.rows = reinterpret_cast<CellRow*>(base + kSRows);
   t.staged = reinterpret_cast<CellOut*>(base + kSStaged);
-  t.wprefix = reinterpret_cast<unsigned*>(base + kSWPre);
   t.bsum = reinterpret_cast<unsigned*>(base + kSBSum);
   t.lpix = reinterpret_cast<unsigned short*>(base + kSLPix);
   t.ldepth = base + kSLDepth;
   t.lconf = reinterpret_cast<float*>(base + kSLConf);
+  t.cell_at = reinterpret_cast<unsigned*>(t.lconf);
   t.lcount = reinterpret_cast<unsigned*>(base + kSLCount);
   t.lcell = reinterpret_cast<unsigned*>(base + kSLCell);
   t.n_words = (n_px + 31) / 32;
-  t.n_wblocks = (int)((t.n_words + 1023) / 1024);
+  t.n_wblocks = (int)((t.n_words + kRankWords - 1) / kRankWords);
   return t;
 }
 

@@ -178,7 +178,21 @@ struct __align__(16) CoarseEntry {
 };
 constexpr unsigned kBaseNone = (1u << 27) - 1u;    // base field of a coarse cell without slots
 
-// Fused cell staged by the reduce step (indexed by insertion order) for the emit step.
+// By cell number: exact sums of Eq. 11 {w, w frac xyz, w rgb / 256, members} in units of
+// 2^-(kFixShift + mmin), the cell's key and slot.
+struct __align__(32) CellRow {
+  unsigned long long sum[8];
+  unsigned long long key;
+  unsigned slot;
+  int mmin;                      // smallest exponent, once the weigh step is over
+  unsigned pad[4];
+};
+static_assert(sizeof(CellRow) == 96, "three sectors a cell");
+
+// Bitmap words of an emit block's share.
+constexpr int kRankWords = 256;
+
+// Fused cell staged by the top-k reduce step (by cell number) for the emit step.
 struct __align__(16) CellOut {
   float pos[3];
   float rgb[3];
@@ -190,15 +204,10 @@ struct __align__(16) CellOut {
 };
 static_assert(sizeof(CellOut) == 48, "staged cell layout");
 
-struct FrameCounters {           // zeroed before every frame
+struct FrameCounters {           // zero between frames
   unsigned n_cells, n_coarse;
   unsigned error;
   unsigned n_partials;
-  unsigned long long n_valid, n_gated, n_oor;
-  unsigned bmin_inv[3];          // ~ordered(min): max-reduced so that zero is neutral
-  unsigned bmax[3];              // ordered(max)
-  unsigned scan_done;            // blocks of the scan step that have finished
-  unsigned pad;
   unsigned long long n_slots;    // dense cell slots claimed (sum over coarse cells of 8^l)
 };
 

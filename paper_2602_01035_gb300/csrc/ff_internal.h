@@ -18,7 +18,7 @@ struct FramePtrs {               // one frame's caller-owned device images, per 
 struct Tables {                  // context-owned device scratch
   // cells: dense slots, coarse cell c owns [cbase(c), cbase(c) + 8^level(c))
   SlotRec* frec;                 // key, list head and smallest exponent per slot
-  unsigned* fused;               // used slots, in claim order
+  unsigned* fused;               // slots by cell number: those past the output's capacity (top-k: all)
   unsigned max_slots;
   // coarse hash table (open addressing), ccap entries
   CoarseEntry* coarse;
@@ -31,15 +31,13 @@ struct Tables {                  // context-owned device scratch
   unsigned* wslot;
   float* wmant;
   int* wexp;
-  // by cell number, max_cells entries: exact sums of Eq. 11 (eight a cell) and the cell's key
-  unsigned long long* acc;
-  unsigned long long* ckey;
+  CellRow* rows;                 // by cell number, max_cells entries
   Partial* part;                 // top-k variant: (tile, cell) partials, max_partials entries
   unsigned max_partials;
-  CellOut* staged;               // fused cells by claim order, max_cells entries
+  CellOut* staged;               // top-k variant: fused cells by cell number, max_cells entries
   unsigned* bitmap;              // representative bitmap, one bit per pixel
-  unsigned* wprefix;             // per-word exclusive prefix within its 1024-word block
-  unsigned* bsum;                // per 1024-word block: exclusive prefix after the scan
+  unsigned* cell_at;             // cell number at a representative's pixel (the place of lconf)
+  unsigned* bsum;                // representatives per kRankWords words of the bitmap
   long long n_words;
   int n_wblocks;
   int n_min, max_level;          // level rule (Sec. II.5(1)d)

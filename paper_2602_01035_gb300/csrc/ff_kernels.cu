@@ -2,7 +2,6 @@
 //
 // Launch sequence of one frame (all on the caller's stream; from the level step on,
 // optionally as programmatic dependent launches, see pdl_release / pdl_wait):
-//   memset   frame counters + representative bitmap
 //   screen   (only with a depth screen set) D^r of Eq. 8 into the context's buffers
 //   count    (a) decode + gate (Eq. 9) of units of 32x8 pixels, a warp each; the gated pixels are
 //            listed, back-projected (Eq. 8) and counted per coarse cell (Sec. II.5(1)c); per-block
@@ -13,13 +12,12 @@
 //            as mantissa/exponent; (c) cell key (Sec. II.5(1)e) and dense slot; per cell its
 //            representative (Sec. II.5(2)a) and smallest weight exponent
 //   sum      (d) exact fixed-point sums of omega, omega P, omega RGB per cell (Eq. 11) at the scale
-//            of its smallest exponent
-//   reduce   per cell: Eq. 11 from its sums, stage the fused cell, mark its representative; the used
-//            slots and coarse entries are cleared for the next frame
+//            of its smallest exponent; the representatives are marked, the coarse entries cleared
 //            (top-k variant: k_assign_topk keeps each tile's most confident members of a cell
-//            instead of weigh and sum, and k_reduce_topk weighs and fuses each cell's k)
-//   scan     ranks of the representatives (output order) and frame statistics
-//   emit     fused cells in representative order
+//            instead of weigh, and k_reduce_topk weighs and fuses each cell's k instead of sum)
+//   emit     ranks of the representatives (output order), Eq. 11 from each cell's sums, output and
+//            frame statistics; the used slots, the bitmap and the counters are cleared for the next
+//            frame
 // Outside the frame sequence: k_copyout (served frames: cloud into pinned host memory),
 // k_mc (the multi-camera depth consistency error of Eq. 12 on a point set), k_confidence
 // (Eq. 3 confidence from depth) and the stand-alone depth screen.
@@ -116,6 +114,7 @@ __global__ void __launch_bounds__(kThreads) k_levels(const __grid_constant__ Bat
   const unsigned n_coarse = min(t.cnt->n_coarse, t.cmask + 1u);
   const int lane = threadIdx.x & 31;
   const unsigned long long cap = t.max_slots;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < t.n_wblocks; i += gridDim.x * blockDim.x) t.bsum[i] = 0u;
   for (unsigned base = blockIdx.x * blockDim.x; base < n_coarse; base += gridDim.x * blockDim.x) {
     const unsigned i = base + threadIdx.x;
     unsigned cs = 0, l = 0;
@@ -547,7 +546,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ B
     }
     if (lane < 4) reinterpret_cast<float4*>(&s_cam[warp])[lane] = __ldg(reinterpret_cast<const float4*>(t.bconst + cam) + lane);
     __syncwarp();
-    const CamHot& cam_c = s_cam[warp];
+    const CamHot cam_c = s_cam[warp];
     // the rays of the unit's columns (a lane one) and rows (the first lanes)
     const float ray_x = __ldg(&rays[cam_c.ray_x + min(x0 + lane, W - 1)].x);
     const float ray_y = __ldg(&rays[cam_c.ray_y + min(y0 + (lane & (kUnitH - 1)), H - 1)].x);
@@ -702,6 +701,76 @@ __device__ __forceinline__ void tile_of(const TileIndex& ti, int T, int& cam, in
   int tx;
   y0 = fast_div(local, (ti.W[cam] + kTileW - 1) / kTileW, ti.div_x[cam], tx) * TH;
   x0 = tx * kTileW;
+}
+
+// ------------------------------------------------------------------ ranks and statistics
+// A slot without representative, number or weight exponent.
+#define kSlotClear make_uint4(0u, 0u, kSlotNone, (unsigned)INT_MAX)
+
+// Marks cell `id` as having its representative at pixel g: a bit of the pixel and the cell's number there
+// (over the list's confidences, which no step reads any more).  The caller counts the bits of each emit
+// block's share of the bitmap.
+__device__ __forceinline__ void mark_cell(const Tables& t, unsigned g, unsigned id) {
+  atomicOr(&t.bitmap[g >> 5], 1u << (g & 31));
+  t.cell_at[g] = id;
+}
+
+// The frame's statistics from the count step's blocks and the counters, by one block, which clears the
+// counters for the next frame (no other block of its kernel reads them).
+template <bool TOPK>
+__device__ __forceinline__ void frame_stats(const Tables& t, const OutDev& out) {
+  __shared__ unsigned long long s_l[3][kThreads / 32];
+  __shared__ unsigned s_b[6][kThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long n[3] = {0ull, 0ull, 0ull};
+  unsigned mn[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, mx[3] = {0u, 0u, 0u};
+  for (int i = threadIdx.x; i < t.n_bstats; i += kThreads) {
+    const BlockStats b = t.bstats[i];
+    n[0] += b.n_valid;
+    n[1] += b.n_gated;
+    n[2] += b.n_oor;
+    for (int k = 0; k < 3; ++k) { mn[k] = min(mn[k], b.bmin[k]); mx[k] = max(mx[k], b.bmax[k]); }
+  }
+  const unsigned nc = __ldcg(&t.cnt->n_cells);
+  if (!TOPK)                                    // cells past the output's capacity (reported): their slots
+    for (unsigned i = (unsigned)out.max_cells + threadIdx.x; i < nc && i < t.max_slots; i += kThreads)
+      *reinterpret_cast<uint4*>(t.frec + t.fused[i]) = kSlotClear;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    for (int o = 16; o > 0; o >>= 1) n[k] += __shfl_xor_sync(0xffffffffu, n[k], o);
+    mn[k] = __reduce_min_sync(0xffffffffu, mn[k]);
+    mx[k] = __reduce_max_sync(0xffffffffu, mx[k]);
+    if (lane == 0) { s_l[k][warp] = n[k]; s_b[k][warp] = mn[k]; s_b[3 + k][warp] = mx[k]; }
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int q = 1; q < kThreads / 32; ++q)
+    for (int k = 0; k < 3; ++k) {
+      n[k] += s_l[k][q];
+      mn[k] = min(mn[k], s_b[k][q]);
+      mx[k] = max(mx[k], s_b[3 + k][q]);
+    }
+  fuseflow_stats st = {};
+  st.n_valid = (int64_t)n[0];
+  st.n_gated = (int64_t)n[1];
+  st.n_out_of_range = (int64_t)n[2];
+  unsigned err = __ldcg(&t.cnt->error);
+  if ((long long)nc > out.max_cells) err |= kErrCells;
+  if (TOPK && __ldcg(&t.cnt->n_partials) > t.max_partials) err |= kErrPartials;
+  st.n_cells = (int64_t)(nc < out.max_cells ? nc : out.max_cells);
+  for (int k = 0; k < 3; ++k) {
+    st.bbox[k] = n[1] ? (float)((double)from_ordered(mn[k]) * out.unit_m) : __int_as_float(0x7f800000);
+    st.bbox[3 + k] = n[1] ? (float)((double)from_ordered(mx[k]) * out.unit_m) : __int_as_float(0xff800000);
+  }
+  st.error = (int32_t)err;
+  st.n_coarse = (int32_t)__ldcg(&t.cnt->n_coarse);
+  *out.stats = st;
+  *t.cnt = FrameCounters{};
+}
+
+// u64 -> float32 through two 32-bit conversions (at most two roundings)
+__device__ __forceinline__ float u64_to_f32(unsigned long long x) {
+  return __fmaf_rn(__uint2float_rn((unsigned)(x >> 32)), 4294967296.0f, __uint2float_rn((unsigned)x));
 }
 
 // ------------------------------------------------------------------ weigh step
@@ -931,12 +1000,13 @@ __global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64) k_weigh(const __grid_cons
   for (unsigned q = threadIdx.x; q < n; q += blockDim.x) {
     const unsigned id = s_first + q, slot = s_slot[q];
     t.frec[slot].head = id;
-    t.fused[id] = slot;                     // a number for each slot at most
     if ((long long)id < fa.out.max_cells) {
-      t.ckey[id] = s_key[q];
-      uint4* a = reinterpret_cast<uint4*>(t.acc + 8ull * id);
+      uint4* a = reinterpret_cast<uint4*>(t.rows + id);
 #pragma unroll
       for (int k = 0; k < 4; ++k) a[k] = make_uint4(0u, 0u, 0u, 0u);
+      a[4] = make_uint4((unsigned)s_key[q], (unsigned)(s_key[q] >> 32), slot, 0u);
+    } else {
+      t.fused[id] = slot;                   // past the capacity; a number for each slot at most
     }
   }
 }
@@ -954,6 +1024,7 @@ __device__ __forceinline__ unsigned long long fixed_term(float v) {
 
 // Shared memory of a warp of the sum step, in 16-byte words: 36 rows of 64 bytes, 32 cell numbers.
 constexpr int kSumWarpWords = 36 * 4 + 32 / 4;
+constexpr int kTileShares = 16;              // emit blocks that a tile counts representatives for
 
 // Eq. 11: the sums of w, w P and w RGB of each cell as exact integers at the scale 2^-(36 + m_min) of
 // its smallest weight exponent, one 64-byte row a cell {w, w frac xyz, w rgb / 256, members}, added
@@ -961,7 +1032,7 @@ constexpr int kSumWarpWords = 36 * 4 + 32 / 4;
 // then take a row each of eight successive points, a lane a term, and send one reduction of 64
 // contiguous bytes per run of points of one cell (eight lanes on a row measured 3 times faster than
 // a lane a row: the reductions of a row travel together).  Bound by L2's reductions: 64 us for 3.7 M
-// points, where 64-byte rows alone take 50 (75 G rows/s).  Weigh and sum take 185 us on 8x1280x720;
+// points, where 64-byte rows alone take 50 (75 G rows/s); with the representatives' marks 72.  Weigh and sum take 185 us on 8x1280x720;
 // one kernel that gathered each tile's cells in shared-memory tables and wrote a record per tile and
 // cell for a later walk of the cells' record lists took 211 (tables, records and their barriers: 120).
 template <typename DT, int NB, int TH>
@@ -981,6 +1052,7 @@ __global__ void k_sum(const __grid_constant__ BatchArgs<NB> args) {
   const int W = ti.W[cam], H = ti.H[cam];
   const unsigned off = (unsigned)ti.off[cam];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ unsigned s_share[kTileShares];
   uint4* const s_row = reinterpret_cast<uint4*>(smem) + warp * kSumWarpWords;
   unsigned* const s_id = reinterpret_cast<unsigned*>(s_row + 36 * 4);
   const CamHot& cc = t.bconst[cam].cam;
@@ -988,6 +1060,20 @@ __global__ void k_sum(const __grid_constant__ BatchArgs<NB> args) {
   pdl_wait();
   const TileList<WT::Units> list(t, ti, cam, off, W, H, x0, y0);
   const unsigned max_cells = (unsigned)fa.out.max_cells;
+  // representatives of the tile by emit block, from the first pixel's on; counted here before they go to
+  // the frame's counters (an update a cell took 10 us more on 8x1280x720, 170 us on 16x1024^2)
+  const unsigned share0 = (off + (unsigned)(y0 * W + x0)) / (32u * kRankWords);
+  if (threadIdx.x < kTileShares) s_share[threadIdx.x] = 0u;
+  __syncthreads();
+  // beside the tile's points, a part of the coarse entries to clear (no later step reads them)
+  {
+    const unsigned n_coarse = min(__ldcg(&t.cnt->n_coarse), t.cmask + 1u), step = (unsigned)t.n_tiles * blockDim.x;
+    for (unsigned i = (unsigned)T * blockDim.x + threadIdx.x; i < n_coarse; i += step) {
+      const unsigned cs = __ldcg(t.cused + i);
+      t.coarse[cs].key = kKeyEmpty;
+      t.coarse[cs].count = 0u;
+    }
+  }
   const int term = lane & 7, group = lane >> 3;
 #pragma unroll 1
   for (int i0 = warp * 32; i0 < list.n; i0 += (int)blockDim.x) {
@@ -998,10 +1084,10 @@ __global__ void k_sum(const __grid_constant__ BatchArgs<NB> args) {
       const unsigned at = list.at(i, unit);
       const unsigned ls = __ldcg(t.wslot + at), slot = ls & kBaseNone;
       if (slot != kBaseNone) {
-        const uint2 rec = __ldcg(reinterpret_cast<const uint2*>(&t.frec[slot].head));   // number, exponent
+        const uint4 rec = __ldcg(reinterpret_cast<const uint4*>(t.frec + slot));   // representative, number, exponent
         const unsigned e = __ldcg(t.lpix + at);
         const float z = Depth<DT>::z(__ldcg(static_cast<const DT*>(t.ldepth) + at)), mu = __ldcg(t.wmant + at);
-        const int sh = __ldcg(t.wexp + at) - (int)rec.y;
+        const int sh = __ldcg(t.wexp + at) - (int)rec.w;
         const int x = x0 + (int)(e & (kTileW - 1)), y = y0 + (int)((e & 0xffu) / kTileW) + unit * kUnitH;
         const uint8_t* p3 = col + 3u * (unsigned)(y * W + x);
         const unsigned rgb[3] = {__ldg(p3), __ldg(p3 + 1), __ldg(p3 + 2)};
@@ -1020,7 +1106,17 @@ __global__ void k_sum(const __grid_constant__ BatchArgs<NB> args) {
           v[4 + a] = fixed_term(__fmul_rn(w, __fsub_rn(__uint_as_float(0x47000000u | rgb[a]), 32768.0f)));
         }
         v[7] = 1ull;
-        if (rec.x < max_cells) id = rec.x;
+        if (rec.z < max_cells) {
+          id = rec.z;
+          const unsigned g = off + (unsigned)(y * W + x);
+          if (rec.x == ~g) {                    // the cell's representative
+            t.rows[id].mmin = (int)rec.w;       // the emit step would read slots in another order, 4 times slower
+            mark_cell(t, g, id);
+            const unsigned q = g / (32u * kRankWords) - share0;
+            if (q < kTileShares) atomicAdd(&s_share[q], 1u);
+            else atomicAdd(&t.bsum[share0 + q], 1u);
+          }
+        }
         uint4* row = s_row + (lane + (lane >> 3)) * 4;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -1038,15 +1134,17 @@ __global__ void k_sum(const __grid_constant__ BatchArgs<NB> args) {
       const unsigned next = s_id[p];
       const uint2 q = reinterpret_cast<const uint2*>(s_row + (p + group) * 4 + ((term >> 1) ^ ((p >> 1) & 3)))[term & 1];
       if (next != cur) {
-        if (cur != kSlotNone) atomicAdd(t.acc + 8ull * cur + term, sum);
+        if (cur != kSlotNone) atomicAdd(&t.rows[cur].sum[term], sum);
         cur = next;
         sum = 0ull;
       }
       sum += ((unsigned long long)q.y << 32) | q.x;
     }
-    if (cur != kSlotNone) atomicAdd(t.acc + 8ull * cur + term, sum);
+    if (cur != kSlotNone) atomicAdd(&t.rows[cur].sum[term], sum);
     __syncwarp();
   }
+  __syncthreads();
+  if (threadIdx.x < kTileShares && s_share[threadIdx.x]) atomicAdd(&t.bsum[share0 + threadIdx.x], s_share[threadIdx.x]);
 }
 
 // ------------------------------------------------------------------ assign step
@@ -1295,68 +1393,6 @@ __global__ void __launch_bounds__(AssignTile<TH>::Threads) k_assign_topk(const _
   }
 }
 
-// ------------------------------------------------------------------ reduce step
-// u64 -> float32 through two 32-bit conversions (at most two roundings)
-__device__ __forceinline__ float u64_to_f32(unsigned long long x) {
-  return __fmaf_rn(__uint2float_rn((unsigned)(x >> 32)), 4294967296.0f, __uint2float_rn((unsigned)x));
-}
-
-template <int NB>
-__global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ BatchArgs<NB> args) {
-  const Tables& t = args.f[batch_frame_y<NB>()].t;
-  const OutDev& out = args.f[batch_frame_y<NB>()].out;
-  pdl_release();
-  pdl_wait();
-  const unsigned n_cells = min(t.cnt->n_cells, t.max_slots);
-  const unsigned n_coarse = min(t.cnt->n_coarse, t.cmask + 1u);
-  const unsigned n = max(n_cells, n_coarse);
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    if (i < n_cells) {
-      const unsigned slot = t.fused[i];
-      const uint4 rec = __ldcg(reinterpret_cast<const uint4*>(t.frec + slot));
-      // ready for the next frame: no representative, no number, exponent INT_MAX
-      *reinterpret_cast<uint4*>(t.frec + slot) = make_uint4(0u, 0u, kSlotNone, (unsigned)INT_MAX);
-      if ((long long)i < out.max_cells) {
-        const int mmin = (int)rec.w;
-        const unsigned long long key = t.ckey[i];
-        const ulonglong2* row = reinterpret_cast<const ulonglong2*>(t.acc + 8ull * i);
-        unsigned long long S[8];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          const ulonglong2 v = __ldcg(row + a);
-          S[2 * a] = v.x;
-          S[2 * a + 1] = v.y;
-        }
-        CellOut c;
-        // Eq. 11 in float32: position = edge (k + S_k / S_0), colour = 256 S_c / S_0,
-        // weight = S_0 2^-(36 + mmin); each result is within a few float32 roundings
-        const int l = (int)(key >> 60);
-        const float edge = __fmul_rn(out.s0_m, pow2f(-l));
-        const float Wf = u64_to_f32(S[0]);
-        const float inv = S[0] ? __frcp_rn(Wf) : __int_as_float(0x7fc00000);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          const int ka = (int)((key >> (40 - 20 * a)) & 0xfffff) - kKeyBias;
-          c.pos[a] = __fmaf_rn(edge, (float)ka, __fmul_rn(edge, __fmul_rn(u64_to_f32(S[1 + a]), inv)));
-          c.rgb[a] = __fmul_rn(256.0f, __fmul_rn(u64_to_f32(S[4 + a]), inv));
-        }
-        c.weight = ldexpf(Wf, -kFixShift - min(mmin, 1 << 30));
-        c.count = (unsigned)S[7];
-        c.rep = ~rec.x;
-        c.pad = 0u;
-        c.key = key;
-        t.staged[i] = c;
-        atomicOr(&t.bitmap[c.rep >> 5], 1u << (c.rep & 31));
-      }
-    }
-    if (i < n_coarse) {
-      const unsigned cs = t.cused[i];
-      t.coarse[cs].key = kKeyEmpty;
-      t.coarse[cs].count = 0u;
-    }
-  }
-}
-
 // ------------------------------------------------------------------ top-k reduce
 // Sec. II.5(2) variant, per cell: merge the tiles' top-k lists (the k largest packed
 // (ordered(C) << 32) | ~g keys of the union: order-independent), then for each of the
@@ -1472,10 +1508,14 @@ __global__ void __launch_bounds__(kThreads, 3) k_reduce_topk(const __grid_consta
       cell.key = rec.key;
       if ((long long)i < out.max_cells) {
         t.staged[i] = cell;
-        if (have) atomicOr(&t.bitmap[g >> 5], 1u << (g & 31));   // g < n_px (checked above)
+        if (have) {                             // g < n_px (checked above)
+          mark_cell(t, g, i);
+          // one update for the lanes whose pixels fall into one share
+          const unsigned share = g / (32u * kRankWords), peers = __match_any_sync(__activemask(), share);
+          if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&t.bsum[share], (unsigned)__popc(peers));
+        }
       }
-      reinterpret_cast<unsigned long long*>(&t.frec[slot])[1] =
-          ((unsigned long long)(unsigned)INT_MAX << 32) | kSlotNone;
+      *reinterpret_cast<uint4*>(t.frec + slot) = kSlotClear;         // ready for the next frame
     }
     if (i < n_coarse) {
       const unsigned cs = t.cused[i];
@@ -1549,161 +1589,101 @@ __global__ void __launch_bounds__(kThreads) k_points(const RigDev* __restrict__ 
   }
 }
 
-// ------------------------------------------------------------------ scan + stats
-__device__ __forceinline__ unsigned block_excl_scan_1024(unsigned v, unsigned* s_w, unsigned& total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned x = v;
+// ------------------------------------------------------------------ emit
+// Block b of a frame takes pixels [8192 b, 8192 (b + 1)): the ranks of their representatives follow from
+// the earlier blocks' counts (one pass over at most a few thousand numbers) and the bits of the block's
+// own 256 words, which it leaves clear for the next frame; then a thread a cell, in rank order, so that
+// the output is written in order: Eq. 11 from the cell's sums, or the cell that the top-k reduce step
+// staged.  One block more writes the frame's statistics and clears the counters.  Bound by the latency of
+// the scattered row reads: 19 us for 187,000 cells, 116 us for 1.7 M; a reduce, a scan and an emit kernel
+// and a clear before the frame took 22 + 12 + 17 + 6 us and 255 + 25 + 134 + 6 us.
+template <bool TOPK, int NB>
+__global__ void __launch_bounds__(kThreads) k_emit(const __grid_constant__ BatchArgs<NB> args) {
+  static_assert(kRankWords == kThreads, "a bitmap word a thread");
+  __shared__ unsigned s_w[kThreads / 32][2];
+  __shared__ unsigned short s_px[32 * kRankWords];
+  const Tables& t = args.f[batch_frame_y<NB>()].t;
+  const OutDev& out = args.f[batch_frame_y<NB>()].out;
+  pdl_release();
+  pdl_wait();
+  const int b = (int)blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (b >= t.n_wblocks) {
+    if (b == t.n_wblocks) frame_stats<TOPK>(t, out);
+    return;
+  }
+  unsigned before = 0u;
+  for (int i = threadIdx.x; i < b; i += kThreads) before += __ldcg(t.bsum + i);
+  const long long w = (long long)b * kRankWords + threadIdx.x;
+  unsigned v = w < t.n_words ? __ldcg(t.bitmap + w) : 0u;
+  if (v) t.bitmap[w] = 0u;
+  const unsigned mine = __popc(v);
+  unsigned x = mine;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  if (lane == 31) s_w[warp] = x;
+  before = __reduce_add_sync(0xffffffffu, before);
+  if (lane == 31) {
+    s_w[warp][0] = x;
+    s_w[warp][1] = before;
+  }
   __syncthreads();
-  if (warp == 0) {
-    unsigned w = s_w[lane];
+  unsigned base = 0u, at = x - mine, total = 0u;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
-    }
-    s_w[lane] = w;
+  for (int k = 0; k < kThreads / 32; ++k) {
+    base += s_w[k][1];
+    if (k < warp) at += s_w[k][0];
+    total += s_w[k][0];
   }
+  for (; v; v &= v - 1u) s_px[at++] = (unsigned short)(threadIdx.x * 32 + __ffs(v) - 1);
   __syncthreads();
-  total = s_w[31];
-  const unsigned before = warp ? s_w[warp - 1] : 0u;
-  __syncthreads();
-  return before + x - v;
-}
-
-// Block b scans bitmap words [1024 b, 1024 b + 1024) and folds a share of the count step's
-// per-block statistics into the frame counters; the last block to finish (a fenced
-// counter, no waiting) scans the per-block sums and writes the frame statistics.
-template <int NB>
-__global__ void __launch_bounds__(1024) k_scan(const __grid_constant__ BatchArgs<NB> args) {
-  __shared__ unsigned s_w[32];
-  __shared__ unsigned long long s_l[3][32];
-  __shared__ unsigned s_b[6][32];
-  __shared__ bool s_last;
-  const Tables& t = args.f[batch_frame_y<NB>()].t;
-  const OutDev& out = args.f[batch_frame_y<NB>()].out;
-  const unsigned nblk = (unsigned)t.n_wblocks;     // this frame's blocks (the grid may be wider)
-  pdl_release();
-  pdl_wait();
-  if (blockIdx.x >= nblk) return;                  // uniform over the block
-  const long long w = (long long)blockIdx.x * 1024 + threadIdx.x;
-  const unsigned v = (w < t.n_words) ? __popc(t.bitmap[w]) : 0u;
-  unsigned total;
-  const unsigned ex = block_excl_scan_1024(v, s_w, total);
-  if (w < t.n_words) t.wprefix[w] = ex;
-  if (threadIdx.x == 0) t.bsum[blockIdx.x] = total;
-
-  // statistics of the count step's blocks [b0, b1)
-  const int per = (t.n_bstats + (int)nblk - 1) / (int)nblk;
-  const int b0 = blockIdx.x * per, b1 = min(t.n_bstats, b0 + per);
-  unsigned long long nv = 0, ng = 0, noor = 0;
-  unsigned bmin[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, bmax[3] = {0u, 0u, 0u};
-  for (int i = b0 + threadIdx.x; i < b1; i += 1024) {
-    const BlockStats b = t.bstats[i];
-    nv += b.n_valid;
-    ng += b.n_gated;
-    noor += b.n_oor;
-    for (int k = 0; k < 3; ++k) { bmin[k] = min(bmin[k], b.bmin[k]); bmax[k] = max(bmax[k], b.bmax[k]); }
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int o = 16; o > 0; o >>= 1) {
-    nv += __shfl_xor_sync(0xffffffffu, nv, o);
-    ng += __shfl_xor_sync(0xffffffffu, ng, o);
-    noor += __shfl_xor_sync(0xffffffffu, noor, o);
-  }
-  for (int k = 0; k < 3; ++k) {
-    bmin[k] = __reduce_min_sync(0xffffffffu, bmin[k]);
-    bmax[k] = __reduce_max_sync(0xffffffffu, bmax[k]);
-  }
-  if (lane == 0) {
-    s_l[0][warp] = nv; s_l[1][warp] = ng; s_l[2][warp] = noor;
-    for (int k = 0; k < 3; ++k) { s_b[k][warp] = bmin[k]; s_b[3 + k][warp] = bmax[k]; }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long a0 = 0, a1 = 0, a2 = 0;
-    unsigned mn[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, mx[3] = {0u, 0u, 0u};
-    for (int q = 0; q < 32; ++q) {
-      a0 += s_l[0][q]; a1 += s_l[1][q]; a2 += s_l[2][q];
-      for (int k = 0; k < 3; ++k) { mn[k] = min(mn[k], s_b[k][q]); mx[k] = max(mx[k], s_b[3 + k][q]); }
+  for (unsigned r = threadIdx.x; r < total; r += kThreads) {
+    const unsigned g = (unsigned)b * (32u * kRankWords) + s_px[r];
+    const unsigned id = __ldcg(t.cell_at + g);
+    const unsigned long long rank = (unsigned long long)base + r;
+    if (rank >= (unsigned long long)out.max_cells) continue;         // marked cells never exceed it
+    CellOut c;
+    if constexpr (TOPK) {
+      c = t.staged[id];
+    } else {
+      const CellRow* row = t.rows + id;
+      unsigned long long S[8];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const ulonglong2 p = __ldcg(reinterpret_cast<const ulonglong2*>(row->sum) + a);
+        S[2 * a] = p.x;
+        S[2 * a + 1] = p.y;
+      }
+      const ulonglong2 p = __ldcg(reinterpret_cast<const ulonglong2*>(&row->key));
+      const unsigned slot = (unsigned)p.y;
+      const int mmin = (int)(p.y >> 32);
+      *reinterpret_cast<uint4*>(t.frec + slot) = kSlotClear;         // ready for the next frame
+      // Eq. 11 in float32: position = edge (k + S_k / S_0), colour = 256 S_c / S_0,
+      // weight = S_0 2^-(36 + mmin); each result is within a few float32 roundings
+      const int l = (int)(p.x >> 60);
+      const float edge = __fmul_rn(out.s0_m, pow2f(-l));
+      const float Wf = u64_to_f32(S[0]);
+      const float inv = S[0] ? __frcp_rn(Wf) : __int_as_float(0x7fc00000);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int ka = (int)((p.x >> (40 - 20 * a)) & 0xfffff) - kKeyBias;
+        c.pos[a] = __fmaf_rn(edge, (float)ka, __fmul_rn(edge, __fmul_rn(u64_to_f32(S[1 + a]), inv)));
+        c.rgb[a] = __fmul_rn(256.0f, __fmul_rn(u64_to_f32(S[4 + a]), inv));
+      }
+      c.weight = ldexpf(Wf, -kFixShift - min(mmin, 1 << 30));
+      c.count = (unsigned)S[7];
+      c.key = p.x;
     }
-    if (a0) atomicAdd(&t.cnt->n_valid, a0);
-    if (a1) atomicAdd(&t.cnt->n_gated, a1);
-    if (a2) atomicAdd(&t.cnt->n_oor, a2);
-    for (int k = 0; k < 3; ++k) {
-      if (mn[k] != 0xffffffffu) atomicMax(&t.cnt->bmin_inv[k], ~mn[k]);
-      if (mx[k] != 0u) atomicMax(&t.cnt->bmax[k], mx[k]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      out.pos[3 * rank + a] = c.pos[a];
+      out.rgb[3 * rank + a] = c.rgb[a];
     }
-    __threadfence();
-    s_last = atomicAdd(&t.cnt->scan_done, 1u) == nblk - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  // last block: exclusive scan of the per-block sums, then the frame statistics
-  unsigned carry = 0;
-  for (int base = 0; base < t.n_wblocks; base += 1024) {
-    const int i = base + threadIdx.x;
-    const unsigned bv = (i < t.n_wblocks) ? __ldcg(&t.bsum[i]) : 0u;
-    unsigned tot;
-    const unsigned bex = block_excl_scan_1024(bv, s_w, tot);
-    if (i < t.n_wblocks) t.bsum[i] = carry + bex;
-    carry += tot;
-  }
-  if (threadIdx.x == 0) {
-    const FrameCounters& c = *t.cnt;
-    fuseflow_stats st = {};
-    st.n_valid = (int64_t)__ldcg(&c.n_valid);
-    st.n_gated = (int64_t)__ldcg(&c.n_gated);
-    st.n_out_of_range = (int64_t)__ldcg(&c.n_oor);
-    const unsigned nc = __ldcg(&c.n_cells);
-    unsigned err = __ldcg(&c.error);
-    if ((long long)nc > out.max_cells) err |= kErrCells;
-    if (__ldcg(&c.n_partials) > t.max_partials) err |= kErrPartials;
-    st.n_cells = (int64_t)(nc < out.max_cells ? nc : out.max_cells);
-    for (int k = 0; k < 3; ++k) {
-      const unsigned mn = ~__ldcg(&c.bmin_inv[k]), mx = __ldcg(&c.bmax[k]);
-      st.bbox[k] = st.n_gated ? (float)((double)from_ordered(mn) * out.unit_m) : __int_as_float(0x7f800000);
-      st.bbox[3 + k] = st.n_gated ? (float)((double)from_ordered(mx) * out.unit_m) : __int_as_float(0xff800000);
-    }
-    st.error = (int32_t)err;
-    st.n_coarse = (int32_t)__ldcg(&c.n_coarse);
-    *out.stats = st;
-  }
-}
-
-// ------------------------------------------------------------------ emit
-template <int NB>
-__global__ void __launch_bounds__(kThreads) k_emit(const __grid_constant__ BatchArgs<NB> args) {
-  const Tables& t = args.f[batch_frame_y<NB>()].t;
-  const OutDev& out = args.f[batch_frame_y<NB>()].out;
-  pdl_release();
-  pdl_wait();
-  const unsigned n_cells = (unsigned)min((long long)min(t.cnt->n_cells, t.max_slots), out.max_cells);
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n_cells; i += gridDim.x * blockDim.x) {
-    const CellOut c = t.staged[i];
-    const unsigned g = c.rep;
-    if ((long long)g >= t.n_words * 32) continue;          // cell without partials (overflow)
-    const unsigned w = g >> 5;
-    if (!((t.bitmap[w] >> (g & 31)) & 1u)) continue;
-    const unsigned long long rnk = (unsigned long long)t.bsum[w >> 10] + t.wprefix[w] +
-                                   __popc(t.bitmap[w] & ((1u << (g & 31)) - 1u));
-    if (rnk >= (unsigned long long)out.max_cells) continue;
-    out.pos[3 * rnk + 0] = c.pos[0];
-    out.pos[3 * rnk + 1] = c.pos[1];
-    out.pos[3 * rnk + 2] = c.pos[2];
-    out.rgb[3 * rnk + 0] = c.rgb[0];
-    out.rgb[3 * rnk + 1] = c.rgb[1];
-    out.rgb[3 * rnk + 2] = c.rgb[2];
-    out.weight[rnk] = c.weight;
-    out.count[rnk] = c.count;
-    out.rep[rnk] = g;
-    out.key[rnk] = c.key;
+    out.weight[rank] = c.weight;
+    out.count[rank] = c.count;
+    out.rep[rank] = g;
+    out.key[rank] = c.key;
   }
 }
 
@@ -2126,27 +2106,24 @@ int weigh_threads(int tiles, int th) {
 }
 
 // The assign step over the batch's tiles (TH rows a tile; the traced instantiations exist for
-// single frames only): weigh and sum, or the top-k variant's kernel.
+// single frames only): the weigh kernel, or the top-k variant's.
 template <typename DT, int NB, int TH>
 cudaError_t launch_assign(const BatchArgs<NB>& a, int n, bool top_k, bool traced, int max_k1, bool pdl,
                           cudaStream_t s) {
-  const int threads = weigh_threads(a.tile_first[n], TH);
-  const dim3 tiles(a.tile_first[n]), at(AssignTile<TH>::Threads), wt(threads);
-  if (top_k) {
-    if constexpr (NB == 1)
-      if (traced) return launch_k(pdl, k_assign_topk<DT, true, NB, TH>, tiles, at, AssignTile<TH>::Bytes, s, a);
-    return launch_k(pdl, k_assign_topk<DT, false, NB, TH>, tiles, at, AssignTile<TH>::Bytes, s, a);
-  }
-  const size_t sm = WeighTile<TH>::smem(max_k1);
-  cudaError_t e = cudaSuccess;
-  bool done = false;
+  const dim3 tiles(a.tile_first[n]), at(AssignTile<TH>::Threads), wt(weigh_threads(a.tile_first[n], TH));
+  const size_t tk = AssignTile<TH>::Bytes, sm = WeighTile<TH>::smem(max_k1);
   if constexpr (NB == 1)
-    if (traced) {
-      e = launch_k(pdl, k_weigh<DT, true, NB, TH>, tiles, wt, sm, s, a);
-      done = true;
-    }
-  if (!done) e = launch_k(pdl, k_weigh<DT, false, NB, TH>, tiles, wt, sm, s, a);
-  return e != cudaSuccess ? e : launch_k(pdl, k_sum<DT, NB, TH>, tiles, wt, 16 * kSumWarpWords * (threads / 32), s, a);
+    if (traced)
+      return top_k ? launch_k(pdl, k_assign_topk<DT, true, NB, TH>, tiles, at, tk, s, a)
+                   : launch_k(pdl, k_weigh<DT, true, NB, TH>, tiles, wt, sm, s, a);
+  return top_k ? launch_k(pdl, k_assign_topk<DT, false, NB, TH>, tiles, at, tk, s, a)
+               : launch_k(pdl, k_weigh<DT, false, NB, TH>, tiles, wt, sm, s, a);
+}
+
+template <typename DT, int NB, int TH>
+cudaError_t launch_sum(const BatchArgs<NB>& a, int n, bool pdl, cudaStream_t s) {
+  const int threads = weigh_threads(a.tile_first[n], TH);
+  return launch_k(pdl, k_sum<DT, NB, TH>, dim3(a.tile_first[n]), dim3(threads), 16 * kSumWarpWords * (threads / 32), s, a);
 }
 
 // The frame kernels over n frames (NB = 1: one frame; NB = kMaxBatch: a batch of up to
@@ -2167,8 +2144,6 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
   for (int f = 0; f < n; ++f) {
     const Geometry& geo = *fr[f].geo;
     const Tables& t = fr[f].t;
-    err = cudaMemsetAsync(t.cnt, 0, sizeof(FrameCounters) + sizeof(unsigned) * (size_t)t.n_words, s);
-    if (err != cudaSuccess) return err;
     FrameArgs& fa = a.f[f];
     fa.rig = fr[f].rig;
     fa.rays = fr[f].rays;
@@ -2212,20 +2187,23 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
     traced = traced || tr.pw || tr.omega || tr.e || tr.nview || tr.key;
   }
   const int th = g0.tiles.th;
-  if (th == 8) err = launch_assign<DT, NB, 8>(a, n, g0.top_k != 0, traced, max_k1, pdl, s);
-  else if (th == 32) err = launch_assign<DT, NB, 32>(a, n, g0.top_k != 0, traced, max_k1, pdl, s);
-  else err = launch_assign<DT, NB, 16>(a, n, g0.top_k != 0, traced, max_k1, pdl, s);
+  const bool topk = g0.top_k != 0;
+  if (th == 8) err = launch_assign<DT, NB, 8>(a, n, topk, traced, max_k1, pdl, s);
+  else if (th == 32) err = launch_assign<DT, NB, 32>(a, n, topk, traced, max_k1, pdl, s);
+  else err = launch_assign<DT, NB, 16>(a, n, topk, traced, max_k1, pdl, s);
   if (err != cudaSuccess) return err;
   mark(3);
-  if (g0.top_k) {
-    if ((err = launch_k(pdl_reduce, k_reduce_topk<DT, NB>, eb, th3, 0, s, a)) != cudaSuccess) return err;
-  } else {
-    if ((err = launch_k(pdl_reduce, k_reduce<NB>, eb, th3, 0, s, a)) != cudaSuccess) return err;
-  }
+  if (topk) err = launch_k(pdl_reduce, k_reduce_topk<DT, NB>, eb, th3, 0, s, a);
+  else if (th == 8) err = launch_sum<DT, NB, 8>(a, n, pdl_reduce, s);
+  else if (th == 32) err = launch_sum<DT, NB, 32>(a, n, pdl_reduce, s);
+  else err = launch_sum<DT, NB, 16>(a, n, pdl_reduce, s);
+  if (err != cudaSuccess) return err;
   mark(4);
-  if ((err = launch_k(pdl, k_scan<NB>, dim3(max_wblocks, n), dim3(1024), 0, s, a)) != cudaSuccess) return err;
   mark(5);
-  if ((err = launch_k(pdl, k_emit<NB>, eb, th3, 0, s, a)) != cudaSuccess) return err;
+  const dim3 rb(max_wblocks + 1, n);
+  if ((err = topk ? launch_k(pdl, k_emit<true, NB>, rb, th3, 0, s, a) : launch_k(pdl, k_emit<false, NB>, rb, th3, 0, s, a)) !=
+      cudaSuccess)
+    return err;
   mark(6);
   return cudaGetLastError();
 }

@@ -62,3 +62,24 @@ def test_float_depths_beyond_the_grid_range(oracle_mod, coarse):
 def test_sizes_around_units(oracle_mod, w, h):
     rig = S.tiny_rig(n=3, width=w, height=h, fx=40.0, fy=40.0)
     _check(oracle_mod, rig, S.random_frame(rig, seed=7), n_min=2)
+
+
+def test_static_calls_alternate_between_variants(oracle_mod):
+    """The allocation-free entry keeps its tables between calls: a top-k frame leaves nothing in
+    them that a frame of all members would read, nor the other way round."""
+    import test_zz_no_alloc as Z
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_01035_gb300 import fuseflow as F
+    dev, stream = torch.device("cuda"), torch.cuda.current_stream().cuda_stream
+    rig = S.tiny_rig(n=3, width=160, height=120, spread_deg=30.0)
+    for k, seed in ((3, 51), (0, 51), (3, 52), (0, 53)):
+        fr = S.random_frame(rig, seed=seed, flying_frac=0.01)
+        ff = F.FuseFlow(rig, max_cells=8192, top_k=k)
+        try:
+            ref = run_gpu(ff, fr, torch, with_trace=False)
+        finally:
+            ff.close()
+        st, stats, out = Z._static_call(F, rig, fr, 8192, dev, stream, top_k=k)
+        assert st == F.FUSEFLOW_OK and stats.error == 0
+        Z._check_same(ref["cells"], ref["stats"], out, int(stats.n_cells))
