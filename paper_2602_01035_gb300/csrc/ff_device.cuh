@@ -242,10 +242,13 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long k) {
   return k;
 }
 
-// First table position of coarse cell (x, y, z): rows of cells lie side by side in the table, at
-// offsets scattered by odd multipliers.
+// First table position of coarse cell (x, y, z).  The two last lines scatter the cells of a wall: without
+// them its rows lie side by side, overlap, and linear probing needs 8 to 15 probes a cell instead of 1.4 to
+// 2.1 at loads of 0.46 and 0.69 (the longest chain 250 to 550 instead of 18 to 70).
 __device__ __forceinline__ unsigned coarse_hash(int x, int y, int z) {
-  return (unsigned)x + (unsigned)y * 0x9E3779B1u + (unsigned)z * 0x85EBCA77u;
+  unsigned h = (unsigned)x * 0xC2B2AE3Du + (unsigned)y * 0x9E3779B1u + (unsigned)z * 0x85EBCA77u;
+  h = (h ^ (h >> 15)) * 0x2C1B3C6Du;
+  return h ^ (h >> 16);
 }
 
 __device__ __forceinline__ unsigned long long pack_key(int l, int kx, int ky, int kz) {

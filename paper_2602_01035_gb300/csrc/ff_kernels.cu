@@ -48,23 +48,93 @@ constexpr float kInvLn2 = 1.44269504088896340736f;
 __device__ __forceinline__ unsigned coarse_slot(unsigned long long key, unsigned cmask) {
   return coarse_hash((int)((key >> 40) & 0xfffff), (int)((key >> 20) & 0xfffff), (int)(key & 0xfffff)) & cmask;
 }
-__device__ __forceinline__ unsigned coarse_insert(const Tables& t, unsigned long long key) {
-  unsigned h = coarse_slot(key, t.cmask);
-  for (int probe = 0; probe < kMaxProbe; ++probe) {
-    // most keys are there already: a look first keeps their lines free of serialised swaps
-    unsigned long long cur = __ldcg(&t.coarse[h].key);
-    if (cur == key) return h;
-    if (cur == kKeyEmpty) cur = atomicCAS(&t.coarse[h].key, kKeyEmpty, key);
-    if (cur == kKeyEmpty) {
-      const unsigned n = atomicAdd(&t.cnt->n_coarse, 1u);
-      if (n <= t.cmask) t.cused[n] = h;
-      return h;
+// n points of coarse cell (x, y, z) (Sec. II.5(1)c) into the table; its position there.  Called by whole
+// warps, lanes without a cell (`act` false) too: the warp's new cells take their places in the list of used
+// positions with one atomic, as one each on the same counter takes about 1 ns a cell.
+__device__ __forceinline__ unsigned count_cell(const Tables& t, bool act, int x, int y, int z, unsigned n) {
+  const int lane = threadIdx.x & 31;
+  unsigned slot = kSlotNone;
+  bool fresh = false;
+  if (act) {
+    const unsigned long long key = pack_key(0, x, y, z);
+    unsigned h = coarse_slot(key, t.cmask);
+    for (int probe = 0; probe < kMaxProbe; ++probe) {
+      // most keys are there already: a look first keeps their lines free of serialised swaps
+      unsigned long long cur = __ldcg(&t.coarse[h].key);
+      if (cur == kKeyEmpty) {
+        cur = atomicCAS(&t.coarse[h].key, kKeyEmpty, key);
+        fresh = cur == kKeyEmpty;
+      }
+      if (cur == key || fresh) {
+        slot = h;
+        break;
+      }
+      h = (h + 1) & t.cmask;
     }
-    if (cur == key) return h;
-    h = (h + 1) & t.cmask;
+    if (slot != kSlotNone)
+      atomicAdd(&t.coarse[slot].count, n);
+    else
+      atomicOr(&t.cnt->error, kErrCoarseFull);
   }
-  atomicOr(&t.cnt->error, kErrCoarseFull);
-  return kSlotNone;
+  const unsigned m = __ballot_sync(0xffffffffu, fresh);
+  if (m != 0u) {
+    unsigned first = 0;
+    if (lane == 0) first = atomicAdd(&t.cnt->n_coarse, (unsigned)__popc(m));
+    first = __shfl_sync(0xffffffffu, first, 0) + (unsigned)__popc(m & ((1u << lane) - 1u));
+    if (fresh && first <= t.cmask) t.cused[first] = slot;
+  }
+  return slot;
+}
+
+// One point each of K cells a lane (key kKeyEmpty: none), for whole warps: the K places are tried together,
+// each at once with a swap.
+template <int K>
+__device__ __forceinline__ void count_points(const Tables& t, const unsigned long long (&key)[K]) {
+  unsigned h[K], pending = 0, fresh = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    h[k] = coarse_slot(key[k], t.cmask);
+    pending |= key[k] != kKeyEmpty ? 1u << k : 0u;
+  }
+#pragma unroll 1
+  for (int probe = 0; probe < kMaxProbe && pending; ++probe) {
+    unsigned long long old[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if ((pending >> k) & 1u) old[k] = atomicCAS(&t.coarse[h[k]].key, kKeyEmpty, key[k]);
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if ((pending >> k) & 1u) {
+        if (old[k] == kKeyEmpty) fresh |= 1u << k;
+        if (old[k] == kKeyEmpty || old[k] == key[k]) {
+          pending &= ~(1u << k);
+          atomicAdd(&t.coarse[h[k]].count, 1u);
+        } else {
+          h[k] = (h[k] + 1) & t.cmask;
+        }
+      }
+  }
+  if (pending) atomicOr(&t.cnt->error, kErrCoarseFull);
+  __syncwarp();
+  const int lane = threadIdx.x & 31;
+  const unsigned mine = (unsigned)__popc(fresh);
+  unsigned sum = mine;                                               // of the lanes up to this one
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(0xffffffffu, sum, o);
+    if (lane >= o) sum += v;
+  }
+  const unsigned total = __shfl_sync(0xffffffffu, sum, 31);
+  if (total == 0u) return;
+  unsigned at = 0;
+  if (lane == 0) at = atomicAdd(&t.cnt->n_coarse, total);
+  at = __shfl_sync(0xffffffffu, at, 0) + sum - mine;
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if ((fresh >> k) & 1u) {
+      if (at <= t.cmask) t.cused[at] = h[k];
+      ++at;
+    }
 }
 
 // Level and slot base (packed level << 27 | base) of an existing coarse key.
@@ -427,18 +497,11 @@ __device__ __forceinline__ float joint_weight(const RigHot& rig, int k1, float s
 }
 
 // ------------------------------------------------------------------ count step
-// n points of a coarse cell (Sec. II.5(1)c) into the global table; the cell's position there.
-__device__ __forceinline__ unsigned count_cell(const Tables& t, int x, int y, int z, unsigned n) {
-  const unsigned slot = coarse_insert(t, pack_key(0, x, y, z));
-  if (slot != kSlotNone) atomicAdd(&t.coarse[slot].count, n);
-  return slot;
-}
-
-// Position of a cell key in a warp's table of kUnitCells, inserted if new; -1 after 8 probes.
+// Position of a cell key in a warp's table of kUnitCells, inserted if new; -1 after 4 probes.
 __device__ __forceinline__ int unit_cell(unsigned* tab, unsigned key) {
   unsigned h = (key * 0x9E3779B1u) >> 26;
 #pragma unroll 1
-  for (int probe = 0; probe < 8; ++probe) {
+  for (int probe = 0; probe < 4; ++probe) {
     const unsigned cur = *static_cast<volatile unsigned*>(&tab[h]);
     if (cur == key) return (int)h;
     if (cur == 0xffffffffu) {
@@ -449,6 +512,24 @@ __device__ __forceinline__ int unit_cell(unsigned* tab, unsigned key) {
   }
   return -1;
 }
+
+// Camera and first pixel of unit u.
+__device__ __forceinline__ void unit_of(const TileIndex& ti, int u, int& cam, int& x0, int& y0) {
+  int lu = u, ux;
+  if (ti.units_per_cam) {
+    cam = fast_div(u, ti.units_per_cam, ti.div_units, lu);
+  } else {
+    cam = 0;
+    for (int lo = 0, hi = ti.n_cams - 1; lo <= hi;) {
+      const int mid = (lo + hi) >> 1;
+      if (ti.unit[mid] <= u) { cam = mid; lo = mid + 1; } else { hi = mid - 1; }
+    }
+    lu = u - ti.unit[cam];
+  }
+  y0 = fast_div(lu, (ti.W[cam] + kTileW - 1) / kTileW, ti.div_x[cam], ux) * kUnitH;
+  x0 = ux * kTileW;
+}
+constexpr unsigned kUnnumbered = 0x80000000u;   // on a unit's count while points of it are left
 
 // A warp takes units of 32 columns by 8 rows with no block-wide step in between: gate (Eq. 9) and
 // compaction of the gated pixels, a column a lane; then a gated pixel a lane, full warps: back-projection
@@ -477,6 +558,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ B
   __shared__ unsigned char s_occ[kThreads / 32][kUnitCells];
   __shared__ unsigned s_key[kThreads / 32][kUnitCells], s_cnt[kThreads / 32][kUnitCells];
   static_assert(kUnitCells == 64, "two positions a lane, 6-bit hash");
+  constexpr int kMissed = 4;                                         // points without a number tried together by a lane
   __shared__ unsigned s_red[kThreads / 32][9];
   const float tau = fa.hot.tau, inv_s0u = fa.hot.inv_s0u;
   const bool use_conf = fa.hot.use_conf != 0;
@@ -485,24 +567,15 @@ __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ B
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float qnan = __int_as_float(0x7fffffff), inf = __int_as_float(0x7f800000);
   unsigned nv = 0, ng = 0, noor = 0;
+  bool any_rest = false;
   float fmn[3] = {inf, inf, inf}, fmx[3] = {-inf, -inf, -inf};
   const int u0 = local * fa.count_chunks * (kThreads / 32);
   const int u1 = min(u0 + fa.count_chunks * (kThreads / 32), t.n_units);
 #pragma unroll 1
   for (int u = u0 + warp; u < u1; u += kThreads / 32) {
-    int cam, lu = u, ux;
-    if (ti.units_per_cam) {
-      cam = fast_div(u, ti.units_per_cam, ti.div_units, lu);
-    } else {
-      cam = 0;
-      for (int lo = 0, hi = ti.n_cams - 1; lo <= hi;) {
-        const int mid = (lo + hi) >> 1;
-        if (ti.unit[mid] <= u) { cam = mid; lo = mid + 1; } else { hi = mid - 1; }
-      }
-      lu = u - ti.unit[cam];
-    }
+    int cam, x0, y0;
+    unit_of(ti, u, cam, x0, y0);
     const int W = ti.W[cam], H = ti.H[cam];
-    const int y0 = fast_div(lu, (W + kTileW - 1) / kTileW, ti.div_x[cam], ux) * kUnitH, x0 = ux * kTileW;
     int n = 0;
     {
       const DT* __restrict__ dep = static_cast<const DT*>(fp.depth[cam]);
@@ -612,20 +685,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ B
       __syncwarp();
     }
     ng += lane == 0 ? (unsigned)n : 0u;
-    if (__any_sync(0xffffffffu, missed)) {                           // far-flung points, or a full table
-#pragma unroll 1
-      for (int i0 = 0; i0 < n; i0 += 32) {
-        const int i = i0 + lane;
-        float P[3], r[3];
-        int c[3];
-        point(i, i < n ? Depth<DT>::z(s_d[warp][i]) : qnan, P);
-        const bool inr = grid_coords(fa.hot, P, r, c);
-        if (i < n && (lp[i] >> 8) == kNoCellNumber) {                // the lane's own store above
-          if (inr) count_cell(t, c[0], c[1], c[2], 1u);
-          else ++noor;
-        }
-      }
-    }
     // the unit's cells into the global table, one a lane
     const unsigned o0 = __ballot_sync(0xffffffffu, s_key[warp][lane] != 0xffffffffu);
     const unsigned o1 = __ballot_sync(0xffffffffu, s_key[warp][lane + 32] != 0xffffffffu);
@@ -634,15 +693,69 @@ __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ B
     if ((o1 >> lane) & 1u) s_occ[warp][__popc(o0) + __popc(o1 & below)] = (unsigned char)(lane + 32);
     __syncwarp();
     const int cells = __popc(o0) + __popc(o1);
-    for (int q = lane; q < cells; q += 32) {
-      const int h = s_occ[warp][q];
+    for (int q = lane; q - lane < cells; q += 32) {
+      const bool act = q < cells;
+      const int h = act ? s_occ[warp][q] : 0;
       const unsigned key = s_key[warp][h];
-      t.lcell[(long long)u * kUnitCells + h] =
-          count_cell(t, ref[0] - kGridBits + (int)(key >> 20), ref[1] - kGridBits + (int)((key >> 10) & 1023u),
+      const unsigned slot =
+          count_cell(t, act, ref[0] - kGridBits + (int)(key >> 20), ref[1] - kGridBits + (int)((key >> 10) & 1023u),
                      ref[2] - kGridBits + (int)(key & 1023u), s_cnt[warp][h]);
+      if (act) t.lcell[(long long)u * kUnitCells + h] = slot;
     }
-    if (lane == 0) t.lcount[u] = (unsigned)n;
+    const bool rest = __any_sync(0xffffffffu, missed);
+    if (lane == 0) t.lcount[u] = (unsigned)n | (rest ? kUnnumbered : 0u);
+    any_rest = any_rest || rest;
     __syncwarp();                                                    // the staged pixels are free again
+  }
+  // The points without a number (far-flung ones, and of units with more cells than the table takes) go to the
+  // global table by themselves, from the lists.  After the other units: inside their loop this costs its
+  // registers, 3 to 9 % of the step.
+  if (any_rest) {                                                    // uniform over the warp
+    __syncwarp();
+#pragma unroll 1
+    for (int u = u0 + warp; u < u1; u += kThreads / 32) {
+      const unsigned marked = __ldcg(t.lcount + u);
+      if (!(marked & kUnnumbered)) continue;
+      const int n = (int)(marked & ~kUnnumbered);
+      int cam, x0, y0;
+      unit_of(ti, u, cam, x0, y0);
+      const int W = ti.W[cam], H = ti.H[cam];
+      const long long at = unit_list(ti.off[cam], W, H, x0, y0);
+      const DT* ld = static_cast<const DT*>(t.ldepth) + at;
+      const unsigned short* lp = t.lpix + at;
+      if (lane < 4) reinterpret_cast<float4*>(&s_cam[warp])[lane] = __ldg(reinterpret_cast<const float4*>(t.bconst + cam) + lane);
+      __syncwarp();
+      const CamHot& cam_c = s_cam[warp];
+#pragma unroll 1
+      for (int i0 = 0; i0 < n; i0 += 32 * kMissed) {
+        unsigned long long key[kMissed];
+        unsigned e[kMissed];
+        DT d[kMissed];
+#pragma unroll
+        for (int k = 0; k < kMissed; ++k) {                          // the lane's own stores above
+          const int i = i0 + 32 * k + lane;
+          e[k] = i < n ? __ldcg(lp + i) : 0u;
+          d[k] = i < n ? __ldcg(ld + i) : (DT)0;
+        }
+#pragma unroll
+        for (int k = 0; k < kMissed; ++k) {
+          key[k] = kKeyEmpty;
+          if ((e[k] >> 8) == kNoCellNumber) {
+            float P[3], r[3];
+            int c[3];
+            world_point(cam_c, Depth<DT>::z(d[k]), __ldg(&rays[cam_c.ray_x + x0 + (int)(e[k] & (kTileW - 1))].x),
+                        __ldg(&rays[cam_c.ray_y + y0 + (int)((e[k] & 0xffu) / kTileW)].x), P);
+            if (grid_coords(fa.hot, P, r, c))
+              key[k] = pack_key(0, c[0], c[1], c[2]);
+            else
+              ++noor;
+          }
+        }
+        count_points<kMissed>(t, key);
+      }
+      __syncwarp();
+      if (lane == 0) t.lcount[u] = (unsigned)n;
+    }
   }
   // per-block pixel counts and extent
   unsigned vals[9] = {nv, ng, noor};
