@@ -939,20 +939,22 @@ struct TileList {
   }
 };
 
-// Levels and first slots of the units' numbered coarse cells (Sec. II.5(1)d), a number a thread.  (A
-// number that the unit does not use still names some position of the coarse table, an earlier frame's.)
+// Levels and first slots of the units' numbered coarse cells (Sec. II.5(1)d).  (A number that the unit
+// does not use still names some position of the coarse table, an earlier frame's.)
 template <int kUnits>
 __device__ __forceinline__ void load_cell_levels(const Tables& t, const TileIndex& ti, const TileList<kUnits>& list, int cam,
                                                  int W, int x0, int y0, unsigned* s_lb) {
   const int tiles_x = (W + kTileW - 1) / kTileW, u0 = ti.unit[cam] + (y0 >> 3) * tiles_x + (x0 >> 5);
-  const int k = (int)threadIdx.x / kUnitCells, c = (int)threadIdx.x & (kUnitCells - 1);
-  bool listed = false;                            // the unit has a list, and so its numbers
+  for (int i = threadIdx.x; i < kUnits * kUnitCells; i += (int)blockDim.x) {
+    const int k = i / kUnitCells;
+    bool listed = false;                          // the unit has a list, and so its numbers
 #pragma unroll
-  for (int q = 0; q < kUnits; ++q)
-    if (k == q) listed = list.end[q] > (q ? list.end[q > 0 ? q - 1 : 0] : 0);
-  if (listed) {
-    const unsigned slot = __ldcg(t.lcell + (long long)(u0 + k * tiles_x) * kUnitCells + c);
-    s_lb[threadIdx.x] = slot == kSlotNone ? kBaseNone : __ldcg(&t.coarse[slot].lvbase);
+    for (int q = 0; q < kUnits; ++q)
+      if (k == q) listed = list.end[q] > (q ? list.end[q > 0 ? q - 1 : 0] : 0);
+    if (listed) {
+      const unsigned slot = __ldcg(t.lcell + (long long)(u0 + k * tiles_x) * kUnitCells + (i & (kUnitCells - 1)));
+      s_lb[i] = slot == kSlotNone ? kBaseNone : __ldcg(&t.coarse[slot].lvbase);
+    }
   }
 }
 
@@ -1048,7 +1050,6 @@ __global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64) k_weigh(const __grid_cons
   pdl_wait();
   const TileList<WT::Units> list(t, ti, cam, off, W, H, x0, y0);
   if (list.n == 0) return;                  // uniform over the block
-  static_assert(WT::Units * kUnitCells <= WT::Threads, "a thread takes one numbered cell");
   load_cell_levels<WT::Units>(t, ti, list, cam, W, x0, y0, s_lb);
   cp_async_wait();
   __syncthreads();
