@@ -1511,28 +1511,49 @@ __global__ void __launch_bounds__(AssignTile<TH>::Threads) k_assign_topk(const _
 // Sec. II.5(2) variant, per cell: merge the tiles' top-k lists (the k largest packed
 // (ordered(C) << 32) | ~g keys of the union: order-independent), then for each of the
 // cell's k representatives recompute the world point (Eq. 8, the same float32 sequence as
-// the other steps), its consistency over its camera's K-1 views (Eq. 4-7, double-float,
-// global pair rays) and omega = C V (Eq. 10), and fuse them (Eq. 11, normalised, weights
-// scaled by the largest).  Members are counted over the whole cell; the representative is
-// the cell's top member.
+// the other steps), its consistency over its camera's K-1 views (Eq. 4-7, global pair rays)
+// and omega = C V (Eq. 10), and fuse them (Eq. 11, normalised, weights scaled by the
+// largest).  Members are counted over the whole cell; the representative is the cell's top
+// member.
+// A block merges the lists of 128 / k cells, a thread a cell, then weighs their representatives, a thread
+// each, and fuses them, a thread a cell again.  Bound by the latency of the lists, of the scattered samples
+// and between the block's steps (33 % of the issue slots).  k = 3, 187,000 cells of 8x1280x720: 73 us; a
+// thread a cell throughout, its k representatives one after another, 84 us unrolled and 78 us rolled; k = 6
+// on 4x187x146: 12 us instead of 29.  10 blocks an SM (48 registers, spills) 79 us, 6 blocks 89 us; blocks of
+// 64 or 32 threads 76 us.
+constexpr int kTopThreads = 128;
 template <typename DT, int NB>
-__global__ void __launch_bounds__(kThreads, 3) k_reduce_topk(const __grid_constant__ BatchArgs<NB> args) {
+__global__ void __launch_bounds__(kTopThreads, 8) k_reduce_topk(const __grid_constant__ BatchArgs<NB> args) {
   const FrameArgs& fa = args.f[batch_frame_y<NB>()];
   const RigDev* __restrict__ rigp = fa.rig;
   const float2* __restrict__ rays = fa.rays;
   const FramePtrs& fp = fa.fp;
   const Tables& t = fa.t;
   const OutDev& out = fa.out;
+  __shared__ unsigned long long s_key[kTopThreads];                  // a cell's k keys side by side, 0: none
+  __shared__ float s_mu[kTopThreads], s_val[6][kTopThreads];         // mantissa; world point and colour
+  __shared__ int s_mx[kTopThreads];                                  // exponent of the weight
   pdl_release();
   pdl_wait();
   const RigDev& rig = *rigp;
   const unsigned n_cells = min(t.cnt->n_cells, t.max_slots);
   const unsigned n_coarse = min(t.cnt->n_coarse, t.cmask + 1u);
   const unsigned n_part = min(t.cnt->n_partials, t.max_partials);
-  const unsigned n = max(n_cells, n_coarse);
   const int K = rig.top_k;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    if (i < n_cells) {
+  const unsigned per = (unsigned)(kTopThreads / K);
+  for (unsigned i = blockIdx.x * kTopThreads + threadIdx.x; i < n_coarse; i += gridDim.x * kTopThreads) {
+    const unsigned cs = t.cused[i];
+    t.coarse[cs].key = kKeyEmpty;
+    t.coarse[cs].count = 0u;
+  }
+#pragma unroll 1
+  for (unsigned c0 = blockIdx.x * per; c0 < n_cells; c0 += gridDim.x * per) {
+    const unsigned i = c0 + threadIdx.x;
+    const bool mine = threadIdx.x < per && i < n_cells;
+    CellOut cell;
+    s_key[threadIdx.x] = 0ull;
+    __syncthreads();
+    if (mine) {
       const unsigned slot = t.fused[i];
       const SlotRec rec = t.frec[slot];
       unsigned long long top[kMaxTopK];
@@ -1556,70 +1577,81 @@ __global__ void __launch_bounds__(kThreads, 3) k_reduce_topk(const __grid_consta
         p = P.next;
       }
       if (steps > n_part) atomicOr(&t.cnt->error, kErrList);
-      // weights and world points of the representatives
-      float mu[kMaxTopK], P3[kMaxTopK][3], col[kMaxTopK][3];
-      int mx[kMaxTopK];
-      int mmin = INT_MAX, nr = 0;
 #pragma unroll
-      for (int q = 0; q < kMaxTopK; ++q) {      // sorted: the filled entries come first
-        mu[q] = 0.0f;
-        mx[q] = 0;
-        if (q >= K || !top[q]) continue;
-        const unsigned g = ~(unsigned)(top[q] & 0xffffffffull);
-        if ((long long)g >= rig.n_px) {         // not a pixel: a corrupted list (reported)
-          atomicOr(&t.cnt->error, kErrList);
-          top[q] = 0ull;
-          continue;
-        }
+      for (int q = 0; q < kMaxTopK; ++q)
+        if (q < K) s_key[threadIdx.x * K + q] = top[q];
+      cell.count = count;
+      cell.key = rec.key;
+      *reinterpret_cast<uint4*>(t.frec + slot) = kSlotClear;         // ready for the next frame
+    }
+    __syncthreads();
+    if (s_key[threadIdx.x]) {                   // weight and world point of a representative
+      const unsigned g = ~(unsigned)(s_key[threadIdx.x] & 0xffffffffull);
+      if ((long long)g >= rig.n_px) {           // not a pixel: a corrupted list (reported)
+        atomicOr(&t.cnt->error, kErrList);
+        s_key[threadIdx.x] = 0ull;
+      } else {
         int cam = 0;
-        for (int c = 1; c < rig.n_cams; ++c)
-          if ((long long)g >= rig.cam[c].off) cam = c;
-        const CamDev& C = rig.cam[cam];
-        const long long li = (long long)g - C.off;
-        const int y = (int)(li / C.W), x = (int)(li - (long long)y * C.W);
+        for (int lo = 0, hi = fa.ti.n_cams - 1; lo <= hi;) {
+          const int mid = (lo + hi) >> 1;
+          if (fa.ti.off[mid] <= (long long)g) { cam = mid; lo = mid + 1; } else { hi = mid - 1; }
+        }
+        const int W = fa.ti.W[cam];
+        const unsigned li = g - (unsigned)fa.ti.off[cam];
+        const int y = (int)(li / (unsigned)W), x = (int)(li - (unsigned)y * (unsigned)W);
         const float z = Depth<DT>::z(static_cast<const DT*>(fp.depth[cam])[li]);
         const float c = fp.conf[cam][li];
-        const uint8_t* px = fp.rgb[cam] + 3 * li;
-        world_point(C, z, __ldg(&rays[C.ray_x + x].x), __ldg(&rays[C.ray_y + y].x), P3[q]);
-        float sh = 0.0f, sl = 0.0f;
-        int nview = 0;
+        const uint8_t* px = fp.rgb[cam] + 3 * (long long)li;
+        const BlockConst* bc = t.bconst + cam;
+        float P[3], mu, sh = 0.0f, sl = 0.0f;
+        int mx, nview = 0;
+        s_val[3][threadIdx.x] = (float)px[0];
+        s_val[4][threadIdx.x] = (float)px[1];
+        s_val[5][threadIdx.x] = (float)px[2];
+        world_point(bc->cam, z, __ldg(&rays[bc->cam.ray_x + x].x), __ldg(&rays[bc->cam.ray_y + y].x), P);
         if (fa.hot.use_cons && rig.k1 > 0)
-          residual_sum<DT>(t.bconst + cam, t, cam, rig.k1, GlobalPairRays(t.pray + fa.ti.pray[cam], C.W, rig.k1, x, y),
+          residual_sum<DT>(bc, t, cam, rig.k1, GlobalPairRays(t.pray + fa.ti.pray[cam], W, rig.k1, x, y),
                            rigp, fa.hot, rays, fp, z, x, y, sh, sl, nview);
-        joint_weight(fa.hot, rig.k1, sh, sl, c, mu[q], mx[q]);
-        mmin = min(mmin, mx[q]);
-        col[q][0] = px[0];
-        col[q][1] = px[1];
-        col[q][2] = px[2];
-        ++nr;
-      }
-      CellOut cell;
-      float sw = 0.0f, sp[3] = {0.0f, 0.0f, 0.0f}, sc[3] = {0.0f, 0.0f, 0.0f};
+        joint_weight(fa.hot, rig.k1, sh, sl, c, mu, mx);
+        s_mu[threadIdx.x] = mu;
+        s_mx[threadIdx.x] = mx;
 #pragma unroll
-      for (int q = 0; q < kMaxTopK; ++q) {      // Eq. 11, weights relative to the largest
-        if (q >= nr) continue;
-        const int sh = mx[q] - mmin;
-        const float w = sh > 126 ? 0.0f : __fmul_rn(mu[q], pow2f(-sh));
+        for (int a = 0; a < 3; ++a) s_val[a][threadIdx.x] = P[a];
+      }
+    }
+    __syncthreads();
+    if (mine) {
+      const int e0 = (int)threadIdx.x * K;
+      int mmin = INT_MAX;
+      bool any = false;
+      for (int q = 0; q < K; ++q)
+        if (s_key[e0 + q]) {
+          mmin = min(mmin, s_mx[e0 + q]);
+          any = true;
+        }
+      float sw = 0.0f, sp[3] = {0.0f, 0.0f, 0.0f}, sc[3] = {0.0f, 0.0f, 0.0f};
+      for (int q = 0; q < K; ++q) {             // Eq. 11, weights relative to the largest
+        if (!s_key[e0 + q]) continue;
+        const int sh = s_mx[e0 + q] - mmin;
+        const float w = sh > 126 ? 0.0f : __fmul_rn(s_mu[e0 + q], pow2f(-sh));
         sw = __fadd_rn(sw, w);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          sp[a] = __fmaf_rn(w, P3[q][a], sp[a]);
-          sc[a] = __fmaf_rn(w, col[q][a], sc[a]);
+          sp[a] = __fmaf_rn(w, s_val[a][e0 + q], sp[a]);
+          sc[a] = __fmaf_rn(w, s_val[3 + a][e0 + q], sc[a]);
         }
       }
-      const float inv = nr ? __frcp_rn(sw) : __int_as_float(0x7fc00000);
+      const float inv = any ? __frcp_rn(sw) : __int_as_float(0x7fc00000);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         cell.pos[a] = __fmul_rn(__fmul_rn(sp[a], inv), out.unit_f);
         cell.rgb[a] = __fmul_rn(sc[a], inv);
       }
-      cell.weight = nr ? ldexpf(sw, -min(mmin, 1 << 30)) : 0.0f;
-      cell.count = count;
-      const bool have = nr > 0 && top[0] != 0ull;
-      const unsigned g = have ? ~(unsigned)(top[0] & 0xffffffffull) : 0xffffffffu;
+      cell.weight = any ? ldexpf(sw, -min(mmin, 1 << 30)) : 0.0f;
+      const bool have = s_key[e0] != 0ull;
+      const unsigned g = have ? ~(unsigned)(s_key[e0] & 0xffffffffull) : 0xffffffffu;
       cell.rep = g;
       cell.pad = 0u;
-      cell.key = rec.key;
       if ((long long)i < out.max_cells) {
         t.staged[i] = cell;
         if (have) {                             // g < n_px (checked above)
@@ -1629,13 +1661,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_reduce_topk(const __grid_consta
           if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&t.bsum[share], (unsigned)__popc(peers));
         }
       }
-      *reinterpret_cast<uint4*>(t.frec + slot) = kSlotClear;         // ready for the next frame
     }
-    if (i < n_coarse) {
-      const unsigned cs = t.cused[i];
-      t.coarse[cs].key = kKeyEmpty;
-      t.coarse[cs].count = 0u;
-    }
+    __syncthreads();                            // the keys are free again
   }
 }
 
@@ -2400,7 +2427,7 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
   else err = launch_assign<DT, NB, 16>(a, n, topk, traced, max_k1, pdl, s);
   if (err != cudaSuccess) return err;
   mark(3);
-  if (topk) err = launch_k(pdl_reduce, k_reduce_topk<DT, NB>, eb, th3, 0, s, a);
+  if (topk) err = launch_k(pdl_reduce, k_reduce_topk<DT, NB>, dim3(2 * emit, n), dim3(kTopThreads), 0, s, a);
   else if (th == 8) err = launch_sum<DT, NB, 8>(a, n, pdl_reduce, s);
   else if (th == 32) err = launch_sum<DT, NB, 32>(a, n, pdl_reduce, s);
   else err = launch_sum<DT, NB, 16>(a, n, pdl_reduce, s);
