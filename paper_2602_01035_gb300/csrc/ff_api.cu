@@ -914,21 +914,27 @@ int fuseflow_mc_error(fuseflow_ctx* ctx, const float* pos, int64_t n_points,
   const int blocks = ffl::mc_blocks(n_points);
   if (!small_buffers(ctx)) return FUSEFLOW_ERR_OUT_OF_MEMORY;
   double* bsum = static_cast<double*>(ctx->d_mc);
-  long long* bcnt = reinterpret_cast<long long*>(bsum + 1024);
+  long long* bcnt = reinterpret_cast<long long*>(bsum + blocks);       // side by side: one copy
   FramePtrs fp{};
   for (int i = 0; i < ctx->n_cams; ++i) fp.depth[i] = depth[i];
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  std::vector<double> hs(blocks);
-  std::vector<long long> hc(blocks);
+  alignas(double) char h[kMcBytes];
+  const size_t bytes = blocks * (sizeof(double) + sizeof(long long));
   if (launch_mc(ctx->d_rig, fp, ctx->params.depth_format == FUSEFLOW_DEPTH_F32, pos, n_points,
                 ctx->params.depth_scale, occlusion_m, err_m, n_visible, bsum, bcnt, s) != cudaSuccess ||
-      cudaMemcpyAsync(hs.data(), bsum, sizeof(double) * blocks, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaMemcpyAsync(hc.data(), bcnt, sizeof(long long) * blocks, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaMemcpyAsync(h, bsum, bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return FUSEFLOW_ERR_CUDA;
   double sum = 0.0;
   long long cnt = 0;
-  for (int b = 0; b < blocks; ++b) { sum += hs[b]; cnt += hc[b]; }
+  for (int b = 0; b < blocks; ++b) {
+    double bs;
+    long long bc;
+    std::memcpy(&bs, h + sizeof(double) * b, sizeof bs);
+    std::memcpy(&bc, h + sizeof(double) * blocks + sizeof(long long) * b, sizeof bc);
+    sum += bs;
+    cnt += bc;
+  }
   *n_used = cnt;
   *mc_m = cnt ? sum / (double)cnt * ctx->params.depth_scale : std::nan("");
   return FUSEFLOW_OK;
