@@ -541,7 +541,15 @@ constexpr unsigned kUnnumbered = 0x80000000u;   // on a unit's count while point
 // blocks with a table of 2048 cells and runs of equal cells merged across the warp took 59 us.  Finding a
 // unit's cells one after another as the smallest key left took 49 us there, but 236 instead of 154 us
 // where units hold many cells (16x1024^2).
-template <typename DT, int NB>
+constexpr int kCountFew = 2 * 4 * 152;   // blocks: 4 a multiprocessor at once
+
+// FEW: frames of no more units than the chip takes at once or twice, where the step is as long as a crowded
+// unit's chain of probes.  There a unit whose first 32 points have more than 14 cells puts no more into its
+// table, and 8 of its points instead of 4 are under way together: frames of 5x326x319 in a room 94 -> 85 us,
+// 8x248x228 95 -> 87 us (limits of 10 and 20 cells: 87 and 87).  With the test in it the loop takes 3 to 5 %
+// longer in large frames (51.4 us instead of 49.6 at 8x1280x720, 169 instead of 161 at 16x1024x1024), which
+// go without.
+template <typename DT, int NB, bool FEW>
 __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ BatchArgs<NB> args) {
   int local;
   const FrameArgs& fa = args.f[batch_frame<NB>(args.count_first, args.n, (int)blockIdx.x, local)];
@@ -558,7 +566,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ B
   __shared__ unsigned char s_occ[kThreads / 32][kUnitCells];
   __shared__ unsigned s_key[kThreads / 32][kUnitCells], s_cnt[kThreads / 32][kUnitCells];
   static_assert(kUnitCells == 64, "two positions a lane, 6-bit hash");
-  constexpr int kMissed = 4;                                         // points without a number tried together by a lane
+  constexpr int kMissed = FEW ? 8 : 4;                                         // points without a number tried together by a lane
   __shared__ unsigned s_red[kThreads / 32][9];
   const float tau = fa.hot.tau, inv_s0u = fa.hot.inv_s0u;
   const bool use_conf = fa.hot.use_conf != 0;
@@ -647,6 +655,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ B
     DT* __restrict__ ld = static_cast<DT*>(t.ldepth) + at;
     float* __restrict__ lc = t.lconf + at;
     unsigned short* __restrict__ lp = t.lpix + at;
+    bool sparse = false;                                             // hardly two points in a cell
     bool missed = false;                                             // a point without a number
 #pragma unroll 1
     for (int i0 = 0; i0 < n; i0 += 32) {
@@ -672,9 +681,16 @@ __global__ void __launch_bounds__(kThreads, 4) k_count(const __grid_constant__ B
           if (number >= 0) s_cnt[warp][number] += (unsigned)min(32, n - i0);
         }
         number = __shfl_sync(0xffffffffu, number, 0);
-      } else if (key != 0xffffffffu) {
-        number = unit_cell(s_key[warp], key);
-        if (number >= 0) atomicAdd(&s_cnt[warp][number], 1u);
+      } else {
+        if (key != 0xffffffffu && !(FEW && sparse)) {
+          number = unit_cell(s_key[warp], key);
+          if (number >= 0) atomicAdd(&s_cnt[warp][number], 1u);
+        }
+        if (FEW && i0 == 0) {
+          __syncwarp();
+          sparse = __popc(__ballot_sync(0xffffffffu, s_key[warp][lane] != 0xffffffffu)) +
+                       __popc(__ballot_sync(0xffffffffu, s_key[warp][lane + 32] != 0xffffffffu)) > 14;
+        }
       }
       if (act) {
         missed = missed || number < 0;
@@ -2411,7 +2427,9 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
   const bool pdl = pdl_level >= 1 && ev == nullptr;
   const bool pdl_reduce = pdl_level >= 2 && ev == nullptr;
   const dim3 eb(emit, n), th3(kThreads);
-  if ((err = launch_k(false, k_count<DT, NB>, dim3(a.count_first[n]), th3, 0, s, a)) != cudaSuccess ||
+  const bool few = a.count_first[n] <= kCountFew;
+  if ((err = few ? launch_k(false, k_count<DT, NB, true>, dim3(a.count_first[n]), th3, 0, s, a)
+                 : launch_k(false, k_count<DT, NB, false>, dim3(a.count_first[n]), th3, 0, s, a)) != cudaSuccess ||
       (err = launch_k(pdl, k_levels<NB>, eb, th3, 0, s, a)) != cudaSuccess)
     return err;
   mark(2);

@@ -83,3 +83,16 @@ def test_static_calls_alternate_between_variants(oracle_mod):
         st, stats, out = Z._static_call(F, rig, fr, 8192, dev, stream, top_k=k)
         assert st == F.FUSEFLOW_OK and stats.error == 0
         Z._check_same(ref["cells"], ref["stats"], out, int(stats.n_cells))
+
+
+def test_crowded_units_in_few_and_many_blocks():
+    """Units of nearly 256 coarse cells: one frame alone takes the count step of few units, eight
+    in a batch that of many.  The clouds are the same to the bit (no result depends on the order
+    in which cells are found)."""
+    from test_gpu_batch import _batch_vs_plain
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_01035_gb300 import fuseflow
+    rig = S.tiny_rig(n=2, width=640, height=512, fx=600.0, fy=600.0)
+    frames = [(rig, _scattered(rig, 20 + i, 500, 40000)) for i in range(8)]
+    _batch_vs_plain(fuseflow, frames, coarse_cell_m=0.32, max_level=2, n_min=2, max_cells=700000)
