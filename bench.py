@@ -27,7 +27,7 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "depth px/s and frames/s at 8x1280x720 views; p50/p99 latency, served vs plain"
-KERNELS_PER_FRAME = 6      # count, levels, assign, reduce, scan, emit
+KERNELS_PER_FRAME = 5      # count, levels, weigh, sum, emit (top-k: assign and reduce in place of weigh and sum)
 CELL_OUT_BYTES = 44        # pos 12 + rgb 12 + weight 4 + count 4 + rep 4 + key 8
 SERVE_MAX_SLOTS = 2        # frames of one served rig in flight at most (slots asked per rig)
 
@@ -279,7 +279,7 @@ def run_ours(args, rank, world, local_rank):
     fps = job_rate(args.steps * FPS, world, ms)
 
     # ------------------------------------------------------------ recorded fuse calls
-    # one CUDA graph per pool frame (fuseflow_graph_*: the memset and six kernels of a frame
+    # one CUDA graph per pool frame (fuseflow_graph_*: the five kernels of a frame
     # in one launch), replayed in the plain path's order on the same stream
     graphs = [ff.graph(t[0], t[1], t[2]) for t in dtensors]
 
