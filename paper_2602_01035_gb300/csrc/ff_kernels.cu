@@ -471,7 +471,10 @@ __device__ __forceinline__ void residual_sum(const BlockConst* bc, const Tables&
 
 // Eq. 7 and 10 from the residual sum (sh, sl): omega = C' exp(-e) = mu 2^-m with
 // e = m ln 2 + f, f in [0, ln 2), so that mu never underflows (C' = C, or 1 without the
-// confidence term).  Returns e (high part) for traces.
+// confidence term).  A residual beyond float32 (a view's sample near the format's largest value)
+// leaves e infinite or not a number; its weight is 0 at an exponent above every other, so that it
+// adds nothing to a sum and does not set the sum's scale.  Returns e (high part) for traces.
+constexpr int kFarExponent = 1500000000;   // other exponents are at most 1e9 / ln 2
 __device__ __forceinline__ float joint_weight(const RigHot& rig, int k1, float sh, float sl,
                                               float c, float& mu, int& m) {
   float eh = 0.0f, el = 0.0f;
@@ -493,6 +496,11 @@ __device__ __forceinline__ float joint_weight(const RigHot& rig, int k1, float s
   }
   const float base = rig.use_conf ? c : 1.0f;                          // Eq. 10
   mu = __fmul_rn(__fmul_rn(base, expf(-fh)), __fsub_rn(1.0f, fl));
+  if (mu != mu) {
+    mu = 0.0f;
+    m = kFarExponent;
+    eh = __int_as_float(0x7f800000);
+  }
   return eh;
 }
 

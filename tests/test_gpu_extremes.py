@@ -1,0 +1,65 @@
+"""Values at the ends of the accepted ranges, against the oracle at the parity tolerances:
+depth samples so far away that a residual leaves float32."""
+import numpy as np
+import pytest
+
+from paper_2602_01035_gb300 import scenes as S
+from parity import compare, run_gpu
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def F():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_01035_gb300 import fuseflow
+    fuseflow.load()
+    return fuseflow
+
+
+def _fuse(F, rig, fr, with_trace=False, **params):
+    ff = F.FuseFlow(rig, **params)
+    try:
+        gpu = run_gpu(ff, fr, torch, with_trace=with_trace)
+    finally:
+        ff.close()
+    assert gpu["status"] == F.FUSEFLOW_OK, gpu["stats"]
+    return gpu
+
+
+def _with_sentinels(seed):
+    """A rendered float32 frame in which 2 % of the samples are the largest finite float32, as
+    sensors mark "no return"; they are not confident, so that only other cameras' points see them."""
+    rig = S.tiny_rig(n=4, width=96, height=64, depth_format="f32", depth_scale=1.0, spread_deg=25.0)
+    fr = S.random_frame(rig, seed=seed, zero_frac=0.02)
+    rng = np.random.default_rng(seed)
+    for d, c in zip(fr.depth, fr.conf):
+        far = rng.random(d.shape) < 0.02
+        d[far] = np.finfo(np.float32).max
+        c[far] = 0.0
+    return rig, fr
+
+
+@pytest.mark.parametrize("top_k", [0, 7])
+def test_infinite_residual_weighs_nothing(F, oracle_mod, top_k):
+    rig, fr = _with_sentinels(81)
+    params = {"coarse_cell_m": 0.4, "max_level": 0, "n_min": 2, "top_k": top_k}
+    orc = oracle_mod.fuse_frame(rig, fr, params)
+    hit = (orc["gated"] != 0) & (orc["e"] > 1e30)
+    assert hit.sum() > 100
+    assert np.all(np.isin(orc["key"][hit], orc["key"][(orc["gated"] != 0) & (orc["e"] < 1e3)]))
+    gpu = _fuse(F, rig, fr, **params)
+    rep = compare(gpu, orc)
+    assert rep["n_cells_valued"] > 20
+
+
+def test_infinite_residual_of_a_point(F, oracle_mod):
+    from test_gpu_points import _points
+    rig, fr = _with_sentinels(82)
+    orc = oracle_mod.fuse_frame(rig, fr, {})
+    hit = (orc["gated"] != 0) & (orc["e"] > 1e30)
+    assert hit.sum() > 100
+    _, _, _, w, _ = _points(F, rig, fr)
+    assert np.all(w[hit] == 0.0)
