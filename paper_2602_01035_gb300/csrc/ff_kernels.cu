@@ -473,7 +473,9 @@ __device__ __forceinline__ void residual_sum(const BlockConst* bc, const Tables&
 // e = m ln 2 + f, f in [0, ln 2), so that mu never underflows (C' = C, or 1 without the
 // confidence term).  A residual beyond float32 (a view's sample near the format's largest value)
 // leaves e infinite or not a number; its weight is 0 at an exponent above every other, so that it
-// adds nothing to a sum and does not set the sum's scale.  Returns e (high part) for traces.
+// adds nothing to a sum and does not set the sum's scale.  Confidences above 1 move into the
+// exponent (exactly), which keeps mu below 2 for the fixed-point terms.  Returns e (high part) for
+// traces.
 constexpr int kFarExponent = 1500000000;   // other exponents are at most 1e9 / ln 2
 __device__ __forceinline__ float joint_weight(const RigHot& rig, int k1, float sh, float sl,
                                               float c, float& mu, int& m) {
@@ -496,10 +498,16 @@ __device__ __forceinline__ float joint_weight(const RigHot& rig, int k1, float s
   }
   const float base = rig.use_conf ? c : 1.0f;                          // Eq. 10
   mu = __fmul_rn(__fmul_rn(base, expf(-fh)), __fsub_rn(1.0f, fl));
-  if (mu != mu) {
-    mu = 0.0f;
-    m = kFarExponent;
-    eh = __int_as_float(0x7f800000);
+  if (!(mu < 2.0f)) {                       // confidences above 1, or no number
+    if (mu != mu) {
+      mu = 0.0f;
+      m = kFarExponent;
+      eh = __int_as_float(0x7f800000);
+    } else if (mu < __int_as_float(0x7f800000)) {
+      const int bits = __float_as_int(mu);
+      m -= (bits >> 23) - 127;
+      mu = __int_as_float((bits & 0x7fffff) | 0x3f800000);
+    }
   }
   return eh;
 }
@@ -1150,9 +1158,10 @@ __global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64) k_weigh(const __grid_cons
 }
 
 // ------------------------------------------------------------------ sum step
-// rint(v) for 0 <= v < 2^37 as an integer, without 64-bit conversions: floor(v 2^-22) and rint of
-// the rest (exact: both are multiples of ulp(v)) are read off sums with 2^23, and adding the even
-// integer hi 2^22 does not change a round-half-even decision.
+// rint(v) for 0 <= v < 2^45 as an integer, without 64-bit conversions (terms are below 2^37, as
+// weights are below 2: joint_weight): floor(v 2^-22) and rint of the rest (exact: both are
+// multiples of ulp(v)) are read off sums with 2^23, and adding the even integer hi 2^22 does not
+// change a round-half-even decision.
 __device__ __forceinline__ unsigned long long fixed_term(float v) {
   constexpr unsigned kBits = 0x4B000000u;                  // 2^23
   const float h = __fmaf_rd(v, 1.0f / 4194304.0f, 8388608.0f);

@@ -1,5 +1,5 @@
 """Values at the ends of the accepted ranges, against the oracle at the parity tolerances:
-depth samples so far away that a residual leaves float32."""
+depth samples so far away that a residual leaves float32, and confidences above one."""
 import numpy as np
 import pytest
 
@@ -63,3 +63,15 @@ def test_infinite_residual_of_a_point(F, oracle_mod):
     assert hit.sum() > 100
     _, _, _, w, _ = _points(F, rig, fr)
     assert np.all(w[hit] == 0.0)
+
+
+@pytest.mark.parametrize("scale", [255.0, 1000.0, 65535.0, 1e30])
+@pytest.mark.parametrize("top_k", [0, 3])
+def test_confidences_above_one(F, oracle_mod, scale, top_k):
+    """Confidence images on another scale than [0, 1] fuse to the same cloud at that scale."""
+    rig, _, fr = S.config1()
+    fr = S.Frame(fr.depth, [(c * np.float32(scale)).astype(np.float32) for c in fr.conf], fr.rgb)
+    params = {"tau": float(np.float32(0.6) * np.float32(scale)), "top_k": top_k}
+    gpu = _fuse(F, rig, fr, with_trace=True, **params)
+    rep = compare(gpu, oracle_mod.fuse_frame(rig, fr, params))
+    assert rep["n_cells_valued"] > 100
