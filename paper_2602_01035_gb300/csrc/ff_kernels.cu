@@ -880,6 +880,12 @@ __device__ __forceinline__ void frame_stats(const Tables& t, const OutDev& out) 
   if (!TOPK)                                    // cells past the output's capacity (reported): their slots
     for (unsigned i = (unsigned)out.max_cells + threadIdx.x; i < nc && i < t.max_slots; i += kThreads)
       *reinterpret_cast<uint4*>(t.frec + t.fused[i]) = kSlotClear;
+  // cells without a record, as these ran out (reported), are not in the list of cells that the reduce
+  // step clears, but their keys are in their slots
+  if (TOPK && __ldcg(&t.cnt->n_partials) > t.max_partials) {
+    const unsigned n_slots = (unsigned)min(__ldcg(&t.cnt->n_slots), (unsigned long long)t.max_slots);
+    for (unsigned i = threadIdx.x; i < n_slots; i += kThreads) *reinterpret_cast<uint4*>(t.frec + i) = kSlotClear;
+  }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     for (int o = 16; o > 0; o >>= 1) n[k] += __shfl_xor_sync(0xffffffffu, n[k], o);

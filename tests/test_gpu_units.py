@@ -85,6 +85,34 @@ def test_static_calls_alternate_between_variants(oracle_mod):
         Z._check_same(ref["cells"], ref["stats"], out, int(stats.n_cells))
 
 
+def test_static_call_after_top_k_ran_out_of_records():
+    """A top-k frame with more (tile, cell) records than the static entry holds leaves cells that
+    were never listed; nothing of them may pass for a member of a later frame, not even where its
+    members' confidences are negative (they do not gate without the confidence term)."""
+    import test_zz_no_alloc as Z
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_01035_gb300 import fuseflow as F
+    dev, stream = torch.device("cuda"), torch.cuda.current_stream().cuda_stream
+    big = S.tiny_rig(n=2, width=512, height=512)
+    rig = S.tiny_rig(n=3, width=160, height=120, spread_deg=30.0)
+    fr = S.random_frame(rig, seed=54, flying_frac=0.01)
+    low = S.Frame(fr.depth, [c - np.float32(1.5) for c in fr.conf], fr.rgb)
+    for frame, params in ((low, {"use_conf": 0}), (fr, {})):
+        st, stats, _ = Z._static_call(F, big, _scattered(big, 55, 500, 8000), 32768, dev, stream, top_k=3,
+                                      coarse_cell_m=2.0, max_level=4, n_min=1)
+        assert st == F.FUSEFLOW_OK and stats.error & 16       # more records than the buffer holds
+        for _ in range(2):
+            ff = F.FuseFlow(rig, max_cells=8192, **params)
+            try:
+                ref = run_gpu(ff, frame, torch, with_trace=False)
+            finally:
+                ff.close()
+            st, stats, out = Z._static_call(F, rig, frame, 8192, dev, stream, **params)
+            assert st == F.FUSEFLOW_OK and stats.error == 0
+            Z._check_same(ref["cells"], ref["stats"], out, int(stats.n_cells))
+
+
 def test_crowded_units_in_few_and_many_blocks():
     """Units of nearly 256 coarse cells: one frame alone takes the count step of few units, eight
     in a batch that of many.  The clouds are the same to the bit (no result depends on the order
