@@ -439,8 +439,12 @@ __device__ __forceinline__ bool residual_grid(const ViewHot* views, int k1, cons
     }
     ++nview;
   }
-  // S = hi 2^24 + lo and the remainders' sum c as one ff (hi is exact below 2^24: d < 2^24 units)
-  const float hi = __fmul_rn((float)(int)(S >> 24), 16777216.0f), lo = (float)(int)(S & 0xffffff);
+  // S = hi 2^25 + lo, -2^24 <= lo < 2^24, and the remainders' sum c as one ff.  Both parts are exact:
+  // a point and the sample at its pixel lie along one ray of the view, so that |D| < 2^22 and
+  // S < 3 kMaxK1 2^44 < 2^49
+  static_assert(3 * kMaxK1 <= 32, "the high part of a residual sum fits 24 bits");
+  const int hn = (int)((S + (1 << 24)) >> 25);
+  const float hi = __fmul_rn((float)hn, 33554432.0f), lo = (float)(int)((unsigned)S - ((unsigned)hn << 25));
   float s1, e1, e2;
   two_sum(lo, c, s1, e1);
   fast_two_sum(hi, s1, sh, e2);

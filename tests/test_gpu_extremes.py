@@ -1,5 +1,6 @@
 """Values at the ends of the accepted ranges, against the oracle at the parity tolerances:
-depth samples so far away that a residual leaves float32, and confidences above one."""
+depth samples so far away that a residual leaves float32, confidences above one, and residual
+sums of 2^48 grid units squared and more."""
 import numpy as np
 import pytest
 
@@ -75,3 +76,32 @@ def test_confidences_above_one(F, oracle_mod, scale, top_k):
     gpu = _fuse(F, rig, fr, with_trace=True, **params)
     rep = compare(gpu, oracle_mod.fuse_frame(rig, fr, params))
     assert rep["n_cells_valued"] > 100
+
+
+def test_residual_sums_past_48_bits(F, oracle_mod):
+    """Cameras of one pose and 126 degrees: eight whose corner samples lie at the end of the grid's
+    range, and eight more whose corners hold near points 1 mm apart, each of which differs from all
+    of the first eight by nearly the whole range.  One cell a corner, exponents of 16,000 that differ
+    by a half from point to point: an error of 2^-24 of a residual moves its weight by 0.1 %."""
+    n, size = 16, 40
+    f = (size - 1) / 2 / 1.94
+    cams = [S.Camera(f, f, (size - 1) / 2, (size - 1) / 2, size, size, np.eye(3), np.zeros(3)) for _ in range(n)]
+    rig = S.Rig(cams, "f32", 1.0)
+    rng = np.random.default_rng(83)
+    depth, conf, rgb = [], [], []
+    for k in range(n):
+        d, c = np.zeros((size, size), np.float32), np.zeros((size, size), np.float32)
+        for y in (0, size - 1):
+            for x in (0, size - 1):
+                d[y, x] = 65.5 if k < 8 else 1.2 + 1e-3 * (k - 8)
+                c[y, x] = 0.0 if k < 8 else 1.0
+        depth.append(d)
+        conf.append(c)
+        rgb.append(rng.choice(np.array([0, 255], np.uint8), size=(size, size, 3)))
+    fr = S.Frame(depth, conf, rgb)
+    params = {"k_views": 9, "sigma_m": 1.47, "coarse_cell_m": 1.0, "max_level": 0}
+    orc = oracle_mod.fuse_frame(rig, fr, params)
+    e = orc["e"][orc["gated"] != 0]
+    assert len(e) == 32 and e.min() > 1.6e4 and orc["stats"]["n_cells"] == 4
+    rep = compare(_fuse(F, rig, fr, **params), orc)
+    assert rep["n_cells_valued"] == 4
