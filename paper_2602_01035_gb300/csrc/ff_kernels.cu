@@ -1112,8 +1112,10 @@ __global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64) k_weigh(const __grid_cons
       lb = (e >> 8) != kNoCellNumber ? s_lb[(e >> 8) + (unsigned)(unit * kUnitCells)]
                                      : coarse_lvbase(t, pack_key(0, cc[0], cc[1], cc[2]));
     const unsigned ls = point_slot(lb, r, kk, frac), slot = ls & kBaseNone;
-    uint4 rec = make_uint4(0u, 0u, 0u, 0u);                           // representative, number, exponent
-    if (slot != kBaseNone) rec = __ldcg(reinterpret_cast<const uint4*>(t.frec + slot));
+    // representative; number and exponent.  In two words of 64 bits: other blocks raise the key meanwhile,
+    // and only a word is read whole
+    ulonglong2 rec = make_ulonglong2(0ull, 0ull);
+    if (slot != kBaseNone) rec = __ldcg(reinterpret_cast<const ulonglong2*>(t.frec + slot));
     float sh = 0.0f, sl = 0.0f, mu = 0.0f;
     int nview = 0, m = 0;
     if (n_views > 0)
@@ -1126,9 +1128,9 @@ __global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64) k_weigh(const __grid_cons
     if (slot != kBaseNone) {                    // else out of range, or no slot left (reported)
       SlotRec* s = t.frec + slot;
       const unsigned long long key = ((unsigned long long)ordered(c) << 32) | (unsigned)(~g);
-      if ((((unsigned long long)rec.y << 32) | rec.x) < key) atomicMax(&s->key, key);
-      if ((int)rec.w > m) atomicMin(&s->mmin, m);
-      if (rec.z == kSlotNone && atomicCAS(&s->head, kSlotNone, kSlotPending) == kSlotNone) {
+      if (rec.x < key) atomicMax(&s->key, key);
+      if ((int)(rec.y >> 32) > m) atomicMin(&s->mmin, m);
+      if ((unsigned)rec.y == kSlotNone && atomicCAS(&s->head, kSlotNone, kSlotPending) == kSlotNone) {
         const unsigned q = atomicAdd(&s_claims, 1u);
         s_slot[q] = slot;
         s_key[q] = pack_key((int)(ls >> 27), kk[0], kk[1], kk[2]);

@@ -64,6 +64,19 @@ def test_sizes_around_units(oracle_mod, w, h):
     _check(oracle_mod, rig, S.random_frame(rig, seed=7), n_min=2)
 
 
+@pytest.mark.parametrize("equal", [False, True])
+def test_representative_of_one_crowded_cell(oracle_mod, equal):
+    """Eight cells around the origin hold every point, in one image after another of rising
+    confidence (or all of one): each of tens of thousands of points raises its cell's record."""
+    rig = S.tiny_rig(n=4, width=160, height=120, spread_deg=90.0)
+    fr = S.random_frame(rig, seed=9)
+    rise = np.arange(rig.n_pixels, dtype=np.float32).reshape(4, 120, 160) / np.float32(4 * rig.n_pixels)
+    fr = S.Frame(fr.depth, [np.full_like(c, 0.9) if equal else np.float32(0.7) + rise[i] for i, c in enumerate(fr.conf)],
+                 fr.rgb)
+    rep, _ = _check(oracle_mod, rig, fr, coarse_cell_m=100.0, max_level=0)
+    assert rep["n_cells_oracle"] <= 8 and rep["n_cells_matched"] >= 6
+
+
 def test_static_calls_alternate_between_variants(oracle_mod):
     """The allocation-free entry keeps its tables between calls: a top-k frame leaves nothing in
     them that a frame of all members would read, nor the other way round."""
