@@ -66,15 +66,19 @@ def test_sizes_around_units(oracle_mod, w, h):
 
 @pytest.mark.parametrize("equal", [False, True])
 def test_representative_of_one_crowded_cell(oracle_mod, equal):
-    """Eight cells around the origin hold every point, in one image after another of rising
-    confidence (or all of one): each of tens of thousands of points raises its cell's record."""
+    """One cell holds every point, in one image after another of rising confidence (or all of
+    one): each of tens of thousands of points raises the cell's record."""
     rig = S.tiny_rig(n=4, width=160, height=120, spread_deg=90.0)
     fr = S.random_frame(rig, seed=9)
+    for c in rig.cameras:                                  # the scene to the middle of a cell
+        c.t = c.t - c.R @ np.full(3, 50.0)
     rise = np.arange(rig.n_pixels, dtype=np.float32).reshape(4, 120, 160) / np.float32(4 * rig.n_pixels)
     fr = S.Frame(fr.depth, [np.full_like(c, 0.9) if equal else np.float32(0.7) + rise[i] for i, c in enumerate(fr.conf)],
                  fr.rgb)
-    rep, _ = _check(oracle_mod, rig, fr, coarse_cell_m=100.0, max_level=0)
-    assert rep["n_cells_oracle"] <= 8 and rep["n_cells_matched"] >= 6
+    rep, gpu = _check(oracle_mod, rig, fr, coarse_cell_m=100.0, max_level=0)
+    assert rep["n_cells_oracle"] == rep["n_cells_matched"] == 1
+    order = np.concatenate([c.reshape(-1) for c in fr.conf]) * np.concatenate([d.reshape(-1) > 0 for d in fr.depth])
+    assert gpu["cells"]["rep"][0] == np.argmax(order)
 
 
 def test_static_calls_alternate_between_variants(oracle_mod):
