@@ -881,9 +881,6 @@ __device__ __forceinline__ void frame_stats(const Tables& t, const OutDev& out) 
     for (int k = 0; k < 3; ++k) { mn[k] = min(mn[k], b.bmin[k]); mx[k] = max(mx[k], b.bmax[k]); }
   }
   const unsigned nc = __ldcg(&t.cnt->n_cells);
-  if (!TOPK)                                    // cells past the output's capacity (reported): their slots
-    for (unsigned i = (unsigned)out.max_cells + threadIdx.x; i < nc && i < t.max_slots; i += kThreads)
-      *reinterpret_cast<uint4*>(t.frec + t.fused[i]) = kSlotClear;
   // cells without a record, as these ran out (reported), are not in the list of cells that the reduce
   // step clears, but their keys are in their slots
   if (TOPK && __ldcg(&t.cnt->n_partials) > t.max_partials) {
@@ -1158,13 +1155,11 @@ __global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64) k_weigh(const __grid_cons
   for (unsigned q = threadIdx.x; q < n; q += blockDim.x) {
     const unsigned id = s_first + q, slot = s_slot[q];
     t.frec[slot].head = id;
-    if ((long long)id < fa.out.max_cells) {
+    if ((long long)id < fa.out.max_cells) {   // else past the capacity
       uint4* a = reinterpret_cast<uint4*>(t.rows + id);
 #pragma unroll
       for (int k = 0; k < 4; ++k) a[k] = make_uint4(0u, 0u, 0u, 0u);
       a[4] = make_uint4((unsigned)s_key[q], (unsigned)(s_key[q] >> 32), slot, 0u);
-    } else {
-      t.fused[id] = slot;                   // past the capacity; a number for each slot at most
     }
   }
 }
@@ -1275,6 +1270,10 @@ __global__ void k_sum(const __grid_constant__ BatchArgs<NB> args) {
             if (q < kTileShares) atomicAdd(&s_share[q], 1u);
             else atomicAdd(&t.bsum[share0 + q], 1u);
           }
+        } else if (rec.x == ~(off + (unsigned)(y * W + x))) {
+          // past the output's capacity (reported): no row and no mark, so its slot is cleared here; the
+          // cell's other points find no number in it, or one past the capacity
+          *reinterpret_cast<uint4*>(t.frec + slot) = kSlotClear;
         }
         uint4* row = s_row + (lane + (lane >> 3)) * 4;
 #pragma unroll
