@@ -444,6 +444,7 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   ctx->geo.screen = screen_set(params) ? 1 : 0;
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  ctx->geo.sms = sms;
   const int n_tiles = fill_tile_index(*rig, &ctx->geo.tiles, 16);
   ctx->n_units = ctx->geo.tiles.unit[n_cams];
   count_geometry(&ctx->geo, ctx->n_units, default_chunks(ctx->n_units, sms));
@@ -1419,6 +1420,7 @@ extern "C" int fuseflow_fuse_frame_static(const fuseflow_intrinsics* intr,
   count_geometry(&geo, n_units, 1);
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  geo.sms = sms;
   geo.emit_blocks = std::max(1, sms * 8);
   geo.pdl = 2;                                         // at most 2^19 pixels: small frames
   Tables t = static_tables(base, n_px, geo.count_blocks);

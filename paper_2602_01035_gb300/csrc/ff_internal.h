@@ -124,6 +124,7 @@ cudaError_t launch_screen(const ScreenArgs& a, bool depth_f32, long long max_px,
 
 struct Geometry {
   int n_cams;
+  int sms;                       // multiprocessors of the device
   int depth_f32;
   int screen;                    // a screen is set: fuse calls write D^r into screen_buf first
   ScreenArgs scr;                // bounds, sizes and the context's D^r buffers (out)

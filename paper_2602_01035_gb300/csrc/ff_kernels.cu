@@ -561,9 +561,9 @@ constexpr unsigned kUnnumbered = 0x80000000u;   // on a unit's count while point
 // blocks with a table of 2048 cells and runs of equal cells merged across the warp took 59 us.  Finding a
 // unit's cells one after another as the smallest key left took 49 us there, but 236 instead of 154 us
 // where units hold many cells (16x1024^2).
-constexpr int kCountFew = 2 * 4 * 152;   // blocks: 4 a multiprocessor at once
+constexpr int kCountFew = 2 * 4 * (kThreads / 32);   // units a multiprocessor: two rounds of 4 blocks
 
-// FEW: frames of no more units than the chip takes at once or twice, where the step is as long as a crowded
+// FEW: launches of no more units than the chip takes at once or twice (whatever the units per block), where the step is as long as a crowded
 // unit's chain of probes.  There a unit whose first 32 points have more than 14 cells puts no more into its
 // table, and 8 of its points instead of 4 are under way together: frames of 5x326x319 in a room 94 -> 85 us,
 // 8x248x228 95 -> 87 us (limits of 10 and 20 cells: 87 and 87).  With the test in it the loop takes 3 to 5 %
@@ -2379,18 +2379,18 @@ cudaError_t launch_k(bool pdl, void (*kernel)(P...), dim3 grid, dim3 block, size
 
 // Threads of a weigh or sum block: a thread for four pixels, or fewer while all of a launch's blocks
 // fit on the chip at once (a frame of 80 tiles then takes a pixel a thread instead of four in turn).
-int weigh_threads(int tiles, int th) {
+int weigh_threads(int tiles, int th, int sms) {
   int n = 8 * th;
-  while (n < 32 * th && n < 512 && 2ll * n * tiles <= 152 * 1024) n *= 2;
+  while (n < 32 * th && n < 512 && 2ll * n * tiles <= 1024ll * sms) n *= 2;
   return n;
 }
 
 // The assign step over the batch's tiles (TH rows a tile; the traced instantiations exist for
 // single frames only): the weigh kernel, or the top-k variant's.
 template <typename DT, int NB, int TH>
-cudaError_t launch_assign(const BatchArgs<NB>& a, int n, bool top_k, bool traced, int max_k1, bool pdl,
+cudaError_t launch_assign(const BatchArgs<NB>& a, int n, bool top_k, bool traced, int max_k1, int sms, bool pdl,
                           cudaStream_t s) {
-  const dim3 tiles(a.tile_first[n]), at(AssignTile<TH>::Threads), wt(weigh_threads(a.tile_first[n], TH));
+  const dim3 tiles(a.tile_first[n]), at(AssignTile<TH>::Threads), wt(weigh_threads(a.tile_first[n], TH, sms));
   const size_t tk = AssignTile<TH>::Bytes, sm = WeighTile<TH>::smem(max_k1);
   if constexpr (NB == 1)
     if (traced)
@@ -2401,8 +2401,8 @@ cudaError_t launch_assign(const BatchArgs<NB>& a, int n, bool top_k, bool traced
 }
 
 template <typename DT, int NB, int TH>
-cudaError_t launch_sum(const BatchArgs<NB>& a, int n, bool pdl, cudaStream_t s) {
-  const int threads = weigh_threads(a.tile_first[n], TH);
+cudaError_t launch_sum(const BatchArgs<NB>& a, int n, int sms, bool pdl, cudaStream_t s) {
+  const int threads = weigh_threads(a.tile_first[n], TH, sms);
   return launch_k(pdl, k_sum<DT, NB, TH>, dim3(a.tile_first[n]), dim3(threads), 16 * kSumWarpWords * (threads / 32), s, a);
 }
 
@@ -2419,6 +2419,7 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
   std::memset(&a, 0, sizeof(a));
   a.n = n;
   int emit = 1, pdl_level = 2, max_wblocks = 1, max_k1 = 0;
+  long long units = 0;
   const Geometry& g0 = *fr[0].geo;
   cudaError_t err = cudaSuccess;
   for (int f = 0; f < n; ++f) {
@@ -2446,6 +2447,7 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
     }
     a.count_first[f + 1] = a.count_first[f] + geo.count_blocks;
     a.tile_first[f + 1] = a.tile_first[f] + t.n_tiles;
+    units += t.n_units;
     emit = std::max(emit, geo.emit_blocks);
     pdl_level = std::min(pdl_level, geo.pdl);
     max_wblocks = std::max(max_wblocks, t.n_wblocks);
@@ -2457,7 +2459,7 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
   const bool pdl = pdl_level >= 1 && ev == nullptr;
   const bool pdl_reduce = pdl_level >= 2 && ev == nullptr;
   const dim3 eb(emit, n), th3(kThreads);
-  const bool few = a.count_first[n] <= kCountFew;
+  const bool few = units <= (long long)kCountFew * g0.sms;
   if ((err = few ? launch_k(false, k_count<DT, NB, true>, dim3(a.count_first[n]), th3, 0, s, a)
                  : launch_k(false, k_count<DT, NB, false>, dim3(a.count_first[n]), th3, 0, s, a)) != cudaSuccess ||
       (err = launch_k(pdl, k_levels<NB>, eb, th3, 0, s, a)) != cudaSuccess)
@@ -2470,15 +2472,15 @@ cudaError_t launch_frames(const FrameLaunch* fr, int n, cudaStream_t s, cudaEven
   }
   const int th = g0.tiles.th;
   const bool topk = g0.top_k != 0;
-  if (th == 8) err = launch_assign<DT, NB, 8>(a, n, topk, traced, max_k1, pdl, s);
-  else if (th == 32) err = launch_assign<DT, NB, 32>(a, n, topk, traced, max_k1, pdl, s);
-  else err = launch_assign<DT, NB, 16>(a, n, topk, traced, max_k1, pdl, s);
+  if (th == 8) err = launch_assign<DT, NB, 8>(a, n, topk, traced, max_k1, g0.sms, pdl, s);
+  else if (th == 32) err = launch_assign<DT, NB, 32>(a, n, topk, traced, max_k1, g0.sms, pdl, s);
+  else err = launch_assign<DT, NB, 16>(a, n, topk, traced, max_k1, g0.sms, pdl, s);
   if (err != cudaSuccess) return err;
   mark(3);
   if (topk) err = launch_k(pdl_reduce, k_reduce_topk<DT, NB>, dim3(2 * emit, n), dim3(kTopThreads), 0, s, a);
-  else if (th == 8) err = launch_sum<DT, NB, 8>(a, n, pdl_reduce, s);
-  else if (th == 32) err = launch_sum<DT, NB, 32>(a, n, pdl_reduce, s);
-  else err = launch_sum<DT, NB, 16>(a, n, pdl_reduce, s);
+  else if (th == 8) err = launch_sum<DT, NB, 8>(a, n, g0.sms, pdl_reduce, s);
+  else if (th == 32) err = launch_sum<DT, NB, 32>(a, n, g0.sms, pdl_reduce, s);
+  else err = launch_sum<DT, NB, 16>(a, n, g0.sms, pdl_reduce, s);
   if (err != cudaSuccess) return err;
   mark(4);
   mark(5);
