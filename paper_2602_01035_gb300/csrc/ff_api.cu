@@ -966,8 +966,8 @@ int fuseflow_fuse_points(fuseflow_ctx* ctx, const void* const* depth, const floa
                reinterpret_cast<unsigned long long*>(static_cast<char*>(ctx->d_mc) + kMcBytes),
                (float)ctx->params.depth_scale};
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (launch_points(ctx->d_rig, ctx->geo.hot, ctx->d_rays, fp, ctx->tab, pd, ctx->geo.depth_f32 != 0, ctx->geo.tiles, s) !=
-      cudaSuccess)
+  if (launch_points(ctx->d_rig, ctx->geo.hot, ctx->d_rays, fp, ctx->tab, pd, ctx->geo.depth_f32 != 0, ctx->geo.tiles,
+                    ctx->geo.sms, s) != cudaSuccess)
     return FUSEFLOW_ERR_CUDA;
   if (n_valid || n_gated) {
     unsigned long long h[2] = {0ull, 0ull};

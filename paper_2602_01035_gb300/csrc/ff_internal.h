@@ -184,7 +184,7 @@ struct PointsDev {
   float unit_f;
 };
 cudaError_t launch_points(const RigDev* rig, const RigHot& hot, const float2* rays, const FramePtrs& fp, const Tables& t,
-                          const PointsDev& out, bool depth_f32, const TileIndex& tiles, cudaStream_t s);
+                          const PointsDev& out, bool depth_f32, const TileIndex& tiles, int sms, cudaStream_t s);
 
 // Eq. 3 confidence producer: per camera, depth in, float32 confidence out.
 struct ConfArgs {

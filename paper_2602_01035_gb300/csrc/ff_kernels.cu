@@ -1719,67 +1719,79 @@ __global__ void __launch_bounds__(kTopThreads, 8) k_reduce_topk(const __grid_con
 // copied), so the cloud is in pixel order without a compaction pass.
 // A block takes a tile of 32 columns by 16 rows, as the weigh step does: the gated pixels compacted in
 // shared memory and weighed with full warps, the view constants and pair rays staged, and the results
-// laid out by pixel for stores in order.
-// 8x1280x720 (7.4 Mpx, half of them gated): 130 us; a thread a pixel, rays and view constants from global
-// memory, took 191 us, and 167 us on the weigh step's residual.  Bound by the residual's instructions.
+// laid out by pixel for stores in order.  The tile's samples and colours are asked for first, from sizes
+// and offsets in the constant bank, and few tiles take more threads a block, down to a pixel a thread
+// (weigh_threads).  8x1280x720 (7.4 Mpx): 117 us with half of the pixels gated, 49 us with 2 %; without
+// these two points 129 and 66 us, and a thread a pixel with rays and view constants from global memory
+// 189 and 57 us.  2x160x120: 8.2, 10.4 and 7.8 us.  Bound by the residual's instructions.
 struct PointsTile {
-  static constexpr int H = 16, Px = kTileW * H, Threads = 128;
+  static constexpr int H = 16, Px = kTileW * H;
   static constexpr size_t Out = 0;                                 // f32[4][Px]: pos xyz, weight, by pixel
   static constexpr size_t P = Out + 16 * Px;                       // u16[Px]: the gated pixels
   static constexpr size_t BC = P + 2 * Px;                         // constants, column and row pair rays
   static constexpr size_t smem(int k1) { return BC + 16 * (size_t)(4 * (1 + k1) + k1 * (kPrayColGroup + H / 8 * kPrayRowGroup)); }
 };
 
-template <typename DT>
+template <typename DT, int Threads>
 __global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64)
 k_points(const RigDev* __restrict__ rigp, const __grid_constant__ RigHot hot, const float2* __restrict__ rays,
-         const __grid_constant__ FramePtrs fp, const __grid_constant__ Tables t, PointsDev out) {
+         const __grid_constant__ FramePtrs fp, const __grid_constant__ Tables t, const __grid_constant__ TileIndex ti,
+         PointsDev out) {
   using PT = PointsTile;
+  constexpr int kWarps = Threads / 32, kRows = PT::H / kWarps;      // rows a warp
+  static_assert(kRows * kWarps == PT::H, "whole rows a warp");
   extern __shared__ __align__(16) unsigned char smem[];
   float* const s_out = reinterpret_cast<float*>(smem + PT::Out);
   unsigned short* const s_p = reinterpret_cast<unsigned short*>(smem + PT::P);
   const BlockConst& bc = *reinterpret_cast<const BlockConst*>(smem + PT::BC);
   __shared__ unsigned s_n, s_valid;
-  const RigDev& rig = *rigp;
   const int cam = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const CamDev& C = rig.cam[cam];
-  const int W = C.W, H = C.H, k1 = rig.k1, tiles_x = (W + kTileW - 1) / kTileW;
-  const int ty = (int)blockIdx.x / tiles_x, x0 = ((int)blockIdx.x - ty * tiles_x) * kTileW, y0 = ty * PT::H;
+  const int W = ti.W[cam], H = ti.H[cam], k1 = ti.k1, tiles_x = (W + kTileW - 1) / kTileW;
+  int tx;
+  const int y0 = fast_div((int)blockIdx.x, tiles_x, ti.div_x[cam], tx) * PT::H, x0 = tx * kTileW;
   if (y0 >= H) return;                                              // uniform over the block
+  const int w = min(kTileW, W - x0);
+  const long long p0 = (long long)y0 * W + x0;                      // the tile's first pixel
+  const DT* __restrict__ dep = static_cast<const DT*>(fp.depth[cam]) + p0;
+  const float* __restrict__ cf = fp.conf[cam] + p0;
+  const uint8_t* __restrict__ col = fp.rgb[cam] + 3 * p0;
+  const float qnan = __int_as_float(0x7fc00000);
+  DT D[kRows];
+  float c[kRows];
+  uint8_t rgb[kRows][3];
+#pragma unroll
+  for (int k = 0; k < kRows; ++k) {
+    const int y = warp + kWarps * k;
+    const unsigned li = (unsigned)(y * W + lane);                   // W H <= 2^30
+    D[k] = (DT)0;
+    c[k] = 0.0f;
+    if (lane < w && y0 + y < H) {
+      D[k] = dep[li];
+      c[k] = cf[li];
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a)                                     // a row's colours, a byte a lane
+      rgb[k][a] = lane + 32 * a < 3 * w && y0 + y < H ? __ldg(col + 3u * (unsigned)(y * W) + lane + 32 * a) : (uint8_t)0;
+  }
   const int n_views = hot.use_cons ? k1 : 0, n_const = 4 * (1 + n_views), n_cols = n_views * kPrayColGroup;
   const float4* const s_cols = reinterpret_cast<const float4*>(smem + PT::BC) + n_const;
   {
     const float4* gc = reinterpret_cast<const float4*>(t.bconst + cam);
-    const float4* ga = t.pray + t.bconst[cam].cam.pray + (x0 >> 5) * k1 * kPrayColGroup;
-    const float4* gb = t.pray + t.bconst[cam].cam.pray + (tiles_x * kPrayColGroup + (y0 >> 3) * kPrayRowGroup) * k1;
+    const float4* ga = t.pray + ti.pray[cam] + (x0 >> 5) * k1 * kPrayColGroup;
+    const float4* gb = t.pray + ti.pray[cam] + (tiles_x * kPrayColGroup + (y0 >> 3) * kPrayRowGroup) * k1;
     const int n = n_const + n_cols + n_views * (PT::H / 8) * kPrayRowGroup;
-    for (int i = threadIdx.x; i < n; i += PT::Threads) {
+    for (int i = threadIdx.x; i < n; i += Threads) {
       const float4* src = i < n_const ? gc + i : i < n_const + n_cols ? ga + (i - n_const) : gb + (i - n_const - n_cols);
       cp_async16(smem + PT::BC + 16 * i, src);
     }
   }
   if (threadIdx.x == 0) { s_n = 0u; s_valid = 0u; }
   __syncthreads();
-  const DT* __restrict__ dep = static_cast<const DT*>(fp.depth[cam]);
-  const float* __restrict__ cf = fp.conf[cam];
-  const float qnan = __int_as_float(0x7fc00000);
-  DT D[4];
-  float c[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int x = x0 + lane, y = y0 + warp + 4 * k;
-    D[k] = (DT)0;
-    c[k] = 0.0f;
-    if (x < W && y < H) {
-      const unsigned li = (unsigned)(y * W + x);                    // W H <= 2^30
-      D[k] = dep[li];
-      c[k] = cf[li];
-    }
-  }
+  const long long g0 = ti.off[cam] + p0;
   unsigned nv = 0u;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int i = (warp + 4 * k) * kTileW + lane;
+  for (int k = 0; k < kRows; ++k) {
+    const int r = warp + kWarps * k, i = r * kTileW + lane;
     const bool valid = Depth<DT>::valid(D[k]);
     const bool gated = valid && (!hot.use_conf || c[k] > hot.tau);  // Eq. 9
     nv += __popc(__ballot_sync(0xffffffffu, valid));
@@ -1797,13 +1809,16 @@ k_points(const RigDev* __restrict__ rigp, const __grid_constant__ RigHot hot, co
       s_out[3 * i + 2] = qnan;
       s_out[3 * PT::Px + i] = 0.0f;
     }
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      if (lane + 32 * a < 3 * w && y0 + r < H) out.rgb[3 * (g0 + (long long)r * W) + lane + 32 * a] = rgb[k][a];
   }
   if (lane == 0 && nv) atomicAdd(&s_valid, nv);
   cp_async_wait();
   __syncthreads();
   const int n = (int)s_n;
 #pragma unroll 1
-  for (int i = threadIdx.x; i < n; i += PT::Threads) {
+  for (int i = threadIdx.x; i < n; i += Threads) {
     const int q = s_p[i], lx = q & (kTileW - 1), ly = q / kTileW, x = x0 + lx, y = y0 + ly;
     const float z = s_out[3 * q], cq = s_out[3 * q + 1];
     float P[3];
@@ -1819,17 +1834,14 @@ k_points(const RigDev* __restrict__ rigp, const __grid_constant__ RigHot hot, co
     s_out[3 * PT::Px + q] = ldexpf(mu, -min(m, 1 << 30));
   }
   __syncthreads();
-  const int w = min(kTileW, W - x0), h = min(PT::H, H - y0);
-  const long long g0 = C.off + (long long)y0 * W + x0;
-  const uint8_t* __restrict__ col = fp.rgb[cam] + 3ll * ((long long)y0 * W + x0);
-  for (int r = warp; r < h; r += PT::Threads / 32) {                  // a warp a row
+#pragma unroll
+  for (int k = 0; k < kRows; ++k) {                                   // a warp a row
+    const int r = warp + kWarps * k;
+    if (y0 + r >= H) break;
     const long long g = g0 + (long long)r * W;
 #pragma unroll
     for (int a = 0; a < 3; ++a)
-      if (lane + 32 * a < 3 * w) {
-        out.pos[3 * g + lane + 32 * a] = s_out[3 * r * kTileW + lane + 32 * a];
-        out.rgb[3 * g + lane + 32 * a] = __ldg(col + 3ll * r * W + lane + 32 * a);
-      }
+      if (lane + 32 * a < 3 * w) out.pos[3 * g + lane + 32 * a] = s_out[3 * r * kTileW + lane + 32 * a];
     if (lane < w) out.weight[g + lane] = s_out[3 * PT::Px + r * kTileW + lane];
   }
   if (threadIdx.x == 0) {
@@ -2624,18 +2636,39 @@ cudaError_t launch_mc(const RigDev* rig, const FramePtrs& fp, bool depth_f32, co
   return cudaGetLastError();
 }
 
+// Tiles of the point-wise path over all cameras, and the largest camera's.
+static int points_tiles(const TileIndex& ti, int* most = nullptr) {
+  int sum = 0, top = 1;
+  for (int i = 0; i < ti.n_cams; ++i) {
+    const int n = (ti.W[i] + kTileW - 1) / kTileW * ((ti.H[i] + PointsTile::H - 1) / PointsTile::H);
+    sum += n;
+    top = std::max(top, n);
+  }
+  if (most) *most = top;
+  return sum;
+}
+
+template <int Threads>
+static cudaError_t launch_points_n(const RigDev* rig, const RigHot& hot, const float2* rays, const FramePtrs& fp,
+                                   const Tables& t, const PointsDev& out, bool depth_f32, const TileIndex& ti,
+                                   cudaStream_t s) {
+  int most;
+  points_tiles(ti, &most);
+  const dim3 g((unsigned)most, ti.n_cams);
+  const size_t sm = PointsTile::smem(ti.k1);                  // at most 23 KB
+  if (depth_f32) k_points<float, Threads><<<g, Threads, sm, s>>>(rig, hot, rays, fp, t, ti, out);
+  else k_points<uint16_t, Threads><<<g, Threads, sm, s>>>(rig, hot, rays, fp, t, ti, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_points(const RigDev* rig, const RigHot& hot, const float2* rays, const FramePtrs& fp, const Tables& t,
-                          const PointsDev& out, bool depth_f32, const TileIndex& ti, cudaStream_t s) {
+                          const PointsDev& out, bool depth_f32, const TileIndex& ti, int sms, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(out.counts, 0, 2 * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  long long tiles = 1;
-  for (int i = 0; i < ti.n_cams; ++i)
-    tiles = std::max(tiles, (long long)((ti.W[i] + kTileW - 1) / kTileW) * ((ti.H[i] + PointsTile::H - 1) / PointsTile::H));
-  const dim3 g((unsigned)tiles, ti.n_cams);
-  const size_t sm = PointsTile::smem(ti.k1);                  // at most 23 KB
-  if (depth_f32) k_points<float><<<g, PointsTile::Threads, sm, s>>>(rig, hot, rays, fp, t, out);
-  else k_points<uint16_t><<<g, PointsTile::Threads, sm, s>>>(rig, hot, rays, fp, t, out);
-  return cudaGetLastError();
+  const int th = weigh_threads(points_tiles(ti), PointsTile::H, sms);
+  return th == 128   ? launch_points_n<128>(rig, hot, rays, fp, t, out, depth_f32, ti, s)
+         : th == 256 ? launch_points_n<256>(rig, hot, rays, fp, t, out, depth_f32, ti, s)
+                     : launch_points_n<512>(rig, hot, rays, fp, t, out, depth_f32, ti, s);
 }
 
 cudaError_t launch_screen(const ScreenArgs& a, bool depth_f32, long long max_px, cudaStream_t s) {

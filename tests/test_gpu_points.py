@@ -69,3 +69,25 @@ def test_points_match_the_oracle(F, oracle_mod, case):
     assert np.all(np.abs(wg[big] - wo[big]) <= 1e-5 * wo[big])
     assert np.all(np.abs(wg[~big] - wo[~big]) <= W_ABS)
     np.testing.assert_array_equal(col, np.concatenate([x.reshape(-1, 3) for x in fr.rgb]))
+
+
+@pytest.mark.parametrize("fmt", ["u16", "f32"])
+@pytest.mark.parametrize("n", [1, 3, 5])
+def test_points_at_each_number_of_threads(F, oracle_mod, n, fmt):
+    """176, 528 and 880 tiles with cut columns and rows: 512, 256 and 128 threads a block."""
+    rig = S.tiny_rig(n=n, width=333, height=251, depth_format=fmt, depth_scale=1.0 if fmt == "f32" else 0.001,
+                     spread_deg=25.0)
+    fr = S.random_frame(rig, seed=73, zero_frac=0.05)
+    nv, ng, pos, w, col = _points(F, rig, fr)
+    orc = oracle_mod.fuse_frame(rig, fr, {})
+    gated = orc["gated"].astype(bool)
+    assert nv == orc["stats"]["n_valid"] and ng == orc["stats"]["n_gated"] == gated.sum()
+    assert np.all(np.isnan(pos[~gated])) and np.all(w[~gated] == 0.0)
+    dp = np.abs(pos[gated].astype(np.float64) - orc["pw"][gated])
+    assert np.all(dp <= 1e-5 + 1e-6 * np.abs(orc["pw"][gated])), dp.max()
+    ok = gated & ~point_masks(orc)[2]
+    wo, wg = orc["omega"][ok], w[ok].astype(np.float64)
+    big = wo >= W_FLOOR
+    assert np.all(np.abs(wg[big] - wo[big]) <= 1e-5 * wo[big])
+    assert np.all(np.abs(wg[~big] - wo[~big]) <= W_ABS)
+    np.testing.assert_array_equal(col, np.concatenate([x.reshape(-1, 3) for x in fr.rgb]))
