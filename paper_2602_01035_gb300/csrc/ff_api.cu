@@ -60,7 +60,7 @@ struct fuseflow_batch {
   std::vector<fuseflow_ctx*> ctx;
 };
 
-// One fuse call captured as a CUDA graph (the memset and kernels of launch_frame).
+// One fuse call captured as a CUDA graph (the kernels of launch_frame).
 struct fuseflow_graph {
   fuseflow_ctx* ctx = nullptr;
   cudaGraph_t graph = nullptr;
@@ -308,7 +308,6 @@ void build_rig(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* extr,
   const double sig_g = params->sigma_m / unit * ginv;
   if (k1 > 0) split(1.0 / (sig_g * sig_g * k1), rig.hot.einv_h, rig.hot.einv_l);
   rig.depth_f32 = params->depth_format == FUSEFLOW_DEPTH_F32;
-  rig.top_k = params->top_k;
   int nr = 0;
   long long off = 0, np = 0;
   for (int i = 0; i < n_cams; ++i) {
@@ -1034,7 +1033,7 @@ int fuseflow_read_stage_times(fuseflow_ctx* ctx, double* ms, int64_t* n_frames) 
 }
 
 // Launch geometry from a (validated) tuning: the count step's grid follows its chunks per
-// block, and the scan step reads exactly the block statistics that grid writes.
+// block, and the emit step reads exactly the block statistics that grid writes.
 static void apply_tuning(fuseflow_ctx* ctx, const fuseflow_tuning& tu) {
   count_geometry(&ctx->geo, ctx->n_units, tu.count_chunks);
   ctx->tab.n_bstats = ctx->geo.count_blocks;
@@ -1221,7 +1220,7 @@ int64_t fuseflow_device_bytes(const fuseflow_ctx* ctx) {
 // that loads this library until the process exits.  Host code never dereferences the
 // array's name: the device address comes from cudaGetSymbolAddress, taken once per device
 // on that device's first call (which also clears the hash tables and synchronizes the
-// stream).  Later calls reuse the array; the frame's own clear and emit steps leave the
+// stream).  Later calls reuse the array; the frame's own steps leave the
 // tables empty again, so calls in a row need no set-up.  Calls whose GPU work overlaps
 // (several streams, or several host threads) race on the array.
 namespace {

@@ -72,7 +72,6 @@ struct RigDev {
   RigHot hot;
   int n_min;
   int depth_f32;
-  int top_k;                     // Sec. II.5(2)a variant: fuse the top_k members only (0: all)
   long long n_px;
   CamDev cam[kMaxCams];
   PairDev pair[kMaxCams * kMaxK1];
@@ -231,15 +230,6 @@ __host__ __device__ inline float from_ordered(unsigned u) {
   memcpy(&f, &v, 4);
   return f;
 #endif
-}
-
-__device__ __forceinline__ unsigned long long mix64(unsigned long long k) {
-  k ^= k >> 31;
-  k *= 0x7fb5d329728ea185ull;
-  k ^= k >> 27;
-  k *= 0x81dadef4bc2dd44dull;
-  k ^= k >> 33;
-  return k;
 }
 
 // First table position of coarse cell (x, y, z).  The two last lines scatter the cells of a wall: without

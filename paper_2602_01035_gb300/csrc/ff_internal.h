@@ -91,7 +91,7 @@ struct FrameArgs {
   RigHot hot;
   int count_chunks;
   float unit_m;
-  int top_k;
+  int top_k;                     // Sec. II.5(2)a variant: the top_k members of a cell are fused (0: all)
 };
 
 // Frames of one launch of the frame kernels, passed as one __grid_constant__ kernel

@@ -150,9 +150,6 @@ __device__ __forceinline__ unsigned coarse_lvbase(const Tables& t, unsigned long
   return kBaseNone;
 }
 
-// Sec. II.5(1)d for every coarse cell once all counts are in: its level l and a range of
-// 8^l dense cell slots.  Ranges are claimed with one atomic per warp (an inclusive scan of
-// the sizes inside the warp), so their placement depends on scheduling; no result does.
 // Programmatic dependent launch between the kernels of one frame: each kernel lets the next
 // one start launching as soon as all of its own blocks are running (pdl_release), and a
 // kernel waits for the previous one to complete, its memory visible, before it touches
@@ -176,6 +173,9 @@ __device__ __forceinline__ int batch_frame(const int (&first)[NB + 1], int n, in
 template <int NB>
 __device__ __forceinline__ int batch_frame_y() { return NB == 1 ? 0 : (int)blockIdx.y; }
 
+// Sec. II.5(1)d for every coarse cell once all counts are in: its level l and a range of
+// 8^l dense cell slots.  Ranges are claimed with one atomic per warp (an inclusive scan of
+// the sizes inside the warp), so their placement depends on scheduling; no result does.
 template <int NB>
 __global__ void __launch_bounds__(kThreads) k_levels(const __grid_constant__ BatchArgs<NB> args) {
   const Tables& t = args.f[batch_frame_y<NB>()].t;
@@ -1583,7 +1583,7 @@ __global__ void __launch_bounds__(kTopThreads, 8) k_reduce_topk(const __grid_con
   const unsigned n_cells = min(t.cnt->n_cells, t.max_slots);
   const unsigned n_coarse = min(t.cnt->n_coarse, t.cmask + 1u);
   const unsigned n_part = min(t.cnt->n_partials, t.max_partials);
-  const int K = rig.top_k;
+  const int K = fa.top_k;
   const unsigned per = (unsigned)(kTopThreads / K);
   for (unsigned i = blockIdx.x * kTopThreads + threadIdx.x; i < n_coarse; i += gridDim.x * kTopThreads) {
     const unsigned cs = t.cused[i];
