@@ -460,6 +460,11 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   ctx->n_units = ctx->geo.tiles.unit[n_cams];
   count_geometry(&ctx->geo, ctx->n_units, default_chunks(ctx->n_units, sms));
   ctx->geo.emit_blocks = std::max(1, sms * 8);
+  // Programmatic launches for frames one after another on a stream, us a frame at levels 0 / 1 / 2:
+  // 2x160x120 35.2 / 28.7 / 27.7, 4x640x480 61.4 / 55.5 / 53.6, 4x1280x720 142.3 / 138.7 / 136.7; above
+  // 2^21 pixels levels 1 and 2 are within 1 % for all members (8x1280x720 258.9 / 259.0 / 257.7,
+  // 16x1024x1024 828 / 822 / 822), but with top_k = 3 level 2 costs 15 to 24 % (231 / 234 / 269 and
+  // 950 / 945 / 1170; below, 4x1280x720 109 / 107 / 112)
   ctx->geo.pdl = off < (1ll << 21) ? 2 : 1;
 
   // ---------------------------------------------------------------- device memory

@@ -557,7 +557,7 @@ constexpr unsigned kUnnumbered = 0x80000000u;   // on a unit's count while point
 // warp.  Each cell goes to the global table once per unit, with its number of points, and its position
 // in the warp's table is its number in the unit; the gated pixels are listed (pixel and cell number,
 // depth, confidence) for the next steps, which then neither gate again nor probe the global table.
-// 8x1280x720 (7.4 Mpx, 28,800 units): 48 us, bound by instruction issue (74 % of the slots while full);
+// 8x1280x720 (7.4 Mpx, 28,800 units): 49 us, bound by instruction issue (69 % of the slots used);
 // blocks with a table of 2048 cells and runs of equal cells merged across the warp took 59 us.  Finding a
 // unit's cells one after another as the smallest key left took 49 us there, but 236 instead of 154 us
 // where units hold many cells (16x1024^2).
@@ -1020,7 +1020,7 @@ __device__ __forceinline__ unsigned point_slot(unsigned lb, const float r[3], in
 // point that finds none.  All are order-independent but the numbering, which no result depends on.
 // A point looks at its slot first and sends an atomic only where that would change it: most do not.
 // Bound by latency and issue (gathers of the views' depths): 48 registers for uint16 depth, as 40 warps
-// an SM hide more than 32 do (weigh + sum of 8x1280x720: 185 us against 193 at 64); float32 depth, with
+// an SM hide more than 32 do (weigh + sum of 8x1280x720 when they were split: 185 us against 193 at 64); float32 depth, with
 // its checks, is faster at 64 (50 against 53 us on five ragged cameras).
 template <typename DT, bool TRACE, int NB, int TH>
 __global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64) k_weigh(const __grid_constant__ BatchArgs<NB> args) {
@@ -1185,10 +1185,13 @@ constexpr int kTileShares = 16;              // emit blocks that a tile counts r
 // with 64-bit reductions.  A warp lays the terms of its 32 points out in shared memory; eight lanes
 // then take a row each of eight successive points, a lane a term, and send one reduction of 64
 // contiguous bytes per run of points of one cell (eight lanes on a row measured 3 times faster than
-// a lane a row: the reductions of a row travel together).  Bound by L2's reductions: 64 us for 3.7 M
-// points, where 64-byte rows alone take 50 (75 G rows/s); with the representatives' marks 72.  Weigh and sum take 185 us on 8x1280x720;
-// one kernel that gathered each tile's cells in shared-memory tables and wrote a record per tile and
-// cell for a later walk of the cells' record lists took 211 (tables, records and their barriers: 120).
+// a lane a row: the reductions of a row travel together).  8x1280x720: 74 us for 3.73 M points, which
+// send 2.87 M rows (2.15 M more than there are cells in the tiles, as only successive points of a
+// cell are merged); a probe that did nothing but add rows of 64 bytes sent 75 G a second, 38 us for these,
+// so that about half of the time is L2's reductions and the rest the points' own instructions and loads.
+// Weigh and sum took 185 us together before the marks of representatives were added here (10 us), where
+// one kernel that gathered each tile's cells in shared-memory tables and wrote a record per tile and cell
+// for a later walk of the cells' record lists took 211 (tables, records and their barriers: 120).
 template <typename DT, int NB, int TH>
 __global__ void k_sum(const __grid_constant__ BatchArgs<NB> args) {
   using WT = WeighTile<TH>;

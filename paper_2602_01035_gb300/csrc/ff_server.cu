@@ -168,8 +168,8 @@ int record(const Rig& g, Slot& s) {
 }
 
 // Launch geometry of the rig's slots: the autotuned one if any, and with several slots
-// plain stream order (overlapping slots fill the kernel boundaries, and blocks waiting for
-// an earlier kernel would only hold back the other slots' work).
+// plain stream order: recorded calls are fastest in it (8x1280x720: 250 us a replay, 256 at levels
+// 1 and 2; 4x640x480: 52.2, 52.9 and 53.1), and overlapping slots fill the kernel boundaries.
 void apply_tuning(const Rig& g, Slot& s) {
   fuseflow_tuning tu{};
   if (g.tuned) tu = g.tuning;
