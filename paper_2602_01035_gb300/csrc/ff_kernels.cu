@@ -2054,7 +2054,7 @@ __global__ void __launch_bounds__(kThreads) k_mc(const RigDev* __restrict__ rigp
 // gradient G: central difference where both neighbours are valid, one-sided with one, 0
 // with none; sigma_local: population variance of the window's valid depths (m^2); C is
 // normalised by alpha + gamma and is 0 where the depth is invalid.
-// 7.4 Mpx of uint16: 28 us, bound by instruction issue (about 80 instructions a pixel; 150, and 37 us,
+// 7.4 Mpx of uint16: 28.7 us, bound by instruction issue (about 110 instructions a pixel; 150, and 37 us,
 // with each window's count and sum taken over its nine samples and each sample converted and tested apart).
 constexpr int kConfW = 128, kConfH = 32;
 

@@ -1,8 +1,9 @@
 """Edges of the steps that work on units of 32 x 8 pixels, against the oracle at the parity
 tolerances: units with more coarse cells than they have numbers, cells outside a unit's key
 window, grids of no more than 1024 cells an axis (where points leave the grid), float32 depths
-beyond the range of the grid evaluation of the consistency step, and image sizes one pixel to
-each side of the units' and tiles' edges."""
+beyond the range of the grid evaluation of the consistency step, one cell raised by every point,
+image sizes one pixel to each side of the units' and tiles' edges, and the static entry's tables
+after frames of the other variant."""
 import numpy as np
 import pytest
 
