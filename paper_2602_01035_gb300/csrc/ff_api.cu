@@ -589,7 +589,9 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
                    cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(static_cast<char*>(ctx->d_blocks) + pray_at, pray.data(), sizeof(float4) * pray.size(),
                    cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(ctx->d_tables, 0, ctx->table_bytes) != cudaSuccess ||
+        // only what a frame reads before any frame has written it: counters, bitmap and cell numbers
+        cudaMemset(b + o_cnt, 0, o_bst - o_cnt) != cudaSuccess ||
+        cudaMemset(b + o_lcell, 0, sizeof(unsigned) * kUnitCells * (size_t)ctx->n_units) != cudaSuccess ||
         cudaMemset(ctx->d_out, 0, ctx->out_bytes) != cudaSuccess ||
         launch_init_tables(t, ctx->max_slots, ctx->ccap, 0) != cudaSuccess ||
         prepare_launch(rig->depth_f32 != 0) != cudaSuccess ||

@@ -2194,6 +2194,7 @@ __global__ void k_init_tables(Tables t, unsigned fcap, unsigned ccap) {
     if (i < ccap) {
       t.coarse[i].key = kKeyEmpty;
       t.coarse[i].count = 0u;
+      t.coarse[i].lvbase = 0u;
     }
   }
 }
