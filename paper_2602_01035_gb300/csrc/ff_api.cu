@@ -481,7 +481,7 @@ int fuseflow_create(const fuseflow_intrinsics* intr, const fuseflow_extrinsics* 
   const unsigned max_partials = topk ? (unsigned)std::min<long long>(off, 0xfffffffell) : 0u;
   const size_t n_weighed = topk ? 0 : (size_t)off, n_summed = topk ? 0 : (size_t)ctx->max_cells;
   const size_t o_frec = take(sizeof(SlotRec) * ctx->max_slots, 256);
-  const size_t o_fused = take(topk ? sizeof(unsigned) * (size_t)ctx->max_slots : 0, 256);
+  const size_t o_fused = take(sizeof(unsigned) * (size_t)ctx->max_slots, 256);
   const size_t o_coarse = take(sizeof(CoarseEntry) * ctx->ccap, 256);
   const size_t o_cused = take(sizeof(unsigned) * ctx->ccap, 256);
   const size_t o_cnt = take(sizeof(FrameCounters) + sizeof(unsigned) * (size_t)n_words, 256);

@@ -203,7 +203,7 @@ struct __align__(16) CellOut {
 };
 static_assert(sizeof(CellOut) == 48, "staged cell layout");
 
-struct FrameCounters {           // zero between frames
+struct FrameCounters {           // zero between frames, but n_cells, which the level step clears
   unsigned n_cells, n_coarse;
   unsigned error;
   unsigned n_partials;

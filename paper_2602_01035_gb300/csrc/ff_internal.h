@@ -18,7 +18,7 @@ struct FramePtrs {               // one frame's caller-owned device images, per 
 struct Tables {                  // context-owned device scratch
   // cells: dense slots, coarse cell c owns [cbase(c), cbase(c) + 8^level(c))
   SlotRec* frec;                 // key, list head and smallest exponent per slot
-  unsigned* fused;               // top-k variant: slots by cell number
+  unsigned* fused;               // slots by cell number: those past the output's capacity (top-k: all)
   unsigned max_slots;
   // coarse hash table (open addressing), ccap entries
   CoarseEntry* coarse;

@@ -185,6 +185,7 @@ __global__ void __launch_bounds__(kThreads) k_levels(const __grid_constant__ Bat
   const int lane = threadIdx.x & 31;
   const unsigned long long cap = t.max_slots;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < t.n_wblocks; i += gridDim.x * blockDim.x) t.bsum[i] = 0u;
+  if (blockIdx.x == 0 && threadIdx.x == 0) t.cnt->n_cells = 0u;      // the last frame's
   for (unsigned base = blockIdx.x * blockDim.x; base < n_coarse; base += gridDim.x * blockDim.x) {
     const unsigned i = base + threadIdx.x;
     unsigned cs = 0, l = 0;
@@ -865,7 +866,7 @@ __device__ __forceinline__ void mark_cell(const Tables& t, unsigned g, unsigned 
 }
 
 // The frame's statistics from the count step's blocks and the counters, by one block, which clears the
-// counters for the next frame (no other block of its kernel reads them).
+// counters for the next frame (but the number of cells, which other blocks of its kernel read).
 template <bool TOPK>
 __device__ __forceinline__ void frame_stats(const Tables& t, const OutDev& out) {
   __shared__ unsigned long long s_l[3][kThreads / 32];
@@ -917,7 +918,10 @@ __device__ __forceinline__ void frame_stats(const Tables& t, const OutDev& out) 
   st.error = (int32_t)err;
   st.n_coarse = (int32_t)__ldcg(&t.cnt->n_coarse);
   *out.stats = st;
-  *t.cnt = FrameCounters{};
+  t.cnt->n_coarse = 0u;                         // n_cells: by the level step
+  t.cnt->error = 0u;
+  t.cnt->n_partials = 0u;
+  t.cnt->n_slots = 0ull;
 }
 
 // u64 -> float32 through two 32-bit conversions (at most two roundings)
@@ -1155,11 +1159,13 @@ __global__ void __maxnreg__(sizeof(DT) == 2 ? 48 : 64) k_weigh(const __grid_cons
   for (unsigned q = threadIdx.x; q < n; q += blockDim.x) {
     const unsigned id = s_first + q, slot = s_slot[q];
     t.frec[slot].head = id;
-    if ((long long)id < fa.out.max_cells) {   // else past the capacity
+    if ((long long)id < fa.out.max_cells) {
       uint4* a = reinterpret_cast<uint4*>(t.rows + id);
 #pragma unroll
       for (int k = 0; k < 4; ++k) a[k] = make_uint4(0u, 0u, 0u, 0u);
       a[4] = make_uint4((unsigned)s_key[q], (unsigned)(s_key[q] >> 32), slot, 0u);
+    } else {
+      t.fused[id] = slot;                   // past the capacity; a number for each slot at most
     }
   }
 }
@@ -1273,10 +1279,6 @@ __global__ void k_sum(const __grid_constant__ BatchArgs<NB> args) {
             if (q < kTileShares) atomicAdd(&s_share[q], 1u);
             else atomicAdd(&t.bsum[share0 + q], 1u);
           }
-        } else if (rec.x == ~(off + (unsigned)(y * W + x))) {
-          // past the output's capacity (reported): no row and no mark, so its slot is cleared here; the
-          // cell's other points find no number in it, or one past the capacity
-          *reinterpret_cast<uint4*>(t.frec + slot) = kSlotClear;
         }
         uint4* row = s_row + (lane + (lane >> 3)) * 4;
 #pragma unroll
@@ -1876,6 +1878,12 @@ __global__ void __launch_bounds__(kThreads) k_emit(const __grid_constant__ Batch
   if (b >= t.n_wblocks) {
     if (b == t.n_wblocks) frame_stats<TOPK>(t, out);
     return;
+  }
+  if (!TOPK) {                                  // slots of cells past the output's capacity (reported)
+    const unsigned n_cells = min(__ldcg(&t.cnt->n_cells), t.max_slots);
+    for (unsigned i = (unsigned)out.max_cells + (unsigned)b * kThreads + threadIdx.x; i < n_cells;
+         i += (unsigned)t.n_wblocks * kThreads)
+      *reinterpret_cast<uint4*>(t.frec + t.fused[i]) = kSlotClear;
   }
   unsigned before = 0u;
   for (int i = threadIdx.x; i < b; i += kThreads) before += __ldcg(t.bsum + i);
