@@ -1879,12 +1879,7 @@ __global__ void __launch_bounds__(kThreads) k_emit(const __grid_constant__ Batch
     if (b == t.n_wblocks) frame_stats<TOPK>(t, out);
     return;
   }
-  if (!TOPK) {                                  // slots of cells past the output's capacity (reported)
-    const unsigned n_cells = min(__ldcg(&t.cnt->n_cells), t.max_slots);
-    for (unsigned i = (unsigned)out.max_cells + (unsigned)b * kThreads + threadIdx.x; i < n_cells;
-         i += (unsigned)t.n_wblocks * kThreads)
-      *reinterpret_cast<uint4*>(t.frec + t.fused[i]) = kSlotClear;
-  }
+  const unsigned n_cells = TOPK ? 0u : __ldcg(&t.cnt->n_cells);      // for the end: all in flight together
   unsigned before = 0u;
   for (int i = threadIdx.x; i < b; i += kThreads) before += __ldcg(t.bsum + i);
   const long long w = (long long)b * kRankWords + threadIdx.x;
@@ -1959,6 +1954,10 @@ __global__ void __launch_bounds__(kThreads) k_emit(const __grid_constant__ Batch
     out.rep[rank] = g;
     out.key[rank] = c.key;
   }
+  // slots of cells past the output's capacity (reported)
+  for (unsigned i = (unsigned)out.max_cells + (unsigned)b * kThreads + threadIdx.x; i < min(n_cells, t.max_slots);
+       i += (unsigned)t.n_wblocks * kThreads)
+    *reinterpret_cast<uint4*>(t.frec + t.fused[i]) = kSlotClear;
 }
 
 // Served frames: the cloud's first n cells (n = min(n_cells, capacity)) and the
